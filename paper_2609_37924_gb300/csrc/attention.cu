@@ -71,6 +71,59 @@ struct AttnTcArgs {
   int* status;
 };
 
+// One arrival per warp: the lanes' reads (TMEM) and writes (shared memory,
+// each fenced for the async proxy by its own lane) precede the elected
+// lane's arrive.  128 arrivals per tile and barrier serialise on the barrier
+// word; one per warp does not.
+__device__ __forceinline__ void warp_arrive(uint64_t* bar) {
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
+}
+
+// Max of 64 scores of one row (two chunks of 32); MASKED: only the columns lo <= c < lim count.
+template <bool MASKED>
+__device__ __forceinline__ void max64(const uint32_t (&ra)[32], const uint32_t (&rb)[32], int lo, int lim,
+                                      float (&mx)[4]) {
+#pragma unroll
+  for (int k = 0; k < 32; ++k) {
+    float a = __uint_as_float(ra[k]), b = __uint_as_float(rb[k]);
+    if (MASKED) {
+      a = k < lim && k >= lo ? a : -INFINITY;
+      b = 32 + k < lim && 32 + k >= lo ? b : -INFINITY;
+    }
+    mx[k & 3] = fmax3(mx[k & 3], a, b);
+  }
+}
+
+// P = 2^(s * scale - m) of 32 columns of one row: bf16 pairs into the four
+// 16-byte chunks chunk0 .. chunk0+3 of the row's 128-byte swizzled line, the
+// fp32 values added to the packed sums.  The masked and the plain form are
+// separate instantiations: with the column tests predicated into one body the
+// hd-64 kernel issued about 400 instructions per warp and tile.
+template <bool MASKED>
+__device__ __forceinline__ void exp32(const uint32_t (&r)[32], uint64_t sc2, uint64_t negm2, int lo, int lim,
+                                      uint64_t (&ps2)[2], uint8_t* line, int chunk0, int row) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    uint32_t pk[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int k = 8 * q + 2 * j;
+      float x0, x1;
+      f2_unpack(f2_fma(f2_pack(__uint_as_float(r[k]), __uint_as_float(r[k + 1])), sc2, negm2), x0, x1);
+      float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
+      if (MASKED) {
+        p0 = k < lim && k >= lo ? p0 : 0.0f;
+        p1 = k + 1 < lim && k + 1 >= lo ? p1 : 0.0f;
+      }
+      ps2[j & 1] = f2_add(ps2[j & 1], f2_pack(p0, p1));
+      __nv_bfloat162 t = __floats2bfloat162_rn(p0, p1);
+      pk[j] = *reinterpret_cast<uint32_t*>(&t);
+    }
+    *reinterpret_cast<uint4*>(line + (((chunk0 + q) ^ (row & 7)) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+  }
+}
+
 // WIN: the sliding window of local layers is in force (a separate
 // instantiation, so that the kernel without it carries no window code).
 template <int HD, int TKV, bool WIN>
@@ -118,15 +171,18 @@ __global__ void __launch_bounds__(192, AttnTcCfg<HD, TKV>::MIN_BLOCKS)
   const int t0 = max(split * args.tiles_per_split, kv_begin / TKV);   // first tile of this CTA
   const int n_tiles = max(0, min((kv_end + TKV - 1) / TKV, (split + 1) * args.tiles_per_split) - t0);
 
+  // softmax warps that own at least one virtual row; the others leave their
+  // rows of Q, P and O undefined (nothing reads those rows of D) and only wait
+  const int act_warps = (min(TQ, n_virt - m0) + 31) / 32;
   if (threadIdx.x == 0) {
-    mbar_init(q_full, 128);            // the softmax threads stage Q
+    mbar_init(q_full, act_warps);      // the softmax warps stage Q
     for (int s = 0; s < 2; ++s) {
       mbar_init(&kv_full[s], 1);
       mbar_init(&kv_empty[s], 1);
     }
     mbar_init(s_full, 1);
-    mbar_init(s_free, 128);
-    mbar_init(p_full, 128);
+    mbar_init(s_free, act_warps);
+    mbar_init(p_full, act_warps);
     mbar_init(o_full, 1);
     mbar_init(drain, 1);
     *abort_flag = 0;
@@ -170,39 +226,39 @@ __global__ void __launch_bounds__(192, AttnTcCfg<HD, TKV>::MIN_BLOCKS)
       if (issued1 > 0) mbar_wait_bounded(&kv_full[1], (issued1 - 1) & 1, &never, args.status);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ------------------------------------------------------------- MMA issuer
+    {   // ------------------------------------------------------------- MMA issuer (the whole warp, one elected lane)
       constexpr uint32_t idesc_s = idesc_bf16_f32(TQ, TKV);
       constexpr uint32_t idesc_o = idesc_bf16_f32(TQ, HD);
-      bool ok = n_tiles > 0 && mbar_wait_bounded(q_full, 0, abort_flag, args.status);
-      const uint32_t q0 = smem_u32(sQ), p0 = smem_u32(sP);
+      bool ok = n_tiles > 0 && warp_wait_bounded(q_full, 0, abort_flag, args.status);
+      const uint64_t q0 = sdesc_kmajor_sw128(smem_u32(sQ)), p0 = sdesc_kmajor_sw128(smem_u32(sP));
       for (int i = 0; ok && i < n_tiles; ++i) {
         const int st = i & 1;
-        if (!mbar_wait_bounded(&kv_full[st], (i >> 1) & 1, abort_flag, args.status)) break;
-        if (i > 0 && !mbar_wait_bounded(s_free, (i - 1) & 1, abort_flag, args.status)) break;
+        if (!warp_wait_bounded(&kv_full[st], (i >> 1) & 1, abort_flag, args.status)) break;
+        if (i > 0 && !warp_wait_bounded(s_free, (i - 1) & 1, abort_flag, args.status)) break;
         tc_fence_after();
-        const uint32_t k0 = smem_u32(sK + st * C::K_BYTES), v0 = smem_u32(sV + st * C::V_BYTES);
+        const uint64_t k0 = sdesc_kmajor_sw128(smem_u32(sK + st * C::K_BYTES));
+        const uint64_t v0 = sdesc_kmajor_sw128(smem_u32(sV + st * C::V_BYTES));
 #pragma unroll
         for (int kk = 0; kk < HD / 16; ++kk)
-          umma_bf16(t_s, sdesc_kmajor_sw128(q0 + (kk >> 2) * 16384 + (kk & 3) * 32),
-                    sdesc_kmajor_sw128(k0 + (kk >> 2) * (TKV * 128) + (kk & 3) * 32), idesc_s, kk != 0);
+          umma_bf16(t_s, q0 + (((kk >> 2) * 16384 + (kk & 3) * 32) >> 4),
+                    k0 + (((kk >> 2) * (TKV * 128) + (kk & 3) * 32) >> 4), idesc_s, kk != 0);
         umma_commit(s_full);
         // P of tile i is in shared memory and any rescale of O by the softmax
         // threads is complete: O += P V
-        if (!mbar_wait_bounded(p_full, i & 1, abort_flag, args.status)) break;
+        if (!warp_wait_bounded(p_full, i & 1, abort_flag, args.status)) break;
         tc_fence_after();
 #pragma unroll
         for (int kk = 0; kk < TKV / 16; ++kk)
-          umma_bf16(t_o, sdesc_kmajor_sw128(p0 + (kk >> 2) * 16384 + (kk & 3) * 32),
-                    sdesc_kmajor_sw128(v0 + (kk >> 2) * (HD * 128) + (kk & 3) * 32), idesc_o, (i != 0) || (kk != 0));
+          umma_bf16(t_o, p0 + (((kk >> 2) * 16384 + (kk & 3) * 32) >> 4),
+                    v0 + (((kk >> 2) * (HD * 128) + (kk & 3) * 32) >> 4), idesc_o, (i != 0) || (kk != 0));
         umma_commit(o_full);
         umma_commit(&kv_empty[st]);
       }
       umma_commit(drain);
       volatile int never = 0;
-      mbar_wait_bounded(drain, 0, &never, args.status);
+      warp_wait_bounded(drain, 0, &never, args.status);
     }
-  } else {
+  } else if ((warp & 3) < act_warps) {
     // --------------------------------------------------------------- softmax
     // One virtual query row per thread (row = TMEM lane).  O is accumulated
     // in TMEM by the P V MMAs of all key tiles.  The exponentials of every
@@ -234,7 +290,7 @@ __global__ void __launch_bounds__(192, AttnTcCfg<HD, TKV>::MIN_BLOCKS)
         }
       }
       fence_proxy_async_smem();
-      mbar_arrive(q_full);
+      warp_arrive(q_full);
     }
     float m_ref = -INFINITY, l_run = 0.0f;
     bool ok = true;
@@ -249,25 +305,18 @@ __global__ void __launch_bounds__(192, AttnTcCfg<HD, TKV>::MIN_BLOCKS)
       const int lim = kv_hi - key0;                                   // visible keys of this tile: [lo, lim)
       const int lo = WIN ? qpos - args.window + 1 - key0 : 0;
       const bool masked = __any_sync(0xffffffffu, lim < TKV || (WIN && lo > 0));   // warp-uniform path choice
-      // pass 1: row max over the tile, 64 columns per TMEM round trip
+      // pass 1: row max over the tile, 64 columns per TMEM round trip (64-key
+      // tiles keep them in registers for pass 2)
       float mxa[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};   // independent chains
+      uint32_t ra[32], rb[32];
 #pragma unroll
       for (int c = 0; c < TKV / 64; ++c) {
-        uint32_t ra[32], rb[32];
         tmem_ld32_nowait(t_s + lane_off + 64 * c, ra);
         tmem_ld32_nowait(t_s + lane_off + 64 * c + 32, rb);
         tmem_wait_ld(ra);
         tmem_bind(rb);
-        if (masked) {
-#pragma unroll
-          for (int k = 0; k < 32; ++k)
-            mxa[k & 3] = fmax3(mxa[k & 3],
-                               64 * c + k < lim && 64 * c + k >= lo ? __uint_as_float(ra[k]) : -INFINITY,
-                               64 * c + 32 + k < lim && 64 * c + 32 + k >= lo ? __uint_as_float(rb[k]) : -INFINITY);
-        } else {
-#pragma unroll
-          for (int k = 0; k < 32; ++k) mxa[k & 3] = fmax3(mxa[k & 3], __uint_as_float(ra[k]), __uint_as_float(rb[k]));
-        }
+        if (masked) max64<true>(ra, rb, lo - 64 * c, lim - 64 * c, mxa);
+        else max64<false>(ra, rb, 0, 64, mxa);
       }
       const float m_tile = fmax3(fmaxf(mxa[0], mxa[1]), mxa[2], mxa[3]) * args.scale_log2;
       float m_new = m_ref, factor = 1.0f;
@@ -283,45 +332,34 @@ __global__ void __launch_bounds__(192, AttnTcCfg<HD, TKV>::MIN_BLOCKS)
         tc_fence_after();
 #pragma unroll
         for (int c = 0; c < HD / 32; ++c) {
-          uint32_t ra[32];
-          tmem_ld32_nowait(t_o + lane_off + 32 * c, ra);
-          tmem_wait_ld(ra);
+          uint32_t ro[32];
+          tmem_ld32_nowait(t_o + lane_off + 32 * c, ro);
+          tmem_wait_ld(ro);
 #pragma unroll
-          for (int k = 0; k < 32; ++k) ra[k] = __float_as_uint(__uint_as_float(ra[k]) * factor);
-          tmem_st32(t_o + lane_off + 32 * c, ra);
+          for (int k = 0; k < 32; ++k) ro[k] = __float_as_uint(__uint_as_float(ro[k]) * factor);
+          tmem_st32(t_o + lane_off + 32 * c, ro);
         }
         tmem_wait_st();
         l_run *= factor;
       }
-      // pass 2: P = 2^(s * scale - m_new) as bf16 into the swizzled A-operand layout, 32 columns per trip
+      // pass 2: P = 2^(s * scale - m_new) as bf16 into the swizzled A-operand layout (keys 64 c .. 64 c + 63: atom c)
       const uint64_t negm2 = f2_pack(-m_new, -m_new);
       uint64_t ps2[2] = {0, 0};                  // packed partial sums, two chains
 #pragma unroll
-      for (int c = 0; c < TKV / 32; ++c) {
-        uint32_t ra[32];
-        tmem_ld32_nowait(t_s + lane_off + 32 * c, ra);
-        tmem_wait_ld(ra);
-        uint32_t pk[16];
-#pragma unroll
-        for (int k = 0; k < 32; k += 2) {
-          float x0, x1;
-          f2_unpack(f2_fma(f2_pack(__uint_as_float(ra[k]), __uint_as_float(ra[k + 1])), sc2, negm2), x0, x1);
-          float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
-          if (masked) {
-            p0 = 32 * c + k < lim && 32 * c + k >= lo ? p0 : 0.0f;
-            p1 = 32 * c + k + 1 < lim && 32 * c + k + 1 >= lo ? p1 : 0.0f;
-          }
-          ps2[(k >> 1) & 1] = f2_add(ps2[(k >> 1) & 1], f2_pack(p0, p1));
-          __nv_bfloat162 t = __floats2bfloat162_rn(p0, p1);
-          pk[k / 2] = *reinterpret_cast<uint32_t*>(&t);
+      for (int c = 0; c < TKV / 64; ++c) {
+        if (TKV > 64) {
+          tmem_ld32_nowait(t_s + lane_off + 64 * c, ra);
+          tmem_ld32_nowait(t_s + lane_off + 64 * c + 32, rb);
+          tmem_wait_ld(ra);
+          tmem_bind(rb);
         }
-        // keys 32c .. 32c+31: atom (32c / 64), 16-byte chunks (32c % 64) / 8 .. +3
-        uint8_t* atom = prow0 + (c >> 1) * 16384;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int chunk = (c & 1) * 4 + q;
-          *reinterpret_cast<uint4*>(atom + ((chunk ^ (row & 7)) << 4)) =
-              make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
+        uint8_t* line = prow0 + c * 16384;
+        if (masked) {
+          exp32<true>(ra, sc2, negm2, lo - 64 * c, lim - 64 * c, ps2, line, 0, row);
+          exp32<true>(rb, sc2, negm2, lo - 64 * c - 32, lim - 64 * c - 32, ps2, line, 4, row);
+        } else {
+          exp32<false>(ra, sc2, negm2, 0, 64, ps2, line, 0, row);
+          exp32<false>(rb, sc2, negm2, 0, 64, ps2, line, 4, row);
         }
       }
       float a0, a1, b0, b1;
@@ -331,8 +369,8 @@ __global__ void __launch_bounds__(192, AttnTcCfg<HD, TKV>::MIN_BLOCKS)
       m_ref = m_new;
       tc_fence_before();
       fence_proxy_async_smem();
-      mbar_arrive(s_free);
-      mbar_arrive(p_full);
+      warp_arrive(s_free);
+      warp_arrive(p_full);
     }
     const size_t bk = static_cast<size_t>(b) * args.n_kv_heads + hk;
     if (args.splits > 1 && ok && n_tiles == 0) {
@@ -459,16 +497,17 @@ __global__ void __launch_bounds__(192, AttnDbCfg<HD_>::MIN_BLOCKS)
   const int kv_end = args.causal ? min(args.kv_len, args.ctx + r_max + 1) : args.kv_len;
   const int n_tiles = (kv_end + TKV - 1) / TKV;
 
+  const int act_warps = (min(TQ, n_virt - m0) + 31) / 32;   // softmax warps that own a virtual row
   if (threadIdx.x == 0) {
-    mbar_init(q_full, 128);
+    mbar_init(q_full, act_warps);
     for (int s = 0; s < NST; ++s) {
       mbar_init(&kv_full[s], 1);
       mbar_init(&kv_empty[s], 1);
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(&s_full[s], 1);
-      mbar_init(&s_free[s], 128);
-      mbar_init(&p_full[s], 128);
+      mbar_init(&s_free[s], act_warps);
+      mbar_init(&p_full[s], act_warps);
     }
     mbar_init(o_full, 1);
     mbar_init(drain, 1);
@@ -513,35 +552,35 @@ __global__ void __launch_bounds__(192, AttnDbCfg<HD_>::MIN_BLOCKS)
         if (issued[s] > 0) mbar_wait_bounded(&kv_full[s], (issued[s] - 1) & 1, &never, args.status);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ------------------------------------------------------------- MMA issuer
+    {   // ------------------------------------------------------------- MMA issuer (the whole warp, one elected lane)
       constexpr uint32_t idesc_s = idesc_bf16_f32(TQ, TKV);
       constexpr uint32_t idesc_o = idesc_bf16_f32(TQ, HD);
-      bool ok = n_tiles > 0 && mbar_wait_bounded(q_full, 0, abort_flag, args.status);
-      const uint32_t q0 = smem_u32(sQ);
+      bool ok = n_tiles > 0 && warp_wait_bounded(q_full, 0, abort_flag, args.status);
+      const uint64_t q0 = sdesc_kmajor_sw128(smem_u32(sQ));
       for (int i = 0; ok && i <= n_tiles; ++i) {
         if (i < n_tiles) {
           // S(i) = Q K(i)^T into S buffer i & 1, once the softmax has released it (tile i - 2)
           const int st = i % NST, sb = i & 1;
-          if (!mbar_wait_bounded(&kv_full[st], (i / NST) & 1, abort_flag, args.status)) break;
-          if (i >= 2 && !mbar_wait_bounded(&s_free[sb], ((i - 2) >> 1) & 1, abort_flag, args.status)) break;
+          if (!warp_wait_bounded(&kv_full[st], (i / NST) & 1, abort_flag, args.status)) break;
+          if (i >= 2 && !warp_wait_bounded(&s_free[sb], ((i - 2) >> 1) & 1, abort_flag, args.status)) break;
           tc_fence_after();
-          const uint32_t k0 = smem_u32(sK + st * C::K_BYTES);
+          const uint64_t k0 = sdesc_kmajor_sw128(smem_u32(sK + st * C::K_BYTES));
 #pragma unroll
           for (int kk = 0; kk < HD / 16; ++kk)
-            umma_bf16(tmem + sb * TKV, sdesc_kmajor_sw128(q0 + (kk >> 2) * 16384 + (kk & 3) * 32),
-                      sdesc_kmajor_sw128(k0 + (kk >> 2) * (TKV * 128) + (kk & 3) * 32), idesc_s, kk != 0);
+            umma_bf16(tmem + sb * TKV, q0 + (((kk >> 2) * 16384 + (kk & 3) * 32) >> 4),
+                      k0 + (((kk >> 2) * (TKV * 128) + (kk & 3) * 32) >> 4), idesc_s, kk != 0);
           umma_commit(&s_full[sb]);
         }
         if (i >= 1) {
           // O += P(j) V(j) for the previous tile, once its probabilities are in shared memory
           const int j = i - 1, pb = j & 1, st = j % NST;
-          if (!mbar_wait_bounded(&p_full[pb], (j >> 1) & 1, abort_flag, args.status)) break;
+          if (!warp_wait_bounded(&p_full[pb], (j >> 1) & 1, abort_flag, args.status)) break;
           tc_fence_after();
-          const uint32_t p0 = smem_u32(sP + pb * C::P_BYTES), v0 = smem_u32(sV + st * C::V_BYTES);
+          const uint64_t p0 = sdesc_kmajor_sw128(smem_u32(sP + pb * C::P_BYTES));
+          const uint64_t v0 = sdesc_kmajor_sw128(smem_u32(sV + st * C::V_BYTES));
 #pragma unroll
           for (int kk = 0; kk < TKV / 16; ++kk)
-            umma_bf16(t_o, sdesc_kmajor_sw128(p0 + kk * 32), sdesc_kmajor_sw128(v0 + kk * 32), idesc_o,
+            umma_bf16(t_o, p0 + ((kk * 32) >> 4), v0 + ((kk * 32) >> 4), idesc_o,
                       (j != 0) || (kk != 0));
           umma_commit(o_full);
           umma_commit(&kv_empty[st]);
@@ -550,9 +589,9 @@ __global__ void __launch_bounds__(192, AttnDbCfg<HD_>::MIN_BLOCKS)
       }
       umma_commit(drain);
       volatile int never = 0;
-      mbar_wait_bounded(drain, 0, &never, args.status);
+      warp_wait_bounded(drain, 0, &never, args.status);
     }
-  } else {
+  } else if ((warp & 3) < act_warps) {
     // --------------------------------------------------------------- softmax
     // One virtual query row per thread (row = TMEM lane), the reference-max
     // scheme of attn_tc_kernel (O rescaled only when a tile's max exceeds the
@@ -578,7 +617,7 @@ __global__ void __launch_bounds__(192, AttnDbCfg<HD_>::MIN_BLOCKS)
         }
       }
       fence_proxy_async_smem();
-      mbar_arrive(q_full);
+      warp_arrive(q_full);
     }
     float m_ref = -INFINITY, l_run = 0.0f;
     bool ok = true;
@@ -598,18 +637,11 @@ __global__ void __launch_bounds__(192, AttnDbCfg<HD_>::MIN_BLOCKS)
       tmem_bind(rb);
       // S is in registers: its TMEM buffer goes back to the MMA thread (S(i+2)) at once
       tc_fence_before();
-      mbar_arrive(&s_free[sb]);
+      warp_arrive(&s_free[sb]);
       // pass 1: row max over the tile (both halves stay in registers for pass 2)
       float mxa[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-      if (masked) {
-#pragma unroll
-        for (int k = 0; k < 32; ++k)
-          mxa[k & 3] = fmax3(mxa[k & 3], k < lim ? __uint_as_float(ra[k]) : -INFINITY,
-                             32 + k < lim ? __uint_as_float(rb[k]) : -INFINITY);
-      } else {
-#pragma unroll
-        for (int k = 0; k < 32; ++k) mxa[k & 3] = fmax3(mxa[k & 3], __uint_as_float(ra[k]), __uint_as_float(rb[k]));
-      }
+      if (masked) max64<true>(ra, rb, 0, lim, mxa);
+      else max64<false>(ra, rb, 0, 64, mxa);
       const float m_tile = fmax3(fmaxf(mxa[0], mxa[1]), mxa[2], mxa[3]) * args.scale_log2;
       float m_new = m_ref, factor = 1.0f;
       if (m_ref == -INFINITY) {
@@ -638,29 +670,12 @@ __global__ void __launch_bounds__(192, AttnDbCfg<HD_>::MIN_BLOCKS)
       uint8_t* prow = sP + sb * C::P_BYTES + row * 128;
       const uint64_t negm2 = f2_pack(-m_new, -m_new);
       uint64_t ps2[2] = {0, 0};
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        const uint32_t* r = c ? rb : ra;
-        uint32_t pk[16];
-#pragma unroll
-        for (int k = 0; k < 32; k += 2) {
-          float x0, x1;
-          f2_unpack(f2_fma(f2_pack(__uint_as_float(r[k]), __uint_as_float(r[k + 1])), sc2, negm2), x0, x1);
-          float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
-          if (masked) {
-            p0 = 32 * c + k < lim ? p0 : 0.0f;
-            p1 = 32 * c + k + 1 < lim ? p1 : 0.0f;
-          }
-          ps2[(k >> 1) & 1] = f2_add(ps2[(k >> 1) & 1], f2_pack(p0, p1));
-          __nv_bfloat162 t = __floats2bfloat162_rn(p0, p1);
-          pk[k / 2] = *reinterpret_cast<uint32_t*>(&t);
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int chunk = c * 4 + q;
-          *reinterpret_cast<uint4*>(prow + ((chunk ^ (row & 7)) << 4)) =
-              make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
-        }
+      if (masked) {
+        exp32<true>(ra, sc2, negm2, 0, lim, ps2, prow, 0, row);
+        exp32<true>(rb, sc2, negm2, 0, lim - 32, ps2, prow, 4, row);
+      } else {
+        exp32<false>(ra, sc2, negm2, 0, 64, ps2, prow, 0, row);
+        exp32<false>(rb, sc2, negm2, 0, 64, ps2, prow, 4, row);
       }
       float a0, a1, b0, b1;
       f2_unpack(ps2[0], a0, a1);
@@ -668,7 +683,7 @@ __global__ void __launch_bounds__(192, AttnDbCfg<HD_>::MIN_BLOCKS)
       l_run += (a0 + a1) + (b0 + b1);
       m_ref = m_new;
       fence_proxy_async_smem();
-      mbar_arrive(&p_full[sb]);
+      warp_arrive(&p_full[sb]);
     }
     // o_done, not o_full: at this point P V(n-2) may still be running as well
     if (ok && n_tiles > 0 && warp_wait_bounded(o_done, 0, abort_flag, args.status)) {

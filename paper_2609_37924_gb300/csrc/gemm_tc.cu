@@ -239,28 +239,27 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------------------------------------------------------- MMA issuer
+      // ---------------------------------------------------------------- MMA issuer (the whole warp, one elected lane)
       constexpr uint32_t idesc = idesc_bf16_f32(BM, BN);
       int stage = 0;
       uint32_t phase = 0;
       int acc = 0;
       uint32_t acc_phase = 0;
-      for (int unit = blockIdx.x; unit < units && !*abort_flag; unit += gridDim.x) {
+      for (int unit = blockIdx.x; unit < units; unit += gridDim.x) {
         const int ks = unit % args.splits;
         const int kb0 = ks * args.kb_per_split, kb1 = min(kblocks, kb0 + args.kb_per_split);
-        if (!mbar_wait_bounded(&tempty[acc], acc_phase ^ 1, abort_flag, args.status)) break;
+        if (!warp_wait_bounded(&tempty[acc], acc_phase ^ 1, abort_flag, args.status)) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + acc * BN;
         bool ok = true;
         for (int kb = kb0; kb < kb1; ++kb) {
-          if (!mbar_wait_bounded(&full[stage], phase, abort_flag, args.status)) { ok = false; break; }
+          if (!warp_wait_bounded(&full[stage], phase, abort_flag, args.status)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t a0 = smem_u32(sA + stage * A_BYTES);
-          const uint32_t b0 = smem_u32(sB + stage * B_BYTES);
+          const uint64_t a0 = sdesc_kmajor_sw128(smem_u32(sA + stage * A_BYTES));
+          const uint64_t b0 = sdesc_kmajor_sw128(smem_u32(sB + stage * B_BYTES));
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k) {
-            umma_bf16(d_tmem, sdesc_kmajor_sw128(a0 + 32 * k), sdesc_kmajor_sw128(b0 + 32 * k), idesc,
+            umma_bf16(d_tmem, a0 + 2 * k, b0 + 2 * k, idesc,
                       (kb != kb0) || (k != 0));
           }
           umma_commit(&empty[stage]);
@@ -270,11 +269,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         umma_commit(&tfull[acc]);
         if (++acc == 2) { acc = 0; acc_phase ^= 1; }
       }
-      // all MMAs issued by this thread are complete before TMEM is freed
+      // all MMAs issued by this warp are complete before TMEM is freed
       umma_commit(drain);
       volatile int never = 0;
-      mbar_wait_bounded(drain, 0, &never, args.status);
-    }
+      warp_wait_bounded(drain, 0, &never, args.status);
   } else {
     // ------------------------------------------------------------------ epilogue
     const int quad = warp & 3;               // TMEM lanes 32*quad .. 32*quad+31 (hardware rule)
@@ -432,28 +430,28 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && leader) {
-      // ---------------------------------------------------------------- MMA issuer (even CTA)
+    if (leader) {
+      // ---------------------------------------------------------------- MMA issuer (even CTA; the whole warp, one elected lane)
       constexpr uint32_t idesc = idesc_bf16_f32(2 * BM, PBN);
       int stage = 0;
       uint32_t phase = 0;
       int acc = 0;
       uint32_t acc_phase = 0;
-      for (int unit = u0; unit < units && !*abort_flag; unit += ustep) {
+      for (int unit = u0; unit < units; unit += ustep) {
         const int ks = unit % args.splits;
         const int kb0 = ks * args.kb_per_split, kb1 = min(kblocks, kb0 + args.kb_per_split);
-        if (!mbar_wait_bounded(&tempty[acc], acc_phase ^ 1, abort_flag, args.status)) break;
+        if (!warp_wait_bounded(&tempty[acc], acc_phase ^ 1, abort_flag, args.status)) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + acc * PBN;
         bool ok = true;
         for (int kb = kb0; kb < kb1; ++kb) {
-          if (!mbar_wait_bounded(&full[stage], phase, abort_flag, args.status)) { ok = false; break; }
+          if (!warp_wait_bounded(&full[stage], phase, abort_flag, args.status)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t a0 = smem_u32(sA + stage * P_A_BYTES);
-          const uint32_t b0 = smem_u32(sB + stage * P_B_BYTES);
+          const uint64_t a0 = sdesc_kmajor_sw128(smem_u32(sA + stage * P_A_BYTES));
+          const uint64_t b0 = sdesc_kmajor_sw128(smem_u32(sB + stage * P_B_BYTES));
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k) {
-            umma_bf16_pair(d_tmem, sdesc_kmajor_sw128(a0 + 32 * k), sdesc_kmajor_sw128(b0 + 32 * k), idesc,
+            umma_bf16_pair(d_tmem, a0 + 2 * k, b0 + 2 * k, idesc,
                            (kb != kb0) || (k != 0));
           }
           umma_commit_pair_mc(&empty[stage], 0x3);
@@ -466,7 +464,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       // every pair MMA is complete (both CTAs' TMEM written) before TMEM is freed
       umma_commit_pair_mc(drain, 0x1);
       volatile int never = 0;
-      mbar_wait_bounded(drain, 0, &never, args.status);
+      warp_wait_bounded(drain, 0, &never, args.status);
     }
   } else {
     // ------------------------------------------------------------------ epilogue (both CTAs)
