@@ -133,21 +133,25 @@ struct TcArgs {
 
 // Tiles run N-fastest: the CTAs in flight share A tiles (activations, the
 // large operand) through L2, and every weight matrix of the model fits in L2.
-// At the start of a tile the producer asks L2 for the global rows its
-// epilogue will read (residual stream, h, gate), so the epilogue does not wait
-// on DRAM latency.
+// While the MMA warp fills an accumulator, its epilogue warps ask L2 for the
+// fp32 rows that their epilogue will read (h, base): each lane its own row's
+// share of the tile's columns, so the epilogue does not wait on DRAM latency.
+// The producer thread must not do this: 128 prefetches, one per row, kept it
+// from its loads for about 12,000 cycles per tile, two thirds of a 12-k-block
+// tile (16 x 1024 rows, d 768: the layer's W_o and W_down took 113 us, now
+// 83).  The residual epilogue needs no prefetch: its TMA reduce-adds are
+// performed at L2 and nothing waits for them (with one from the epilogue
+// lanes the layers are 0.7 % slower).
 template <int EPI>
-__device__ __forceinline__ void prefetch_epilogue_inputs(const TcArgs& a, int mb, int nb, int ncols = BN) {
-  const EpiParams& p = a.ep;
-  const float* src = nullptr;
-  int ld = 0;
-  if constexpr (EPI == EPI_RESID) { src = p.resid; ld = p.ldr; }
-  else if constexpr (EPI == EPI_FUSION2 || EPI == EPI_ADD || EPI == EPI_PA_UP) { src = p.base; ld = p.ldb; }
-  if (!src) return;
-  const int n0 = nb * ncols, ncol = min(ncols, p.N - n0);
-  if (ncol <= 0 || (ld & 3) || (n0 & 3)) return;
-  const uint32_t bytes = static_cast<uint32_t>(ncol) * 4u & ~15u;
-  for (int r = mb * BM; r < min(mb * BM + BM, p.M); ++r) prefetch_l2(src + static_cast<size_t>(r) * ld + n0, bytes);
+__device__ __forceinline__ void prefetch_epilogue_inputs(const TcArgs& a, int m, int nb, int part, int nsplit,
+                                                         int ncols = BN) {
+  if constexpr (EPI == EPI_FUSION2 || EPI == EPI_ADD || EPI == EPI_PA_UP) {
+    const EpiParams& p = a.ep;
+    const int w = ncols / nsplit, n0 = nb * ncols + part * w, ncol = min(w, p.N - n0);
+    if (ncol <= 0 || m >= p.M || (p.ldb & 3) || (reinterpret_cast<uintptr_t>(p.base) & 15)) return;
+    const uint32_t bytes = static_cast<uint32_t>(ncol) * 4u & ~15u;
+    if (bytes) prefetch_l2(p.base + static_cast<size_t>(m) * p.ldb + n0, bytes);
+  }
 }
 
 template <int EPI>
@@ -211,7 +215,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         const int tile = unit / args.splits, ks = unit % args.splits;
         const int nb = tile % args.n_tiles_n, mb = tile / args.n_tiles_n;
         const int kb0 = ks * args.kb_per_split, kb1 = min(kblocks, kb0 + args.kb_per_split);
-        if (args.splits == 1) prefetch_epilogue_inputs<EPI>(args, mb, nb);
         bool ok = true;
         for (int kb = kb0; kb < kb1; ++kb) {
           if (!mbar_wait_bounded(&empty[stage], phase ^ 1, abort_flag, args.status)) { ok = false; break; }
@@ -281,10 +284,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     int acc = 0;
     uint32_t acc_phase = 0;
     for (int unit = blockIdx.x; unit < units; unit += gridDim.x) {
-      if (!warp_wait_bounded(&tfull[acc], acc_phase, abort_flag, args.status)) break;
-      tc_fence_after();
       const int tile = unit / args.splits, ks = unit % args.splits;
       const int nb = tile % args.n_tiles_n, mb = tile / args.n_tiles_n;
+      if (args.splits == 1 && part < nsplit)
+        prefetch_epilogue_inputs<EPI>(args, mb * BM + quad * 32 + lane, nb, part, nsplit);
+      if (!warp_wait_bounded(&tfull[acc], acc_phase, abort_flag, args.status)) break;
+      tc_fence_after();
       TmemSrc src{tmem_base + static_cast<uint32_t>(acc * BN) + (static_cast<uint32_t>(quad * 32) << 16),
                   args.staged ? sOut + (warp - 2) * STAGE_OUT_BYTES : nullptr, {&tmC, &tmC2}, mb * BM + quad * 32};
       const int m = mb * BM + quad * 32 + lane;
@@ -406,7 +411,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         const int nb = tile % args.n_tiles_n;
         const int mb = 2 * (tile / args.n_tiles_n) + static_cast<int>(rank);   // this CTA's 128-row block
         const int kb0 = ks * args.kb_per_split, kb1 = min(kblocks, kb0 + args.kb_per_split);
-        if (args.splits == 1) prefetch_epilogue_inputs<EPI>(args, mb, nb, PBN);
         const int brow = args.b_split > 0 ? (rank ? args.b_split : 0) + nb * (PBN / 2) : nb * PBN + rank * (PBN / 2);
         bool ok = true;
         for (int kb = kb0; kb < kb1; ++kb) {
@@ -475,11 +479,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
     int acc = 0;
     uint32_t acc_phase = 0;
     for (int unit = u0; unit < units; unit += ustep) {
-      if (!warp_wait_bounded(&tfull[acc], acc_phase, abort_flag, args.status)) break;
-      tc_fence_after();
       const int tile = unit / args.splits, ks = unit % args.splits;
       const int nb = tile % args.n_tiles_n;
       const int mb = 2 * (tile / args.n_tiles_n) + static_cast<int>(rank);
+      if (args.splits == 1 && part < nsplit)
+        prefetch_epilogue_inputs<EPI>(args, mb * BM + quad * 32 + lane, nb, part, nsplit, PBN);
+      if (!warp_wait_bounded(&tfull[acc], acc_phase, abort_flag, args.status)) break;
+      tc_fence_after();
       TmemSrc src{tmem_base + static_cast<uint32_t>(acc * PBN) + (static_cast<uint32_t>(quad * 32) << 16),
                   args.staged ? sOut + (warp - 2) * STAGE_OUT_BYTES : nullptr, {&tmC, &tmC2}, mb * BM + quad * 32};
       const int m = mb * BM + quad * 32 + lane;
