@@ -130,7 +130,6 @@ template <int HD, int TKV, bool WIN>
 __global__ void __launch_bounds__(192, AttnTcCfg<HD, TKV>::MIN_BLOCKS)
     attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                    const AttnTcArgs args) {
-  pdl_enter();
   using C = AttnTcCfg<HD, TKV>;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = smem_raw;
@@ -197,6 +196,7 @@ __global__ void __launch_bounds__(192, AttnTcCfg<HD, TKV>::MIN_BLOCKS)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_enter();   // barriers and TMEM are set up while the previous kernel finishes
   const uint32_t tmem = *tmem_slot;
   const uint32_t t_s = tmem, t_o = tmem + TKV;
 
@@ -462,7 +462,6 @@ template <int HD_>
 __global__ void __launch_bounds__(192, AttnDbCfg<HD_>::MIN_BLOCKS)
     attn_db_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                    const AttnTcArgs args) {
-  pdl_enter();
   using C = AttnDbCfg<HD_>;
   constexpr int HD = C::HD, TKV = C::TKV, NST = C::STAGES;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -524,6 +523,7 @@ __global__ void __launch_bounds__(192, AttnDbCfg<HD_>::MIN_BLOCKS)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_enter();   // barriers and TMEM are set up while the previous kernel finishes
   const uint32_t tmem = *tmem_slot;
   const uint32_t t_o = tmem + 2 * TKV;
 

@@ -216,11 +216,14 @@ __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint
 // umma_commit: arrive once on `bar` when every tcgen05 op issued so far by the
 // elected lane is done (warp-collective).
 // -------------------------------------------- programmatic dependent launch
-// Every kernel of the library calls this before its first global-memory
-// access: it waits until the previous kernel of the stream has completed and
-// its writes are visible (a no-op when there is no programmatic dependency),
-// then lets the next kernel start launching; that kernel's CTAs wait in this
-// same call before they touch memory, so only launch latency overlaps.
+// Every kernel of the library calls this before its first access to memory
+// that another kernel writes: it waits until the previous kernel of the
+// stream has completed and its writes are visible (a no-op when there is no
+// programmatic dependency), then lets the next kernel start launching; that
+// kernel's CTAs wait in this same call, so launch latency and whatever a
+// kernel does ahead of the call (barriers, TMEM, the first weight tiles)
+// overlap the end of its predecessor.  The wait comes before the release:
+// when a kernel starts, every kernel before its predecessor has completed.
 __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -126,6 +126,7 @@ struct TcArgs {
   int kb_wrap;             // > 0: split hi + lo operand of kb_wrap k-blocks per half: k-block kb reads A's
                            // k-block (kb odd ? kb_wrap : 0) + kb / 2 and B's k-block kb / 2, so that the two
                            // reads of a B tile follow each other (the second one hits L2)
+  int b_early;             // B is constant (model weights): its first stages load ahead of pdl_enter
   int* status;
   const int* m_dev;        // optional device row count (<= M): tiles past it are skipped
   EpiParams ep;
@@ -159,7 +160,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmC2,
                    const TcArgs args) {
-  pdl_enter();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sA = smem;
@@ -198,11 +198,34 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
+  const int kblocks = (args.K + BK - 1) / BK;
+  auto k_of_a = [&](int kb) { return (args.kb_wrap > 0 ? (kb & 1) * args.kb_wrap + (kb >> 1) : kb) * BK; };
+  auto load_b = [&](int stage, int kb, int nb) {
+    const int x = (args.kb_wrap > 0 ? kb >> 1 : kb) * BK;
+    if (args.b_split > 0) {
+      tma_load_2d(sB + stage * B_BYTES, &tmB, &full[stage], x, nb * (BN / 2));
+      tma_load_2d(sB + stage * B_BYTES + B_BYTES / 2, &tmB, &full[stage], x, args.b_split + nb * (BN / 2));
+    } else {
+      tma_load_2d(sB + stage * B_BYTES, &tmB, &full[stage], x, nb * BN);
+    }
+  };
+  // constant B: the first unit's first B tiles are on their way while the
+  // previous kernel finishes (without m_dev every CTA has a first unit)
+  int pre = 0;
+  if (args.b_early && warp == 0 && lane == 0) {
+    const int tile = blockIdx.x / args.splits, kb0 = (blockIdx.x % args.splits) * args.kb_per_split;
+    pre = min(STAGES, min(kblocks, kb0 + args.kb_per_split) - kb0);
+    for (int s = 0; s < pre; ++s) {
+      mbar_arrive_expect_tx(&full[s], STAGE_BYTES);
+      load_b(s, kb0 + s, tile % args.n_tiles_n);
+    }
+  }
+  pdl_enter();
+
   const int m_run = args.m_dev ? min(args.M, *args.m_dev) : args.M;   // read after pdl_enter
   const int num_m = (m_run + BM - 1) / BM;
   const int tiles = num_m * args.n_tiles_n;
   const int units = tiles * args.splits;
-  const int kblocks = (args.K + BK - 1) / BK;
 
   if (warp == 0) {
     if (lane == 0) {
@@ -218,17 +241,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         bool ok = true;
         for (int kb = kb0; kb < kb1; ++kb) {
           if (!mbar_wait_bounded(&empty[stage], phase ^ 1, abort_flag, args.status)) { ok = false; break; }
-          mbar_arrive_expect_tx(&full[stage], STAGE_BYTES);
-          const int kba = args.kb_wrap > 0 ? (kb & 1) * args.kb_wrap + (kb >> 1) : kb;
-          const int kbb = args.kb_wrap > 0 ? kb >> 1 : kb;
-          tma_load_2d(sA + stage * A_BYTES, &tmA, &full[stage], kba * BK, mb * BM);
-          if (args.b_split > 0) {
-            tma_load_2d(sB + stage * B_BYTES, &tmB, &full[stage], kbb * BK, nb * (BN / 2));
-            tma_load_2d(sB + stage * B_BYTES + B_BYTES / 2, &tmB, &full[stage], kbb * BK,
-                        args.b_split + nb * (BN / 2));
+          if (pre > 0) {
+            --pre;                 // B of this stage is already on its way
           } else {
-            tma_load_2d(sB + stage * B_BYTES, &tmB, &full[stage], kbb * BK, nb * BN);
+            mbar_arrive_expect_tx(&full[stage], STAGE_BYTES);
+            load_b(stage, kb, nb);
           }
+          tma_load_2d(sA + stage * A_BYTES, &tmA, &full[stage], k_of_a(kb), mb * BM);
           ++issued[stage];
           if (++stage == STAGES) { stage = 0; phase ^= 1; }
         }
@@ -349,7 +368,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
     gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmC2,
                     const TcArgs args) {
-  pdl_enter();
   using PC = PairCfg<PBN>;
   constexpr int P_STAGES = PC::STAGES, P_A_BYTES = PC::A_BYTES, P_B_BYTES = PC::B_BYTES;
   constexpr int P_STAGE_BYTES = PC::STAGE_BYTES;
@@ -394,16 +412,36 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
+  const int kblocks = (args.K + BK - 1) / BK;
+  const int u0 = static_cast<int>(blockIdx.x >> 1), ustep = static_cast<int>(gridDim.x >> 1);
+  const uint32_t full_l0 = cluster_addr(full, 0);   // the even CTA's full[0]
+  auto k_of_a = [&](int kb) { return (args.kb_wrap > 0 ? (kb & 1) * args.kb_wrap + (kb >> 1) : kb) * BK; };
+  auto load_b = [&](int stage, int kb, int nb) {   // this CTA's half of the B tile
+    const int x = (args.kb_wrap > 0 ? kb >> 1 : kb) * BK;
+    const int brow = args.b_split > 0 ? (rank ? args.b_split : 0) + nb * (PBN / 2)
+                                      : nb * PBN + static_cast<int>(rank) * (PBN / 2);
+    tma_load_2d_pair(sB + stage * P_B_BYTES, &tmB, full_l0 + 8u * stage, x, brow);
+  };
+  // constant B: the first unit's first B tiles are on their way while the
+  // previous kernel finishes (without m_dev every cluster has a first unit)
+  int pre = 0;
+  if (args.b_early && warp == 0 && lane == 0) {
+    const int tile = u0 / args.splits, kb0 = (u0 % args.splits) * args.kb_per_split;
+    pre = min(P_STAGES, min(kblocks, kb0 + args.kb_per_split) - kb0);
+    for (int s = 0; s < pre; ++s) {
+      if (leader) mbar_arrive_expect_tx(&full[s], 2 * P_STAGE_BYTES);
+      load_b(s, kb0 + s, tile % args.n_tiles_n);
+    }
+  }
+  pdl_enter();
+
   const int m_run = args.m_dev ? min(args.M, *args.m_dev) : args.M;   // read after pdl_enter
   const int num_m2 = (m_run + 2 * BM - 1) / (2 * BM);
   const int units = num_m2 * args.n_tiles_n * args.splits;   // unit = (pair tile, K slice)
-  const int u0 = static_cast<int>(blockIdx.x >> 1), ustep = static_cast<int>(gridDim.x >> 1);
-  const int kblocks = (args.K + BK - 1) / BK;
 
   if (warp == 0) {
     if (lane == 0) {
       // ---------------------------------------------------------------- producer (both CTAs)
-      const uint32_t full_l0 = cluster_addr(full, 0);   // the even CTA's full[0]
       int stage = 0;
       uint32_t phase = 0;
       for (int unit = u0; unit < units && !*abort_flag; unit += ustep) {
@@ -411,16 +449,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         const int nb = tile % args.n_tiles_n;
         const int mb = 2 * (tile / args.n_tiles_n) + static_cast<int>(rank);   // this CTA's 128-row block
         const int kb0 = ks * args.kb_per_split, kb1 = min(kblocks, kb0 + args.kb_per_split);
-        const int brow = args.b_split > 0 ? (rank ? args.b_split : 0) + nb * (PBN / 2) : nb * PBN + rank * (PBN / 2);
         bool ok = true;
         for (int kb = kb0; kb < kb1; ++kb) {
           if (!mbar_wait_bounded(&empty[stage], phase ^ 1, abort_flag, args.status)) { ok = false; break; }
-          if (leader) mbar_arrive_expect_tx(&full[stage], 2 * P_STAGE_BYTES);
-          const uint32_t fb = full_l0 + 8u * stage;
-          const int kba = args.kb_wrap > 0 ? (kb & 1) * args.kb_wrap + (kb >> 1) : kb;
-          const int kbb = args.kb_wrap > 0 ? kb >> 1 : kb;
-          tma_load_2d_pair(sA + stage * P_A_BYTES, &tmA, fb, kba * BK, mb * BM);
-          tma_load_2d_pair(sB + stage * P_B_BYTES, &tmB, fb, kbb * BK, brow);
+          if (pre > 0) {
+            --pre;                 // B of this stage is already on its way
+          } else {
+            if (leader) mbar_arrive_expect_tx(&full[stage], 2 * P_STAGE_BYTES);
+            load_b(stage, kb, nb);
+          }
+          tma_load_2d_pair(sA + stage * P_A_BYTES, &tmA, full_l0 + 8u * stage, k_of_a(kb), mb * BM);
           if (++stage == P_STAGES) { stage = 0; phase ^= 1; }
         }
         if (!ok) break;
@@ -649,6 +687,7 @@ const char* gemm_tc(const GemmCall& g, cudaStream_t s) {
   if (g.epi == EPI_PA_GATE && g.N > BN) return "gate GEMM needs N <= 256";
   a.status = g.status;
   a.m_dev = g.m_dev;
+  a.b_early = g.b_weights && !g.m_dev;
   a.ep = g.ep;
   a.ep.M = g.M;
   a.ep.N = g.N;

@@ -37,6 +37,8 @@ struct GemmCall {
   int* status;
   const int* m_dev = nullptr;   // optional device row count <= M (tcgen05 path): tiles past it are skipped
   int k_b = 0;           // > 0: B has k_b columns and A's K = 2 k_b columns [hi | lo] both multiply B (split operand)
+  bool b_weights = false;   // B was written before the previous kernel of the stream started (model weights):
+                            // the tensor-core kernels may load it ahead of their grid dependency
   float* split_buf;      // fp32 partials for split-K (null: no split)
   size_t split_bytes;
   int launched;          // out: kernels launched

@@ -323,9 +323,11 @@ void probe_end(tadm_handle* h, cudaStream_t s, int idx, int kind, double flops, 
 // the recorded work is that of the k_b-deep product the method computes.
 tadm_status gemm(tadm_handle* h, const void* A, int64_t a_rows, int lda, const void* B, int ldb, int M, int N, int K,
                  int epi, const EpiParams& ep, cudaStream_t s, bool out_f32 = false, const int* m_dev = nullptr,
-                 int k_b = 0) {
+                 int k_b = 0, bool b_weights = true) {
   GemmCall g{};
   g.k_b = k_b;
+  // every call here follows another kernel of the same stream, whose own wait covered whatever wrote the weights
+  g.b_weights = b_weights;
   g.A = A;
   g.B = B;
   g.M = M;
@@ -1494,7 +1496,8 @@ tadm_status tadm_generate_entropy_bound(tadm_handle* h, const int32_t* prompt, i
         EpiParams es{};
         es.out = sig;
         es.ldo = c.d_model;
-        TRYS(gemm(h, p, n_rows, c.vocab, et, c.vocab, n_rows, c.d_model, c.vocab, EPI_STORE, es, s, true));
+        TRYS(gemm(h, p, n_rows, c.vocab, et, c.vocab, n_rows, c.d_model, c.vocab, EPI_STORE, es, s, true, nullptr, 0,
+                  false));                    // E^T is written by this call
       }
       TRY(eb_accept(ent, batch, R, prompt_len, out, total, c.vocab, eta, seed, i, s));
     }
