@@ -30,6 +30,7 @@ struct EpiParams {
   float* resid;
   int ldr;
   int resid_tma;            // EPI_RESID on the tensor-core path: resid += acc by TMA reduce-add (map in the source)
+  int f32_tma;              // EPI_STORE (fp32) / EPI_LMHEAD logits on the tensor-core path: TMA stores (map in the source)
   const float* base;        // EPI_ADD base, EPI_FUSION2 h, EPI_PA_UP H0
   int ldb;
   const void* bias;         // [N] weights dtype
@@ -300,6 +301,12 @@ __device__ __forceinline__ void epilogue_row(const EpiParams& p, int m, int n_bl
       src.load(c, v);
       const int n0 = n_blk * ncols + 32 * c;
       const int nv = min(32, p.N - n0);
+      if constexpr (Src::kStaged && EPI == EPI_STORE) {
+        if (p.f32_tma) {
+          if (nv > 0 && src.row0 < p.M) src.store32f(n0, v);   // the map clips ragged rows / columns
+          continue;
+        }
+      }
       if (!row_ok || nv <= 0) continue;
       const size_t mrow = static_cast<size_t>(m);
       if constexpr (EPI == EPI_STORE) {
@@ -498,8 +505,15 @@ __device__ __forceinline__ void epilogue_row(const EpiParams& p, int m, int n_bl
       src.load(c, v);
       const int n0 = n_blk * ncols + 32 * c;
       const int nv = min(32, p.N - n0);
+      bool stored = false;
+      if constexpr (Src::kStaged) {
+        if (p.f32_tma && nv > 0 && src.row0 < p.M) {
+          src.store32f(n0, v);
+          stored = true;
+        }
+      }
       if (!row_ok || nv <= 0) continue;
-      if (p.logits) store32(p.logits, 0, static_cast<size_t>(m) * p.ld_logits + n0, v, nv);
+      if (p.logits && !stored) store32(p.logits, 0, static_cast<size_t>(m) * p.ld_logits + n0, v, nv);
       float cmx = -INFINITY;
       int carg = -1;
 #pragma unroll

@@ -44,11 +44,12 @@ constexpr size_t SMEM_BYTES = 1024 + STAGES * STAGE_BYTES + EPI_WARPS * STAGE_OU
 struct TmemSrc {
   static constexpr bool kStaged = true;
   uint32_t taddr;
-  uint8_t* stage;                      // 32 rows x 128 B, 128-byte swizzle; null: direct stores
+  uint8_t* stage;                      // 32 rows x 128 B, 128-byte swizzle
+  bool use_stage;                      // bf16 outputs / residual rows go through the box
   const CUtensorMap* tm_out[2];
   int row0;                            // first of the warp's 32 output rows
-  __device__ __forceinline__ bool staged() const { return stage != nullptr; }
-  __device__ __forceinline__ bool has_box() const { return stage != nullptr; }
+  __device__ __forceinline__ bool staged() const { return use_stage; }
+  __device__ __forceinline__ bool has_box() const { return use_stage; }
   // row `lane` of a 32 x 32 fp32 box (128-byte rows, 16-byte chunks XOR-swizzled by row)
   __device__ __forceinline__ void put_row(const float (&v)[32]) {
     const int lane = threadIdx.x & 31;
@@ -83,6 +84,22 @@ struct TmemSrc {
     __syncwarp();
     if (lane == 0) {
       tma_reduce_add_2d(tm_out[0], stage, x, row0);
+      bulk_commit();
+    }
+  }
+  // the same box, stored instead of added: one TMA store of the warp's 32 x 32
+  // fp32 chunk at column x (whole 128-byte lines; a lane storing its own row
+  // writes 32 rows x 16 bytes per instruction).  slice < 0: the 2-D output
+  // map; otherwise K slice `slice` of the 3-D map of split-K partials.
+  __device__ __forceinline__ void store32f(int x, const float (&v)[32], int slice = -1) {
+    const int lane = threadIdx.x & 31;
+    if (lane == 0) bulk_wait_read0();   // the previous store has read the box
+    put_row(v);
+    fence_proxy_async_smem();
+    __syncwarp();
+    if (lane == 0) {
+      if (slice < 0) tma_store_2d(tm_out[0], stage, x, row0);
+      else tma_store_3d(tm_out[0], stage, x, row0, slice);
       bulk_commit();
     }
   }
@@ -121,6 +138,7 @@ struct TcArgs {
   size_t part_stride;
   int ldp;
   int staged;              // bf16 outputs go through the per-warp boxes and TMA stores
+  int part_tma;            // split-K partials go through them too (tmC: the 3-D map [splits][M][ldp])
   int b_split;             // >0: B tile = 128 rows at n*128 and 128 rows at b_split + n*128
   int n_tiles_n;
   int kb_wrap;             // > 0: split hi + lo operand of kb_wrap k-blocks per half: k-block kb reads A's
@@ -310,7 +328,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       if (!warp_wait_bounded(&tfull[acc], acc_phase, abort_flag, args.status)) break;
       tc_fence_after();
       TmemSrc src{tmem_base + static_cast<uint32_t>(acc * BN) + (static_cast<uint32_t>(quad * 32) << 16),
-                  args.staged ? sOut + (warp - 2) * STAGE_OUT_BYTES : nullptr, {&tmC, &tmC2}, mb * BM + quad * 32};
+                  sOut + (warp - 2) * STAGE_OUT_BYTES, args.staged != 0, {&tmC, &tmC2}, mb * BM + quad * 32};
       const int m = mb * BM + quad * 32 + lane;
       if (args.splits > 1) {
         // raw fp32 partial of this K slice, tile-local column order
@@ -318,7 +336,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         float* dst = args.part + ks * args.part_stride + static_cast<size_t>(m) * args.ldp + nb * BN;
         for (int c = part * (BN / 64); c < (part + 1) * (BN / 64); ++c) {
           src.load(c, v);
-          if (m < args.M) store32(dst, 0, 32 * c, v, 32);
+          if (!args.part_tma) {
+            if (m < args.M) store32(dst, 0, 32 * c, v, 32);
+          } else if (src.row0 < args.M) {
+            src.store32f(nb * BN + 32 * c, v, ks);   // the map clips ragged rows
+          }
         }
       } else if (part < nsplit) {
         epilogue_row<EPI>(args.ep, m, nb, BN, src, part, nsplit);
@@ -327,7 +349,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       mbar_arrive(&tempty[acc]);
       if (++acc == 2) { acc = 0; acc_phase ^= 1; }
     }
-    if (args.staged && lane == 0) bulk_wait0();   // every TMA store of this warp (if any) is complete
+    if (lane == 0) bulk_wait0();   // every TMA store of this warp (if any) is complete
   }
 
   tc_fence_before();
@@ -525,7 +547,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       if (!warp_wait_bounded(&tfull[acc], acc_phase, abort_flag, args.status)) break;
       tc_fence_after();
       TmemSrc src{tmem_base + static_cast<uint32_t>(acc * PBN) + (static_cast<uint32_t>(quad * 32) << 16),
-                  args.staged ? sOut + (warp - 2) * STAGE_OUT_BYTES : nullptr, {&tmC, &tmC2}, mb * BM + quad * 32};
+                  sOut + (warp - 2) * STAGE_OUT_BYTES, args.staged != 0, {&tmC, &tmC2}, mb * BM + quad * 32};
       const int m = mb * BM + quad * 32 + lane;
       if (args.splits > 1) {
         // raw fp32 partial of this K slice: this CTA's 128 rows of the pair tile, columns in natural order
@@ -534,7 +556,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
           float* dst = args.part + ks * args.part_stride + static_cast<size_t>(m) * args.ldp + nb * PBN;
           for (int c = part * (PBN / 64); c < (part + 1) * (PBN / 64); ++c) {
             src.load(c, v);
-            if (m < args.M) store32(dst, 0, 32 * c, v, 32);
+            if (!args.part_tma) {
+              if (m < args.M) store32(dst, 0, 32 * c, v, 32);
+            } else if (src.row0 < args.M) {
+              src.store32f(nb * PBN + 32 * c, v, ks);   // the map clips ragged rows
+            }
           }
         }
       } else if (part < nsplit && mb * BM < args.M) {   // the odd CTA's rows may lie past M
@@ -545,7 +571,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       if (lane == 0) mbar_arrive_remote(tempty_l0 + 8u * acc);
       if (++acc == 2) { acc = 0; acc_phase ^= 1; }
     }
-    if (args.staged && lane == 0) bulk_wait0();
+    if (lane == 0) bulk_wait0();
   }
 
   tc_fence_before();
@@ -603,6 +629,17 @@ bool make_f32_map(CUtensorMap* m, const void* ptr, int64_t rows, int64_t cols, i
   cuuint32_t box[2] = {32, 32};
   cuuint32_t estr[2] = {1, 1};
   return g_encode(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(ptr), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// 3-D fp32 map over the split-K partials [splits][rows][ldp], box 32 rows x 32 columns, 128-byte swizzle.
+bool make_part_map(CUtensorMap* m, const void* ptr, int64_t rows, int64_t ldp, int splits) {
+  cuuint64_t dims[3] = {static_cast<cuuint64_t>(ldp), static_cast<cuuint64_t>(rows), static_cast<cuuint64_t>(splits)};
+  cuuint64_t strides[2] = {static_cast<cuuint64_t>(ldp * 4), static_cast<cuuint64_t>(rows * ldp * 4)};
+  cuuint32_t box[3] = {32, 32, 1};
+  cuuint32_t estr[3] = {1, 1, 1};
+  return g_encode(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(ptr), dims, strides, box, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -697,6 +734,8 @@ const char* gemm_tc(const GemmCall& g, cudaStream_t s) {
   a.staged = 0;
   auto aligned = [](const void* p, int ld) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && ld % 8 == 0; };
   a.ep.resid_tma = 0;
+  a.ep.f32_tma = 0;
+  a.part_tma = 0;
   if (g.epi == EPI_RESID || g.epi == EPI_FUSION2) {
     a.staged = 1;   // the boxes serve as transpose scratch, or as the source of TMA reduce-adds
     if (g.epi == EPI_RESID && (reinterpret_cast<uintptr_t>(g.ep.resid) & 15) == 0 && g.ep.ldr % 4 == 0 &&
@@ -710,6 +749,14 @@ const char* gemm_tc(const GemmCall& g, cudaStream_t s) {
         make_out_map(&tc2, g.ep.out2, g.M, g.N - g.ep.d_split, g.ep.ldo2))
       a.staged = 1;
   }
+  // fp32 outputs of the plain epilogue and the head's logits: TMA stores of 32 x 32 boxes
+  const float* f32_out = g.epi == EPI_STORE && !g.ep.out_bf16 ? static_cast<const float*>(g.ep.out)
+                         : g.epi == EPI_LMHEAD                ? g.ep.logits
+                                                              : nullptr;
+  const int f32_ld = g.epi == EPI_STORE ? g.ep.ldo : g.ep.ld_logits;
+  if (f32_out && (reinterpret_cast<uintptr_t>(f32_out) & 15) == 0 && f32_ld % 4 == 0 &&
+      make_f32_map(&tc, f32_out, g.M, g.N, f32_ld))
+    a.ep.f32_tma = 1;
   const int tiles = ((g.M + BM - 1) / BM) * a.n_tiles_n;
   // split-K when the tiles cannot fill the SMs and K is long: fixed-order
   // reduction afterwards, so results do not depend on the split
@@ -750,6 +797,7 @@ const char* gemm_tc(const GemmCall& g, cudaStream_t s) {
       a2.part = g.split_buf;
       a2.part_stride = static_cast<size_t>(g.M) * a2.ldp;
       a2.staged = 0;
+      a2.part_tma = make_part_map(&tc, a2.part, g.M, a2.ldp, a2.splits);
       const cudaError_t e = g.epi == EPI_RESID ? launch_epi_pair<EPI_RESID>(ta, tbh, tc, tc2, a2, pu * a2.splits, s)
                                                : launch_epi_pair<EPI_STORE>(ta, tbh, tc, tc2, a2, pu * a2.splits, s);
       if (e != cudaSuccess) return cudaGetErrorString(e);
@@ -779,6 +827,7 @@ const char* gemm_tc(const GemmCall& g, cudaStream_t s) {
       a2.part = g.split_buf;
       a2.part_stride = static_cast<size_t>(g.M) * a2.ldp;
       a2.staged = 0;
+      a2.part_tma = make_part_map(&tc, a2.part, g.M, a2.ldp, a2.splits);
       const cudaError_t e = launch_epi_pair<EPI_QKV>(ta, tbh, tc, tc2, a2, pu * a2.splits, s);
       if (e != cudaSuccess) return cudaGetErrorString(e);
       const_cast<GemmCall&>(g).launched = 1;
@@ -799,6 +848,7 @@ const char* gemm_tc(const GemmCall& g, cudaStream_t s) {
       a.part = g.split_buf;
       a.part_stride = static_cast<size_t>(g.M) * a.ldp;
       a.staged = 0;
+      a.part_tma = make_part_map(&tc, a.part, g.M, a.ldp, a.splits);
     }
   }
   // CTA pairs (256 x 256 tiles, cta_group::2) for every unsplit GEMM of more
