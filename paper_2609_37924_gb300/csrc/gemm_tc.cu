@@ -749,12 +749,14 @@ const char* gemm_tc(const GemmCall& g, cudaStream_t s) {
         make_out_map(&tc2, g.ep.out2, g.M, g.N - g.ep.d_split, g.ep.ldo2))
       a.staged = 1;
   }
-  // fp32 outputs of the plain epilogue and the head's logits: TMA stores of 32 x 32 boxes
+  // fp32 outputs of the plain epilogue and the head's logits: TMA stores of
+  // 32 x 32 boxes, where the last column ends on 16 bytes (N % 4 == 0: TMA
+  // clips to 16 bytes, and columns past N are the caller's)
   const float* f32_out = g.epi == EPI_STORE && !g.ep.out_bf16 ? static_cast<const float*>(g.ep.out)
                          : g.epi == EPI_LMHEAD                ? g.ep.logits
                                                               : nullptr;
   const int f32_ld = g.epi == EPI_STORE ? g.ep.ldo : g.ep.ld_logits;
-  if (f32_out && (reinterpret_cast<uintptr_t>(f32_out) & 15) == 0 && f32_ld % 4 == 0 &&
+  if (f32_out && (reinterpret_cast<uintptr_t>(f32_out) & 15) == 0 && f32_ld % 4 == 0 && g.N % 4 == 0 &&
       make_f32_map(&tc, f32_out, g.M, g.N, f32_ld))
     a.ep.f32_tma = 1;
   const int tiles = ((g.M + BM - 1) / BM) * a.n_tiles_n;
