@@ -6,6 +6,8 @@
 //  - argmax ties go to the lowest id; selection ties to the lowest position;
 //  - carry-over: only positions still holding MASK are candidates, so
 //    unmasked tokens never change.
+#include <algorithm>
+
 #include "kernels.h"
 
 namespace tadm {
@@ -403,10 +405,57 @@ __global__ void __launch_bounds__(NT) remdm_sample_kernel(const float* __restric
   }
 }
 
-// remdm_sample_kernel with the row's probabilities staged once in shared
-// memory (q_v = exp(l_v - max), 0 for MASK; vocab * 4 bytes of dynamic
-// shared memory): the bisection sums read shared memory with a strided
-// (bank-conflict-free) assignment, the id-order draw uses contiguous ranges.
+// Sums of three values over the 32 lanes, in lanes 0 (v0), 8 (v1) and 16 (v2):
+// the first two exchange steps halve the number of values a lane carries, so
+// six shuffles do the work of fifteen.
+__device__ __forceinline__ float lane_sum3(float v0, float v1, float v2) {
+  const int lane = threadIdx.x & 31;
+  const bool h16 = lane & 16, h8 = lane & 8;
+  // lanes < 16 keep (v0, v1), lanes >= 16 keep (v2, 0)
+  const float a = (h16 ? v2 : v0) + __shfl_xor_sync(0xffffffffu, h16 ? v0 : v2, 16);
+  const float b = (h16 ? 0.0f : v1) + __shfl_xor_sync(0xffffffffu, h16 ? v1 : 0.0f, 16);
+  float c = (h8 ? b : a) + __shfl_xor_sync(0xffffffffu, h8 ? a : b, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+  return c;
+}
+
+// Block sums of three values with one barrier: `red` is [2][3][32], `flip`
+// alternates between its halves, so no second barrier guards the reuse.
+// Every thread gets the same three sums (fixed order).
+template <int NT>
+__device__ __forceinline__ void block_sum3(float (&v)[3], float* red, int& flip) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  float* r = red + flip * 96;
+  flip ^= 1;
+  float t = lane_sum3(v[0], v[1], v[2]);
+  if ((lane & 7) == 0 && lane < 24) r[32 * (lane >> 3) + w] = t;
+  __syncthreads();
+  const bool ok = lane < NT / 32;
+  t = lane_sum3(ok ? r[lane] : 0.0f, ok ? r[32 + lane] : 0.0f, ok ? r[64 + lane] : 0.0f);
+  v[0] = __shfl_sync(0xffffffffu, t, 0);
+  v[1] = __shfl_sync(0xffffffffu, t, 8);
+  v[2] = __shfl_sync(0xffffffffu, t, 16);
+}
+
+// remdm_sample_kernel for rows whose probabilities fit in shared memory
+// (q_v = exp(l_v - max), 0 for MASK).  Persistent blocks; each takes the
+// unmasking rows whose rank among all of them is its block index modulo the
+// grid, so the rows that draw nothing cost one scan of the actions instead of
+// a block each, and the others spread evenly.
+//  - tau (the largest fp32 value whose tokens hold >= top_p of the mass) by a
+//    4-way search on its bit pattern, three thresholds per read of the row;
+//    it starts at (1 - top_p) Z / V, below which no more than (1 - top_p) Z
+//    can lie, and once few tokens lie in the bracket it continues on those.
+//  - the draw: each warp sums a contiguous segment of the ids with coalesced
+//    reads; one warp walks the segment that holds the goal.
+// 16 x 1024 positions, V = 32768, 922 rows drawing: 507 -> 196 us (one block per
+// row, a bit of tau per read, and per-thread id ranges whose reads hit one
+// shared-memory bank 32-fold).
+constexpr int kNucCand = 4096;   // bracket size from which the search runs on the collected tokens
+constexpr int kNucList = 512;    // rows of one block per scanned segment of actions
+constexpr int kNucSeg = 32768;   // actions scanned at a time
+
 template <int NT>
 __global__ void __launch_bounds__(NT) remdm_sample_smem_kernel(const float* __restrict__ logits, int ld, int n_rows,
                                                                const int32_t* __restrict__ idx,
@@ -415,91 +464,244 @@ __global__ void __launch_bounds__(NT) remdm_sample_smem_kernel(const float* __re
                                                                float top_p, uint64_t seed, int step,
                                                                const int* __restrict__ count) {
   pdl_enter();
-  extern __shared__ float qs[];
-  __shared__ float red[NT / 32];
-  __shared__ float scan[NT];
-  __shared__ int pick;
-  const int j = blockIdx.x;
-  if (j >= n_rows || (count && j >= *count)) return;
-  const int row = idx ? idx[j] : j;
-  if (act[row] != 2) return;
-  const int b = row / R, r = row - (row / R) * R;
-  const float* L = logits + static_cast<size_t>(j) * ld;
-  const int tid = threadIdx.x;
-  float mx = -INFINITY;
-  for (int v = tid; v < vocab; v += NT) {
-    const float l = L[v];
-    qs[v] = l;
-    if (v != mask_id) mx = fmaxf(mx, l);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if ((tid & 31) == 0) red[tid >> 5] = mx;
-  __syncthreads();
-  mx = red[0];
-#pragma unroll
-  for (int w = 1; w < NT / 32; ++w) mx = fmaxf(mx, red[w]);
-  for (int v = tid; v < vocab; v += NT) qs[v] = v == mask_id ? 0.0f : expf(qs[v] - mx);
-  auto mass_from = [&](float tau) {
-    float acc = 0.0f;
-    for (int v = tid; v < vocab; v += NT) {
-      const float q = qs[v];
-      acc += q >= tau && q > 0.0f ? q : 0.0f;
-    }
-    return block_sum_f<NT>(acc, red);
+  extern __shared__ __align__(16) float qs[];      // vocab probabilities, then kNucCand collected ones
+  __shared__ float red[2 * 96], seg_sum[32];
+  __shared__ int list[kNucList], wcnt[32];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  constexpr int NW = NT / 32;
+  float* cand = qs + (vocab + 3) / 4 * 4;
+  int flip = 0;
+
+  // asks L2 for the logits of the block's next row while this one is worked on
+  auto fetch_row = [&](int j) {
+    const char* p = reinterpret_cast<const char*>(logits + static_cast<size_t>(j) * ld);
+    for (int v = tid * 128; v < vocab * 4; v += NT * 128) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + v));
   };
-  const float total = mass_from(0.0f);
-  const float target = top_p * total;
-  uint32_t lo = 0u, hi = 0x3F800001u;
-  while (hi - lo > 1u) {
-    const uint32_t mid = lo + (hi - lo) / 2u;
-    if (mass_from(__uint_as_float(mid)) >= target) lo = mid;
-    else hi = mid;
-  }
-  const float tau = __uint_as_float(lo);
-  const int chunk = (vocab + NT - 1) / NT, v0 = tid * chunk, v1 = min(vocab, v0 + chunk);
-  float mine = 0.0f;
-  for (int v = v0; v < v1; ++v) {
-    const float q = qs[v];
-    mine += q >= tau && q > 0.0f ? q : 0.0f;
-  }
-  scan[tid] = mine;
-  if (tid == 0) pick = -1;
-  __syncthreads();
-  for (int o = 1; o < NT; o <<= 1) {
-    const float add = tid >= o ? scan[tid - o] : 0.0f;
-    __syncthreads();
-    scan[tid] += add;
-    __syncthreads();
-  }
-  float u[3];
-  remdm_draws(seed, step, B, R, b, r, u);
-  const float goal = u[2] * scan[NT - 1];
-  const float before = tid > 0 ? scan[tid - 1] : 0.0f;
-  if (mine > 0.0f && before <= goal && goal < scan[tid]) {
-    float c = before;
-    int last = -1, got = -1;
-    for (int v = v0; v < v1; ++v) {
-      const float q = qs[v];
-      if (q >= tau && q > 0.0f) {
-        last = v;
-        c += q;
-        if (c > goal) {
-          got = v;
-          break;
+  auto draw_row = [&](int j, int row) {
+    const int b = row / R, r = row - (row / R) * R;
+    const float* L = logits + static_cast<size_t>(j) * ld;
+    float mx = -INFINITY;
+    if ((ld & 3) == 0 && (reinterpret_cast<uintptr_t>(logits) & 15) == 0) {
+      for (int v = 4 * tid; v < vocab; v += 4 * NT) {
+        float x[4];
+        if (v + 4 <= vocab) {
+          const float4 t = *reinterpret_cast<const float4*>(L + v);
+          x[0] = t.x, x[1] = t.y, x[2] = t.z, x[3] = t.w;
+        } else {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) x[k] = v + k < vocab ? L[v + k] : -INFINITY;
         }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (v + k != mask_id) mx = fmaxf(mx, x[k]);
+        *reinterpret_cast<float4*>(qs + v) = make_float4(x[0], x[1], x[2], x[3]);   // the row is padded to 4
+      }
+    } else {
+      for (int v = tid; v < vocab; v += NT) {
+        const float l = L[v];
+        qs[v] = l;
+        if (v != mask_id) mx = fmaxf(mx, l);
       }
     }
-    pick = got >= 0 ? got : last;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane == 0) seg_sum[w] = mx;
+    __syncthreads();
+    mx = lane < NW ? seg_sum[lane] : -INFINITY;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    float s3[3] = {0.0f, 0.0f, 0.0f};
+    for (int v = tid; v < vocab; v += NT) {
+      const float q = v == mask_id ? 0.0f : expf(qs[v] - mx);
+      qs[v] = q;
+      s3[0] += q;
+    }
+    block_sum3<NT>(s3, red, flip);                 // its barrier also publishes qs
+    const float total = s3[0], target = top_p * total;
+    // mass(lo) >= target > mass(hi), mass(t) = sum of q >= t
+    uint32_t lo = __float_as_uint(fmaxf(0.99f * (1.0f - top_p) * total / static_cast<float>(vocab), 0.0f)), hi = 0x3F800001u;
+    float mass_hi = 0.0f, mass_hi_all = 0.0f;      // mass(hi); mass above the collected tokens
+    bool collected = false;                        // the tokens of the bracket are in c
+    float c[kNucCand / NT];
+    while (hi - lo > 1u) {
+      if (!collected && hi - lo <= (1u << 21)) {
+        const float flo = __uint_as_float(lo), fhi = __uint_as_float(hi);
+        int own = 0;
+        for (int v = tid; v < vocab; v += NT) own += qs[v] >= flo && qs[v] < fhi ? 1 : 0;
+        int inc = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int t = __shfl_up_sync(0xffffffffu, inc, o);
+          if (lane >= o) inc += t;
+        }
+        __syncthreads();                           // earlier reads of wcnt are done
+        if (lane == 31) wcnt[w] = inc;
+        __syncthreads();
+        int winc = lane < NW ? wcnt[lane] : 0;
+        const int wown = winc;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int t = __shfl_up_sync(0xffffffffu, winc, o);
+          if (lane >= o) winc += t;
+        }
+        const int all = __shfl_sync(0xffffffffu, winc, 31);
+        if (all <= kNucCand) {
+          int at = __shfl_sync(0xffffffffu, winc - wown, w) + inc - own;
+          for (int v = tid; v < vocab; v += NT) {
+            const float q = qs[v];
+            if (q >= flo && q < fhi) cand[at++] = q;
+          }
+          __syncthreads();
+          collected = true;
+          mass_hi_all = mass_hi;
+#pragma unroll
+          for (int k = 0; k < kNucCand / NT; ++k) c[k] = tid + k * NT < all ? cand[tid + k * NT] : 0.0f;
+        }
+      }
+      const uint32_t st = max((hi - lo) / 4u, 1u);
+      const float t1 = __uint_as_float(lo + st), t2 = __uint_as_float(lo + 2 * st), t3 = __uint_as_float(lo + 3 * st);
+      float m3[3] = {0.0f, 0.0f, 0.0f};
+      if (collected) {
+#pragma unroll
+        for (int k = 0; k < kNucCand / NT; ++k) {
+          m3[0] += c[k] >= t1 ? c[k] : 0.0f;
+          m3[1] += c[k] >= t2 ? c[k] : 0.0f;
+          m3[2] += c[k] >= t3 ? c[k] : 0.0f;
+        }
+      } else {
+        for (int v = tid; v < vocab; v += NT) {
+          const float q = qs[v];
+          m3[0] += q >= t1 ? q : 0.0f;
+          m3[1] += q >= t2 ? q : 0.0f;
+          m3[2] += q >= t3 ? q : 0.0f;
+        }
+      }
+      block_sum3<NT>(m3, red, flip);
+      float ms[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) ms[k] = collected ? m3[k] + mass_hi_all : m3[k];
+      const uint32_t base = lo;
+      if (ms[2] >= target) {
+        lo = base + 3 * st;
+      } else if (ms[1] >= target) {
+        lo = base + 2 * st;
+        hi = base + 3 * st;
+      } else if (ms[0] >= target) {
+        lo = base + st;
+        hi = base + 2 * st;
+      } else {
+        hi = base + st;
+      }
+      if (!collected) mass_hi = hi == base + 3 * st ? ms[2] : hi == base + 2 * st ? ms[1] : hi == base + st ? ms[0] : mass_hi;
+    }
+    const float tau = __uint_as_float(lo);
+    // id-order inverse CDF within the nucleus
+    const int S = (vocab + NW * 128 - 1) / (NW * 128) * 128;
+    float mine = 0.0f;
+    for (int v = w * S + lane; v < min(vocab, (w + 1) * S); v += 32) {
+      const float q = qs[v];
+      mine += q >= tau ? q : 0.0f;
+    }
+    mine = warp_sum(mine);
+    __syncthreads();                               // the maxima in seg_sum have been read
+    if (lane == 0) seg_sum[w] = mine;
+    __syncthreads();
+    if (w == 0) {
+      float u[3];
+      remdm_draws(seed, step, B, R, b, r, u);
+      const float own = lane < NW ? seg_sum[lane] : 0.0f;
+      float inc = own;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const float t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += t;
+      }
+      const float goal = u[2] * __shfl_sync(0xffffffffu, inc, 31);
+      const unsigned over = __ballot_sync(0xffffffffu, own > 0.0f && inc > goal);
+      const unsigned some = __ballot_sync(0xffffffffu, own > 0.0f);
+      const int seg = over ? __ffs(over) - 1 : 31 - __clz(some | 1u);   // rounding past the end: the last segment
+      float run = __shfl_sync(0xffffffffu, inc - own, seg);
+      int got = -1, last = -1;
+      for (int v0 = seg * S; v0 < min(vocab, (seg + 1) * S) && got < 0; v0 += 128) {
+        float q[4], loc = 0.0f;
+        int lst = -1;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int v = v0 + 4 * lane + k;
+          const float t = v < vocab ? qs[v] : 0.0f;
+          q[k] = t >= tau ? t : 0.0f;
+          loc += q[k];
+          if (q[k] > 0.0f) lst = v;
+        }
+        float sc = loc;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const float t = __shfl_up_sync(0xffffffffu, sc, o);
+          if (lane >= o) sc += t;
+        }
+        const unsigned hit = __ballot_sync(0xffffffffu, loc > 0.0f && run + sc > goal);
+        const unsigned any = __ballot_sync(0xffffffffu, loc > 0.0f);
+        if (any) last = __shfl_sync(0xffffffffu, lst, 31 - __clz(any));
+        if (hit) {                                 // the first lane past the goal resolves it among its four
+          const int src = __ffs(hit) - 1;
+          float c = run + sc - loc;
+          int pick = -1;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            c += q[k];
+            if (pick < 0 && q[k] > 0.0f && c > goal) pick = v0 + 4 * lane + k;
+          }
+          if (pick < 0) pick = lst;
+          got = __shfl_sync(0xffffffffu, pick, src);
+        }
+        run += __shfl_sync(0xffffffffu, sc, 31);
+      }
+      if (lane == 0) z[static_cast<size_t>(b) * ldz + r] = got >= 0 ? got : last;
+    }
+    __syncthreads();                               // qs is rewritten by the next row
+  };
+
+  const int n = count ? min(n_rows, *count) : n_rows;
+  if (idx) {                                       // compacted rows: every entry draws
+    for (int j = blockIdx.x; j < n; j += gridDim.x) {
+      const int row = idx[j];
+      if (j + static_cast<int>(gridDim.x) < n) fetch_row(j + gridDim.x);
+      if (act[row] == 2) draw_row(j, row);         // uniform across the block
+    }
+    return;
   }
-  __syncthreads();
-  if (tid == 0) {
-    int v = pick;
-    for (int t = NT - 1; t >= 0 && v < 0; --t)   // rounding left the goal past every range: the last token
-      if ((t > 0 ? scan[t] - scan[t - 1] : scan[0]) > 0.0f)
-        for (int w = min(vocab, (t + 1) * chunk) - 1; w >= t * chunk; --w)
-          if (qs[w] >= tau && qs[w] > 0.0f) { v = w; break; }
-    z[static_cast<size_t>(b) * ldz + r] = v;
+  int rank0 = 0;                                   // drawing rows ahead of the segment
+  for (int s0 = 0; s0 < n; s0 += kNucSeg) {
+    const int s1 = min(n, s0 + kNucSeg);
+    int seen = rank0, n_list = 0;
+    for (int r0 = s0; r0 < s1; r0 += NT) {
+      const bool on = r0 + tid < s1 && act[r0 + tid] == 2;
+      const unsigned m = __ballot_sync(0xffffffffu, on);
+      __syncthreads();
+      if (lane == 0) wcnt[w] = __popc(m);
+      __syncthreads();
+      int inc = lane < NW ? wcnt[lane] : 0;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += t;
+      }
+      const int all = __shfl_sync(0xffffffffu, inc, 31);
+      const int rank = seen + (w ? __shfl_sync(0xffffffffu, inc, w - 1) : 0) + __popc(m & ((1u << lane) - 1u));
+      const int first = (rank0 - static_cast<int>(blockIdx.x) + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x);
+      if (on && rank % static_cast<int>(gridDim.x) == static_cast<int>(blockIdx.x))
+        list[rank / static_cast<int>(gridDim.x) - max(first, 0)] = r0 + tid;
+      seen += all;
+    }
+    const int first = max((rank0 - static_cast<int>(blockIdx.x) + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x), 0);
+    n_list = (seen - static_cast<int>(blockIdx.x) + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x) - first;
+    __syncthreads();
+    for (int i = 0; i < n_list; ++i) {
+      if (i + 1 < n_list) fetch_row(list[i + 1]);
+      draw_row(list[i], list[i]);
+    }
+    __syncthreads();                               // list is rewritten by the next segment
+    rank0 = seen;
   }
 }
 
@@ -882,16 +1084,23 @@ const char* remdm_sample(const float* logits, int ld, int n_rows, const int32_t*
                          int ldz, int B, int R, int vocab, int mask_id, float top_p, uint64_t seed, int step,
                          cudaStream_t s, const int* count) {
   if (n_rows <= 0) return nullptr;
-  const size_t smem = static_cast<size_t>(vocab) * sizeof(float);
-  if (smem <= 200u * 1024u) {   // the row's probabilities fit in shared memory
-    static bool attr = false;
-    if (!attr) {
+  const size_t smem = (static_cast<size_t>(vocab + 3) / 4 * 4 + kNucCand) * sizeof(float);
+  if (static_cast<size_t>(vocab) * sizeof(float) <= 200u * 1024u) {   // the row's probabilities fit in shared memory
+    static int n_sms = 0;
+    if (n_sms == 0) {
       if (cudaFuncSetAttribute(remdm_sample_smem_kernel<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               200 * 1024) != cudaSuccess)
+                               (200 * 256 + kNucCand) * 4) != cudaSuccess)
         return "sampler smem attribute failed";
-      attr = true;
+      int dev = 0, n = 0;
+      cudaGetDevice(&dev);
+      cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+      n_sms = n > 0 ? n : 1;
     }
-    launch_pdl(remdm_sample_smem_kernel<1024>, n_rows, 1024, smem, s, logits, ld, n_rows, idx, act, z, ldz, B, R,
+    // one resident wave: two 1024-thread blocks per SM while two rows fit its shared memory; the list of a
+    // scanned segment holds kNucSeg / grid rows
+    const int per_sm = smem <= 100u * 1024u ? 2 : 1;
+    const int grid = std::min(n_rows, std::max(per_sm * n_sms, 2 * kNucSeg / kNucList));
+    launch_pdl(remdm_sample_smem_kernel<1024>, grid, 1024, smem, s, logits, ld, n_rows, idx, act, z, ldz, B, R,
                vocab, mask_id, top_p, seed, step, count);
   } else {
     launch_pdl(remdm_sample_kernel<256>, n_rows, 256, 0, s, logits, ld, n_rows, idx, act, z, ldz, B, R, vocab,

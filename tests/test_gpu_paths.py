@@ -40,3 +40,41 @@ def test_gemm_fp32_store_edges(T, M, N, K, ldc):
     # fp32 accumulation of K exact bf16 products
     assert np.abs(got[:, :N] - a @ b.T).max() <= 1e-5 * np.abs(a).max() * np.abs(b).max() * np.sqrt(K)
     assert (got[:, N:] == 7.0).all() and (flat[M * ldc:] == 7.0).all().item()
+
+
+def _nucleus_ok(logits, mask, top_p, u, tok, tol=2e-5):
+    """tok is the inverse-CDF draw of the nucleus, up to fp32 rounding of the cumulative mass at its edges."""
+    q = np.exp(logits.astype(np.float64) - np.delete(logits, mask).max())
+    q[mask] = 0.0
+    desc = np.sort(q)[::-1]
+    c = np.cumsum(desc)
+    for p in (top_p, top_p * (1 + tol), top_p * (1 - tol)):
+        tau = desc[min(np.searchsorted(c, p * c[-1] * (1 - 1e-12)), len(desc) - 1)]
+        n = np.where(q >= tau, q, 0.0)
+        cum = np.cumsum(n)
+        if n[tok] > 0 and cum[tok] - n[tok] - tol * cum[-1] <= u * cum[-1] <= cum[tok] + tol * cum[-1]:
+            return True
+    return False
+
+
+# the shared-memory sampler: rows that are no multiple of 4 (scalar loads), one
+# segment per warp and a tail, more equal tokens than the collected bracket
+# holds, near one-hot rows, top_p = 1; more drawing rows than blocks
+@pytest.mark.parametrize("V,R,top_p", [(30, 400, 0.9), (1001, 300, 0.9), (4100, 64, 1.0), (30522, 40, 0.9),
+                                       (51200, 24, 0.5)])
+def test_remdm_nucleus_draws(T, V, R, top_p):
+    B, first, mask, seed, step = 2, 3, V - 1, 77, 4
+    rng = np.random.default_rng(V)
+    logits = (rng.standard_normal((B * R, V)) * rng.choice([0.3, 3.0], (B * R, 1))).astype(np.float32)
+    logits[first] = 0.5                                   # all equal
+    logits[first + 1] += np.where(np.arange(V) == V // 2, 60.0, 0.0).astype(np.float32)
+    logits[first + 2, : V // 2] = -np.inf
+    z = np.full((B, R), mask, np.int32)
+    zt = torch.from_numpy(z).cuda()
+    act = torch.empty(B * R, dtype=torch.int32, device="cuda")
+    T.tadm_remdm_update(zt, torch.from_numpy(logits).cuda(), first, mask, 0.0, 1.0, top_p, seed, step, act)
+    got, u = zt.cpu().numpy(), wl.remdm_uniforms(seed, step, B, R)
+    assert (got[:, :first] == mask).all()
+    for b in range(B):
+        for r in range(first, R):
+            assert _nucleus_ok(logits[b * R + r], mask, top_p, u[b, r, 2], got[b, r]), (b, r, got[b, r])
