@@ -20,7 +20,7 @@
 //   key tiles, rescaled only when a row's running max grows by more than 2^8.
 // bf16, short rows (attn_bf16_kernel): mma.sync m16n8k16 flash attention;
 //   a CTA takes 64 rows of all query heads of one KV group (one K/V read).
-// fp32: one warp per query row on the CUDA cores.
+// fp32: shared-memory tiles on the CUDA cores, 16 query rows per block.
 #include <cudaTypedefs.h>
 #include <algorithm>
 #include <cstdlib>
@@ -1104,44 +1104,144 @@ __global__ void __launch_bounds__(128) attn_bf16_kernel(const bf16* __restrict__
   }
 }
 
-// fp32: one warp per (query row, head, batch); each lane owns hd/32 dims.
+// fp32 on the CUDA cores: one 128-thread block per 16 query rows of one head.
+// Key tiles of 64 go through shared memory (K rows and V^T rows, both
+// contiguous in the dimension their product runs over); thread (ty, tx) owns
+// rows ty and ty + 8 and keys (then dims) tx + 16 j, so every float4 read
+// feeds four FMAs per partner row.  The online softmax runs once per tile.
+// 4 x 4 heads x 128 rows, hd 64: 93 -> 15.7 us (one warp per query row, a warp
+// reduction and two uncoalesced V reads per key).
+constexpr int FQ = 16, FK = 64, FNT = 128;
+
 template <int HD>
-__global__ void __launch_bounds__(128) attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k,
+struct F32Cfg { static constexpr int FLOATS = FQ * (HD + 4) + FK * (HD + 4) + HD * (FK + 4) + FQ * (FK + 4); };
+
+template <int HD>
+__global__ void __launch_bounds__(FNT) attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k,
                                                        const float* __restrict__ vt, float* __restrict__ o,
                                                        int n_heads, int n_kv_heads, int rows, int ctx,
-                                                       int kv_stride, int causal, int window, float scale) {
+                                                       int kv_stride, int causal, int window, float scale, int vec) {
   pdl_enter();
-  constexpr int PL = HD / 32;
-  const int lane = threadIdx.x & 31;
-  const int row = blockIdx.x * 4 + (threadIdx.x >> 5);
-  const int h = blockIdx.y, b = blockIdx.z;
-  if (row >= rows) return;
+  constexpr int LD = HD + 4, LDP = FK + 4, ND = HD / 16;   // ND: output dims per thread and row
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  float* sQ = reinterpret_cast<float*>(smem_raw);          // [FQ][LD]
+  float* sK = sQ + FQ * LD;                                // [FK][LD]
+  float* sV = sK + FK * LD;                                // [HD][LDP]
+  float* sP = sV + HD * LDP;                               // [FQ][LDP]
+  const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16;
+  const int r0 = blockIdx.x * FQ, h = blockIdx.y, b = blockIdx.z;
   const int hk = h / (n_heads / n_kv_heads);
-  const float* qr = q + ((static_cast<size_t>(b) * n_heads + h) * rows + row) * HD;
+  const float* qb = q + ((static_cast<size_t>(b) * n_heads + h) * rows + r0) * HD;
   const float* kb = k + (static_cast<size_t>(b) * n_kv_heads + hk) * kv_stride * HD;
   const float* vb = vt + (static_cast<size_t>(b) * n_kv_heads + hk) * HD * kv_stride;
-  float qv[PL], acc[PL];
+  const int nr = min(FQ, rows - r0);
+  for (int i = tid; i < FQ * HD; i += FNT) sQ[(i / HD) * LD + i % HD] = i / HD < nr ? qb[i] : 0.0f;
+  // keys that any row of the block may see
+  const int end = causal ? ctx + r0 + nr : ctx + rows;
+  const int begin = window > 0 ? max(0, ctx + r0 - window + 1) : 0;
+  float acc[2][ND], m[2] = {-INFINITY, -INFINITY}, l[2] = {0.0f, 0.0f};
 #pragma unroll
-  for (int i = 0; i < PL; ++i) { qv[i] = qr[lane + 32 * i]; acc[i] = 0.0f; }
-  const int qpos = ctx + row;
-  const int kv_end = causal ? qpos + 1 : ctx + rows;
-  const int kv_lo = window > 0 ? max(0, qpos - window + 1) : 0;   // sliding window start
-  float m = -INFINITY, l = 0.0f;
-  for (int j = kv_lo; j < kv_end; ++j) {
-    float d = 0.0f;
+  for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int i = 0; i < PL; ++i) d += qv[i] * kb[static_cast<size_t>(j) * HD + lane + 32 * i];
-    d = warp_sum(d) * scale;
-    const float mn = fmaxf(m, d);
-    const float c = expf(m - mn), p = expf(d - mn);
-    l = l * c + p;
+    for (int j = 0; j < ND; ++j) acc[i][j] = 0.0f;
+  for (int k0 = begin / FK * FK; k0 < end; k0 += FK) {
+    __syncthreads();                                       // the previous tile has been read
+    if (vec) {
+      for (int i = tid; i < FK * (HD / 4); i += FNT) {
+        const int r = i / (HD / 4), c = i % (HD / 4) * 4;
+        const float4 x = k0 + r < end ? *reinterpret_cast<const float4*>(kb + static_cast<size_t>(k0 + r) * HD + c)
+                                      : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        *reinterpret_cast<float4*>(sK + r * LD + c) = x;
+      }
+      for (int i = tid; i < HD * (FK / 4); i += FNT) {
+        const int r = i / (FK / 4), c = i % (FK / 4) * 4;
+        const float* p = vb + static_cast<size_t>(r) * kv_stride + k0 + c;
+        float4 x = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (k0 + c + 4 <= end) {
+          x = *reinterpret_cast<const float4*>(p);
+        } else {
+          if (k0 + c < end) x.x = p[0];
+          if (k0 + c + 1 < end) x.y = p[1];
+          if (k0 + c + 2 < end) x.z = p[2];
+        }
+        *reinterpret_cast<float4*>(sV + r * LDP + c) = x;
+      }
+    } else {
+      for (int i = tid; i < FK * HD; i += FNT)
+        sK[(i / HD) * LD + i % HD] = k0 + i / HD < end ? kb[static_cast<size_t>(k0) * HD + i] : 0.0f;
+      for (int i = tid; i < HD * FK; i += FNT)
+        sV[(i / FK) * LDP + i % FK] = k0 + i % FK < end ? vb[static_cast<size_t>(i / FK) * kv_stride + k0 + i % FK] : 0.0f;
+    }
+    __syncthreads();
+    float s[2][4];
 #pragma unroll
-    for (int i = 0; i < PL; ++i) acc[i] = acc[i] * c + p * vb[static_cast<size_t>(lane + 32 * i) * kv_stride + j];
-    m = mn;
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) s[i][j] = 0.0f;
+#pragma unroll 4
+    for (int d = 0; d < HD; d += 4) {
+      float4 a[2], c[4];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) a[i] = *reinterpret_cast<const float4*>(sQ + (ty + 8 * i) * LD + d);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) c[j] = *reinterpret_cast<const float4*>(sK + (tx + 16 * j) * LD + d);
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          s[i][j] = fmaf(a[i].w, c[j].w, fmaf(a[i].z, c[j].z, fmaf(a[i].y, c[j].y, fmaf(a[i].x, c[j].x, s[i][j]))));
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int qpos = ctx + r0 + ty + 8 * i;
+      const int hi = causal ? min(end, qpos + 1) : end, lo = window > 0 ? qpos - window + 1 : 0;
+      float mx = m[i];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int key = k0 + tx + 16 * j;
+        s[i][j] = key < hi && key >= lo ? s[i][j] * scale : -INFINITY;
+        mx = fmaxf(mx, s[i][j]);
+      }
+#pragma unroll
+      for (int w = 8; w > 0; w >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, w));
+      const float f = mx == -INFINITY ? 1.0f : expf(m[i] - mx);   // nothing seen yet: nothing to rescale
+      float ps = 0.0f;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float p = s[i][j] == -INFINITY ? 0.0f : expf(s[i][j] - mx);
+        sP[(ty + 8 * i) * LDP + tx + 16 * j] = p;
+        ps += p;
+      }
+#pragma unroll
+      for (int w = 8; w > 0; w >>= 1) ps += __shfl_xor_sync(0xffffffffu, ps, w);
+      l[i] = l[i] * f + ps;
+      m[i] = mx;
+#pragma unroll
+      for (int j = 0; j < ND; ++j) acc[i][j] *= f;
+    }
+    __syncwarp();                                          // a row's probabilities are written and read by one warp
+#pragma unroll 4
+    for (int c = 0; c < FK; c += 4) {
+      float4 p[2];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) p[i] = *reinterpret_cast<const float4*>(sP + (ty + 8 * i) * LDP + c);
+#pragma unroll
+      for (int j = 0; j < ND; ++j) {
+        const float4 v = *reinterpret_cast<const float4*>(sV + (tx + 16 * j) * LDP + c);
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+          acc[i][j] = fmaf(p[i].w, v.w, fmaf(p[i].z, v.z, fmaf(p[i].y, v.y, fmaf(p[i].x, v.x, acc[i][j]))));
+      }
+    }
   }
-  float* orow = o + (static_cast<size_t>(b) * rows + row) * n_heads * HD + static_cast<size_t>(h) * HD;
 #pragma unroll
-  for (int i = 0; i < PL; ++i) orow[lane + 32 * i] = acc[i] / l;
+  for (int i = 0; i < 2; ++i) {
+    const int r = r0 + ty + 8 * i;
+    if (r >= rows) continue;
+    float* orow = o + (static_cast<size_t>(b) * rows + r) * n_heads * HD + static_cast<size_t>(h) * HD;
+#pragma unroll
+    for (int j = 0; j < ND; ++j) orow[tx + 16 * j] = acc[i][j] / l[i];
+  }
 }
 
 template <int HD>
@@ -1167,11 +1267,18 @@ cudaError_t launch_bf16(const AttnCall& a, cudaStream_t s) {
 
 template <int HD>
 cudaError_t launch_f32(const AttnCall& a, cudaStream_t s) {
-  dim3 grid((a.rows + 3) / 4, a.n_heads, a.batch);
-  launch_pdl(attn_f32_kernel<HD>, grid, 128, 0, s, static_cast<const float*>(a.q), static_cast<const float*>(a.k),
-                                           static_cast<const float*>(a.v), static_cast<float*>(a.o), a.n_heads,
-                                           a.n_kv_heads, a.rows, a.ctx, a.kv_stride, a.causal, a.window,
-                                           1.0f / sqrtf(static_cast<float>(HD)));
+  constexpr int smem = F32Cfg<HD>::FLOATS * 4;
+  static bool attr = false;
+  if (!attr) {
+    const cudaError_t e = cudaFuncSetAttribute(attn_f32_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    attr = true;
+  }
+  dim3 grid((a.rows + FQ - 1) / FQ, a.n_heads, a.batch);
+  const int vec = a.kv_stride % 4 == 0 && ((reinterpret_cast<uintptr_t>(a.k) | reinterpret_cast<uintptr_t>(a.v)) & 15) == 0;
+  launch_pdl(attn_f32_kernel<HD>, grid, FNT, smem, s, static_cast<const float*>(a.q), static_cast<const float*>(a.k),
+             static_cast<const float*>(a.v), static_cast<float*>(a.o), a.n_heads, a.n_kv_heads, a.rows, a.ctx, a.kv_stride,
+             a.causal, a.window, 1.0f / sqrtf(static_cast<float>(HD)), vec);
   return cudaGetLastError();
 }
 }  // namespace

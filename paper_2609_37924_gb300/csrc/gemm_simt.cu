@@ -1,13 +1,26 @@
 // fp32 GEMM on the CUDA cores, used by fp32 models (the tiny workload):
 // acc[M, N] = A[M, K] * B[N, K]^T with the same fused epilogues as the tensor
-// core path.  64 x 64 output tile per 256-thread block, 4 x 4 per thread,
-// K staged through shared memory 16 at a time.  EPI_GLU tiles hold 32 gate
-// and 32 up columns; EPI_QKV needs head_dim <= 64.
+// core path.
+//
+// One 256-thread block per TM x 64 output tile (TM = 32, or 16 when 32-row
+// tiles would leave SMs idle).  The GEMMs of this path are a few hundred rows
+// by a few hundred columns, so a launch is paced by the latency of one
+// block's K loop, not by FMA throughput: K advances 64 at a time through a
+// three-stage cp.async ring, and the block's four 64-thread groups each take
+// 16 of the 64 columns of every stage (a split of K inside the block); their
+// partial tiles are summed in group order through shared memory.  Weights
+// (b_weights) start loading ahead of the grid dependency.  Rows of the stage
+// are padded to 68 floats: the 8 column (4 row) addresses of a warp's float4
+// reads fall into different banks.
+// 512 rows: the residual projections (N 256, K 256 and 1024) 95 -> 15.6 us a
+// launch, QKV (N 768, K 256) 36 -> 14.8 us, cold caches (before: 64 x 64
+// tiles, 16 columns of K per synchronous step, 32 to 96 blocks).
+// EPI_GLU tiles hold 32 gate and 32 up columns; EPI_QKV needs head_dim <= 64.
 #include "kernels.h"
 
 namespace tadm {
 namespace {
-constexpr int TM = 64, TN = 64, TK = 16;
+constexpr int TN = 64, TK = 64, LDK = TK + 4, STAGES = 3, GROUPS = 4, NT = 64 * GROUPS;
 
 struct SmemSrc {
   static constexpr bool kStaged = false;
@@ -20,58 +33,165 @@ struct SmemSrc {
   }
 };
 
-template <int EPI>
-__global__ void __launch_bounds__(256) gemm_simt_kernel(const float* __restrict__ A, const float* __restrict__ B,
-                                                        int M, int K, int lda, int ldb, int n_rows_b,
-                                                        int b_split, EpiParams ep) {
-  pdl_enter();
-  __shared__ float sA[TK][TM + 4];
-  __shared__ float sB[TK][TN + 4];
-  __shared__ float sC[TM][TN + 1];
-  const int tid = threadIdx.x;
-  const int tx = tid % 16, ty = tid / 16;
-  const int m0 = blockIdx.y * TM, nb = blockIdx.x;
-  float acc[4][4] = {};
-  for (int k0 = 0; k0 < K; k0 += TK) {
-    for (int i = tid; i < TM * TK; i += 256) {
-      const int r = i / TK, c = i % TK;
-      const int gm = m0 + r, gk = k0 + c;
-      sA[c][r] = (gm < M && gk < K) ? A[static_cast<size_t>(gm) * lda + gk] : 0.0f;
+__device__ __forceinline__ void cp_async(float* dst, const float* src, int bytes, bool ok, bool wide) {
+  const int n = ok ? bytes : 0;   // 0: the destination is zero-filled
+  if (wide) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(n) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(n) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+template <int TM>
+struct SimtCfg { static constexpr int FLOATS = STAGES * (TM + TN) * LDK; };
+
+// VEC: rows of A and B are 16-byte aligned and K % 4 == 0 (16-byte copies); otherwise 4-byte copies.
+template <int EPI, int TM, bool VEC>
+__global__ void __launch_bounds__(NT) gemm_simt_kernel(const float* __restrict__ A, const float* __restrict__ B, int M,
+                                                       int K, int lda, int ldb, int tiles_n, int n_rows_b, int b_split,
+                                                       int b_early, EpiParams ep) {
+  extern __shared__ __align__(16) float smem[];
+  const int tid = threadIdx.x, m0 = blockIdx.x / tiles_n * TM, nb = blockIdx.x % tiles_n;
+  const int ksteps = (K + TK - 1) / TK;
+  constexpr int W = VEC ? 4 : 1, CPR = TK / W;      // copies per row of a stage
+  float* sA = smem;                                 // [STAGES][TM][LDK]
+  float* sB = smem + STAGES * TM * LDK;             // [STAGES][TN][LDK]
+  auto load_a = [&](int ks) {
+    float* dst = sA + (ks % STAGES) * TM * LDK;
+    for (int i = tid; i < TM * CPR; i += NT) {
+      const int r = i / CPR, c = (i % CPR) * W, gk = ks * TK + c;
+      const bool ok = m0 + r < M && gk < K;
+      cp_async(dst + r * LDK + c, ok ? A + static_cast<size_t>(m0 + r) * lda + gk : A, 4 * W, ok, VEC);
+    }
+  };
+  auto load_b = [&](int ks) {
+    float* dst = sB + (ks % STAGES) * TN * LDK;
+    for (int i = tid; i < TN * CPR; i += NT) {
+      const int r = i / CPR, c = (i % CPR) * W, gk = ks * TK + c;
       int gn;
-      if (b_split > 0) gn = (r < TN / 2) ? nb * (TN / 2) + r : b_split + nb * (TN / 2) + (r - TN / 2);
+      if (b_split > 0) gn = r < TN / 2 ? nb * (TN / 2) + r : b_split + nb * (TN / 2) + (r - TN / 2);
       else gn = nb * TN + r;
-      sB[c][r] = (gn < n_rows_b && gk < K) ? B[static_cast<size_t>(gn) * ldb + gk] : 0.0f;
+      const bool ok = gn < n_rows_b && gk < K;
+      cp_async(dst + r * LDK + c, ok ? B + static_cast<size_t>(gn) * ldb + gk : B, 4 * W, ok, VEC);
     }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < TK; ++kk) {
-      float a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) { a[i] = sA[kk][ty * 4 + i]; b[i] = sB[kk][tx * 4 + i]; }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
+  };
+  if (b_early) {
+    for (int s = 0; s < STAGES - 1 && s < ksteps; ++s) load_b(s);
   }
+  pdl_enter();
+  for (int s = 0; s < STAGES - 1; ++s) {
+    if (s < ksteps) {
+      if (!b_early) load_b(s);
+      load_a(s);
+    }
+    cp_commit();
+  }
+  // group g owns columns 16 g .. 16 g + 15 of every stage; within it thread
+  // (ty, tx) owns rows ty + 8 i and columns tx + 8 j of the tile
+  constexpr int RM = TM / 8;
+  const int g = tid / 64, t = tid % 64, ty = t / 8, tx = t % 8;
+  float acc[RM][8];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < RM; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) sC[ty * 4 + i][tx * 4 + j] = acc[i][j];
+    for (int j = 0; j < 8; ++j) acc[i][j] = 0.0f;
+  for (int ks = 0; ks < ksteps; ++ks) {
+    cp_wait<STAGES - 2>();
+    __syncthreads();                                // stage ks has landed; stage ks - 1 has been read by all
+    if (ks + STAGES - 1 < ksteps) {
+      load_b(ks + STAGES - 1);
+      load_a(ks + STAGES - 1);
+    }
+    cp_commit();
+    const float* a0 = sA + (ks % STAGES) * TM * LDK + ty * LDK + 16 * g;
+    const float* b0 = sB + (ks % STAGES) * TN * LDK + tx * LDK + 16 * g;
+#pragma unroll
+    for (int kk = 0; kk < 16; kk += 4) {
+      float4 a[RM], b[8];
+#pragma unroll
+      for (int i = 0; i < RM; ++i) a[i] = *reinterpret_cast<const float4*>(a0 + 8 * i * LDK + kk);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) b[j] = *reinterpret_cast<const float4*>(b0 + 8 * j * LDK + kk);
+#pragma unroll
+      for (int i = 0; i < RM; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
+          acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
+          acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
+          acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
+        }
+    }
+  }
+  // partial tiles of the groups -> their sum in group order, in the first one's place
+  cp_wait<0>();
   __syncthreads();
-  if (tid < TM) {
-    SmemSrc src{&sC[tid][0]};
-    epilogue_row<EPI>(ep, m0 + tid, nb, TN, src);
+  constexpr int LDC = TN + 1, TILE = TM * LDC;
+  static_assert(GROUPS * TILE <= SimtCfg<TM>::FLOATS, "partial tiles fit the stages");
+  float* sC = smem;
+#pragma unroll
+  for (int i = 0; i < RM; ++i)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) sC[g * TILE + (ty + 8 * i) * LDC + tx + 8 * j] = acc[i][j];
+  __syncthreads();
+  for (int e = tid; e < TM * TN; e += NT) {
+    const int o = (e / TN) * LDC + e % TN;
+    float s = sC[o];
+#pragma unroll
+    for (int q = 1; q < GROUPS; ++q) s += sC[q * TILE + o];
+    if constexpr (EPI == EPI_RESID) {               // element-wise, coalesced
+      const int m = m0 + e / TN, n = nb * TN + e % TN;
+      if (m < M && n < ep.N) {
+        float* x = ep.resid + static_cast<size_t>(m) * ep.ldr + n;
+        *x += ep.bias ? s + ld_param(ep.bias, ep.bias_bf16, n) : s;
+      }
+    } else {
+      sC[o] = s;
+    }
   }
+  if constexpr (EPI == EPI_RESID) return;
+  __syncthreads();
+  // the tile's 64 columns of a row go to one thread, or to two where the epilogue's columns are independent
+  constexpr int NS = (EPI == EPI_STORE || EPI == EPI_SILU || EPI == EPI_ADD || EPI == EPI_FUSION1 || EPI == EPI_FUSION2 ||
+                      EPI == EPI_PA_UP) ? 2 : 1;
+  if (tid < TM * NS) {
+    SmemSrc src{sC + (tid % TM) * LDC};
+    epilogue_row<EPI>(ep, m0 + tid % TM, nb, TN, src, tid / TM, NS);
+  }
+}
+
+template <int EPI, int TM, bool VEC>
+cudaError_t launch_tile(const GemmCall& g, int tiles_n, int b_split, int n_rows_b, const EpiParams& ep, cudaStream_t s) {
+  constexpr int smem = SimtCfg<TM>::FLOATS * 4;
+  static bool attr = false;
+  if (!attr) {
+    const cudaError_t e = cudaFuncSetAttribute(gemm_simt_kernel<EPI, TM, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    attr = true;
+  }
+  const unsigned grid = static_cast<unsigned>(tiles_n) * static_cast<unsigned>((g.M + TM - 1) / TM);
+  launch_pdl(gemm_simt_kernel<EPI, TM, VEC>, grid, NT, smem, s, static_cast<const float*>(g.A),
+             static_cast<const float*>(g.B), g.M, g.K, g.lda, g.ldb, tiles_n, n_rows_b, b_split, g.b_weights ? 1 : 0, ep);
+  return cudaGetLastError();
 }
 
 template <int EPI>
 cudaError_t launch(const GemmCall& g, int tiles_n, int b_split, int n_rows_b, const EpiParams& ep, cudaStream_t s) {
-  dim3 grid(tiles_n, (g.M + TM - 1) / TM);
-  launch_pdl(gemm_simt_kernel<EPI>, grid, 256, 0, s, static_cast<const float*>(g.A), static_cast<const float*>(g.B), g.M,
-                                             g.K, g.lda, g.ldb, n_rows_b, b_split, ep);
-  return cudaGetLastError();
+  static int n_sms = 0;
+  if (n_sms == 0) {
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    n_sms = n > 0 ? n : 1;
+  }
+  const bool vec = g.K % 4 == 0 && g.lda % 4 == 0 && g.ldb % 4 == 0 &&
+                   ((reinterpret_cast<uintptr_t>(g.A) | reinterpret_cast<uintptr_t>(g.B)) & 15) == 0;
+  // 16-row tiles until 32-row tiles alone put a block on every SM (512 x 256: 64 against 128 blocks)
+  const bool tall = static_cast<int64_t>(tiles_n) * ((g.M + 31) / 32) >= n_sms;
+  if (vec)
+    return tall ? launch_tile<EPI, 32, true>(g, tiles_n, b_split, n_rows_b, ep, s)
+                : launch_tile<EPI, 16, true>(g, tiles_n, b_split, n_rows_b, ep, s);
+  return launch_tile<EPI, 32, false>(g, tiles_n, b_split, n_rows_b, ep, s);
 }
 }  // namespace
 

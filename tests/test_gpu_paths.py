@@ -78,3 +78,50 @@ def test_remdm_nucleus_draws(T, V, R, top_p):
     for b in range(B):
         for r in range(first, R):
             assert _nucleus_ok(logits[b * R + r], mask, top_p, u[b, r, 2], got[b, r]), (b, r, got[b, r])
+
+
+def f32_tensor(shape, seed):
+    x = wl.normal(seed, 98, int(np.prod(shape)), 0.0, 1.0, "f32").reshape(shape)
+    return torch.from_numpy(x).cuda(), x.astype(np.float64)
+
+
+# fp32 GEMM: 16- and 32-row tiles, 16-byte and 4-byte copies, K shorter than a
+# stage, K ending inside a group's 16 columns, one row and one column
+@pytest.mark.parametrize("M,N,K", [(1, 1, 1), (17, 65, 4), (15, 64, 68), (33, 130, 257), (31, 2000, 132), (700, 900, 260),
+                                   (300, 1100, 30)])
+def test_gemm_f32_tiles(T, M, N, K):
+    A, a = f32_tensor((M, K), 3)
+    B, b = f32_tensor((N, K), 4)
+    C = torch.empty((M, N), dtype=torch.float32, device="cuda")
+    T.tadm_gemm(A, B, C, dtype=0)
+    # sums of K fp32 products of N(0, 1) values: error below K 2^-24 |a| |b|
+    assert np.abs(C.cpu().numpy() - a @ b.T).max() <= 2.0 ** -24 * (K + 4) * np.abs(a).max() * np.abs(b).max()
+
+
+# fp32 attention: rows around the 16-row block, keys around the 64-key tile,
+# an odd key stride (scalar loads), causal, windows that leave whole tiles out
+@pytest.mark.parametrize("hd,Hq,Hkv,rows,ctx,causal,window,pad", [
+    (32, 2, 1, 1, 0, False, 0, 0), (64, 2, 2, 17, 47, False, 0, 0), (64, 4, 2, 16, 48, True, 0, 3),
+    (128, 2, 1, 33, 95, True, 20, 1), (64, 2, 2, 40, 200, False, 70, 0), (32, 4, 4, 130, 0, True, 1, 2)])
+def test_attention_f32_tiles(T, hd, Hq, Hkv, rows, ctx, causal, window, pad):
+    B, n = 2, ctx + rows
+    stride = n + pad
+    q, qa = f32_tensor((B, Hq, rows, hd), 5)
+    k, ka = f32_tensor((B, Hkv, stride, hd), 6)
+    v, va = f32_tensor((B, Hkv, hd, stride), 7)
+    o = torch.empty((B * rows, Hq * hd), dtype=torch.float32, device="cuda")
+    T.tadm_attention(q, k, v, o, Hq, Hkv, rows, ctx, causal, 0, window=window)
+    pos, key = ctx + np.arange(rows)[:, None], np.arange(n)[None, :]
+    see = np.ones((rows, n), bool)
+    if causal:
+        see &= key <= pos
+    if window:
+        see &= pos - key < window
+    got = o.cpu().numpy().reshape(B, rows, Hq, hd)
+    for b in range(B):
+        for h in range(Hq):
+            g = h // (Hq // Hkv)
+            s = np.where(see, qa[b, h] @ ka[b, g, :n].T / np.sqrt(hd), -np.inf)
+            p = np.exp(s - s.max(1, keepdims=True))
+            ref = (p / p.sum(1, keepdims=True)) @ va[b, g, :, :n].T
+            assert np.abs(got[b, :, h] - ref).max() < 2e-5     # fp32 scores of magnitude ~5, sums of n terms
