@@ -1,8 +1,15 @@
 // Split-K reduction for the tcgen05 GEMM: sums the fp32 partials of the K
-// slices in slice order (deterministic) into slice 0, then runs the GEMM's own
-// epilogue on that sum, one thread per (output row, column group) of a
-// 256-column tile; the residual-add and plain-store epilogues do both in one
-// element-wise launch.
+// slices in slice order (deterministic) and runs the GEMM's own epilogue on
+// that sum, in one launch with coalesced reads: element-wise for the epilogues
+// whose outputs depend on one column (GLU: a gate and an up column), a warp
+// per head row for QKV (QK-norm, RoPE, cache write), a warp per row for the
+// paired-attention gate.  The output head, and outputs that are not 16-byte
+// aligned, take two launches: the sum into slice 0, then the epilogue, one
+// thread per (output row, column group) of a 256-column tile.
+// The two launches cost 15 us for the QKV projection of a 32-row block step,
+// 9 us for its GLU and 20 us for the gate of 256 rows (16 to 64 blocks, rows
+// read by one lane each).  With one launch each a batch-1 block step 542 -> 496 us, a 27 B block step
+// 1108 -> 1060 us.
 #include "kernels.h"
 
 namespace tadm {
@@ -67,10 +74,40 @@ __global__ void __launch_bounds__(256) splitk_sum_kernel(float* __restrict__ par
   p[i] = a;
 }
 
-// Element-wise epilogues (residual add, plain store) in one launch: each
-// thread sums four consecutive columns of one row over the slices in slice
-// order, then adds them into the residual stream (+ bias) or stores them,
-// with coalesced 16-byte accesses.  Same sums in the same order as the
+// four consecutive elements at element offset `off` of a bf16 or fp32 array (8- / 16-byte aligned)
+__device__ __forceinline__ float4 ld4(const void* base, int bf, size_t off) {
+  if (!bf) return *reinterpret_cast<const float4*>(static_cast<const float*>(base) + off);
+  const uint2 u = *reinterpret_cast<const uint2*>(static_cast<const bf16*>(base) + off);
+  const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x));
+  const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
+  return make_float4(a.x, a.y, b.x, b.y);
+}
+__device__ __forceinline__ void st4(void* base, int bf, size_t off, const float4& v) {
+  if (!bf) {
+    *reinterpret_cast<float4*>(static_cast<float*>(base) + off) = v;
+    return;
+  }
+  __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+  *reinterpret_cast<uint2*>(static_cast<bf16*>(base) + off) =
+      make_uint2(*reinterpret_cast<uint32_t*>(&a), *reinterpret_cast<uint32_t*>(&b));
+}
+template <class F>
+__device__ __forceinline__ float4 map4(const float4& a, F f) { return make_float4(f(a.x), f(a.y), f(a.z), f(a.w)); }
+__device__ __forceinline__ float4 add4(const float4& a, const float4& b) {
+  return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+}
+__device__ __forceinline__ float4 mul4(const float4& a, const float4& b) {
+  return make_float4(a.x * b.x, a.y * b.y, a.z * b.z, a.w * b.w);
+}
+__device__ __forceinline__ float4 slice_sum(const float* p, size_t stride, int splits) {
+  float4 a = *reinterpret_cast<const float4*>(p);
+  for (int ks = 1; ks < splits; ++ks) a = add4(a, *reinterpret_cast<const float4*>(p + ks * stride));
+  return a;
+}
+
+// Element-wise epilogues in one launch: each thread sums four consecutive
+// columns of one row over the slices in slice order, then runs the epilogue on
+// them, with coalesced 16-byte accesses.  Same sums in the same order as the
 // two-phase path below, so the result does not depend on which one ran.
 template <int EPI>
 __global__ void __launch_bounds__(256) splitk_elem_kernel(EpiParams ep, const float* __restrict__ part, size_t stride,
@@ -80,47 +117,181 @@ __global__ void __launch_bounds__(256) splitk_elem_kernel(EpiParams ep, const fl
   const size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x;
   if (i >= static_cast<size_t>(ep.M) * n4) return;
   const int m = static_cast<int>(i / n4), n = static_cast<int>(i % n4) * 4;
-  const float* p = part + static_cast<size_t>(m) * ldp + n;
-  float4 a = *reinterpret_cast<const float4*>(p);
-  for (int ks = 1; ks < splits; ++ks) {
-    const float4 t = *reinterpret_cast<const float4*>(p + ks * stride);
-    a.x += t.x; a.y += t.y; a.z += t.z; a.w += t.w;
+  const size_t row = static_cast<size_t>(m);
+  if constexpr (EPI == EPI_GLU) {   // a tile's 256 columns: 128 gate columns, then their up columns
+    const float* p = part + row * ldp + (n / 128) * 256 + n % 128;
+    const float4 g = slice_sum(p, stride, splits), u = slice_sum(p + 128, stride, splits);
+    const bool tanh = ep.glu != 0;
+    st4(ep.out, ep.out_bf16, row * ep.ldo + n,
+        mul4(map4(g, [&](float x) { return tanh ? gelu_tanh_f(x) : silu_f(x); }), u));
+    return;
+  }
+  float4 a = slice_sum(part + row * ldp + n, stride, splits);
+  if constexpr (EPI == EPI_RESID || EPI == EPI_FUSION1 || EPI == EPI_FUSION2) {
+    if (ep.bias) a = add4(a, ld4(ep.bias, ep.bias_bf16, n));
   }
   if constexpr (EPI == EPI_RESID) {
-    float4* r = reinterpret_cast<float4*>(ep.resid + static_cast<size_t>(m) * ep.ldr + n);
-    float4 x = *r;
-    if (ep.bias) {
-      a.x += ld_param(ep.bias, ep.bias_bf16, n + 0);
-      a.y += ld_param(ep.bias, ep.bias_bf16, n + 1);
-      a.z += ld_param(ep.bias, ep.bias_bf16, n + 2);
-      a.w += ld_param(ep.bias, ep.bias_bf16, n + 3);
-    }
-    x.x += a.x; x.y += a.y; x.z += a.z; x.w += a.w;
-    *r = x;
-  } else if (ep.out_bf16) {
-    __nv_bfloat162* o = reinterpret_cast<__nv_bfloat162*>(static_cast<bf16*>(ep.out) + static_cast<size_t>(m) * ep.ldo + n);
-    o[0] = __floats2bfloat162_rn(a.x, a.y);
-    o[1] = __floats2bfloat162_rn(a.z, a.w);
-  } else {
-    *reinterpret_cast<float4*>(static_cast<float*>(ep.out) + static_cast<size_t>(m) * ep.ldo + n) = a;
+    float4* r = reinterpret_cast<float4*>(ep.resid + row * ep.ldr + n);
+    *r = add4(*r, a);
+  } else if constexpr (EPI == EPI_STORE) {
+    st4(ep.out, ep.out_bf16, row * ep.ldo + n, a);
+  } else if constexpr (EPI == EPI_SILU) {
+    st4(ep.out, ep.out_bf16, row * ep.ldo + n, map4(a, [](float x) { return silu_f(x); }));
+  } else if constexpr (EPI == EPI_ADD) {
+    a = add4(ld4(ep.base, 0, row * ep.ldb + n), a);
+    st4(ep.out, 0, row * ep.ldo + n, a);
+    if (ep.out2) st4(ep.out2, ep.out_bf16, row * ep.ldo2 + n, a);
+  } else if constexpr (EPI == EPI_FUSION1) {
+    if (n < ep.d_split) st4(ep.out, ep.out_bf16, row * ep.ldo + n, map4(a, [](float x) { return sigmoid_f(x); }));
+    else st4(ep.out2, ep.out_bf16, row * ep.ldo2 + n - ep.d_split, map4(a, [](float x) { return gelu_erf_f(x); }));
+  } else if constexpr (EPI == EPI_FUSION2) {
+    st4(ep.out, 0, row * ep.ldo + n,
+        add4(ld4(ep.base, 0, row * ep.ldb + n), mul4(ld4(ep.gate, ep.out_bf16, row * ep.ldg + n), a)));
+  } else if constexpr (EPI == EPI_PA_UP) {
+    const float gs = static_cast<const float*>(ep.gate)[m] * ep.rowscale[m];
+    st4(ep.out, 0, row * ep.ldo + n, add4(ld4(ep.base, 0, row * ep.ldb + n), map4(a, [&](float x) { return gs * x; })));
   }
 }
 
 // true when the element-wise kernel serves this epilogue (aligned rows, N % 4 == 0)
 bool elem_ok(int epi, const EpiParams& ep, int ldp) {
   if (ep.N % 4 || ldp % 4) return false;
-  if (epi == EPI_RESID)
-    return ep.ldr % 4 == 0 && (reinterpret_cast<uintptr_t>(ep.resid) & 15) == 0;
-  if (epi == EPI_STORE)
-    return ep.ldo % 4 == 0 && (reinterpret_cast<uintptr_t>(ep.out) & 15) == 0;
-  return false;
+  auto al = [](const void* p, int ld) { return ld % 4 == 0 && (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+  const bool bias = !ep.bias || al(ep.bias, 0);
+  switch (epi) {
+    case EPI_RESID: return al(ep.resid, ep.ldr) && bias;
+    case EPI_STORE:
+    case EPI_SILU:
+    case EPI_GLU: return al(ep.out, ep.ldo);
+    case EPI_ADD: return al(ep.out, ep.ldo) && al(ep.base, ep.ldb) && (!ep.out2 || al(ep.out2, ep.ldo2));
+    case EPI_FUSION1: return al(ep.out, ep.ldo) && al(ep.out2, ep.ldo2) && ep.d_split % 4 == 0 && bias;
+    case EPI_FUSION2: return al(ep.out, ep.ldo) && al(ep.base, ep.ldb) && al(ep.gate, ep.ldg) && bias;
+    case EPI_PA_UP: return al(ep.out, ep.ldo) && al(ep.base, ep.ldb);
+    default: return false;
+  }
+}
+
+// QKV epilogue on the slice sums: a block takes 16 rows of one head, a warp
+// two of them; a lane holds the rotate-half pairs (i, i + HD / 2) of HD / 64
+// consecutive dims i, so partials, Q and K move in whole lines.  V rows cross
+// shared memory and leave transposed, 16 positions (one 32-byte sector) of a
+// dim at a time.
+template <int HD>
+__global__ void __launch_bounds__(256) splitk_qkv_kernel(EpiParams ep, const float* __restrict__ part, size_t stride,
+                                                         int ldp, int splits) {
+  pdl_enter();
+  constexpr int P = HD / 64, H2 = HD / 2, RB = 16;
+  __shared__ bf16 sv[HD][RB + 2];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int gh = blockIdx.y, m0 = blockIdx.x * RB;
+  int region = 2, head = gh - ep.n_heads - ep.n_kv_heads;
+  if (gh < ep.n_heads) { region = 0; head = gh; }
+  else if (gh < ep.n_heads + ep.n_kv_heads) { region = 1; head = gh - ep.n_heads; }
+  const void* gain = region == 0 ? ep.q_gain : region == 1 ? ep.k_gain : nullptr;
+#pragma unroll
+  for (int rr = w; rr < RB; rr += 8) {
+    const int m = m0 + rr;
+    if (m >= ep.M) continue;                       // uniform across the warp
+    const float* p = part + static_cast<size_t>(m) * ldp + gh * HD + lane * P;
+    float a[P], c[P];
+#pragma unroll
+    for (int t = 0; t < P; ++t) a[t] = c[t] = 0.0f;
+#pragma unroll 4
+    for (int ks = 0; ks < splits; ++ks) {
+      const float* q = p + ks * stride;
+      if constexpr (P == 2) {
+        const float2 x = *reinterpret_cast<const float2*>(q), y = *reinterpret_cast<const float2*>(q + H2);
+        a[0] += x.x; a[1] += x.y; c[0] += y.x; c[1] += y.y;
+      } else {
+        a[0] += q[0];
+        c[0] += q[H2];
+      }
+    }
+    const int b = m / ep.R, r = m - b * ep.R, pos = ep.ctx + r;
+    if (region == 2) {
+#pragma unroll
+      for (int t = 0; t < P; ++t) {
+        sv[lane * P + t][rr] = __float2bfloat16_rn(a[t]);
+        sv[H2 + lane * P + t][rr] = __float2bfloat16_rn(c[t]);
+      }
+      continue;
+    }
+    if (gain) {
+      float ss = 0.0f;
+#pragma unroll
+      for (int t = 0; t < P; ++t) ss = fmaf(a[t], a[t], fmaf(c[t], c[t], ss));
+      const float inv = rsqrtf(warp_sum(ss) / static_cast<float>(HD) + ep.qk_eps);
+#pragma unroll
+      for (int t = 0; t < P; ++t) {
+        a[t] *= inv * ld_param(gain, ep.bias_bf16, lane * P + t);
+        c[t] *= inv * ld_param(gain, ep.bias_bf16, H2 + lane * P + t);
+      }
+    }
+    if (ep.rope) {
+#pragma unroll
+      for (int t = 0; t < P; ++t) {
+        const float2 cs = ep.rope_tab[static_cast<size_t>(lane * P + t) * ep.rope_npos + pos];
+        const float x = a[t], y = c[t];
+        a[t] = x * cs.x - y * cs.y;
+        c[t] = y * cs.x + x * cs.y;
+      }
+    }
+    bf16* dst = region == 0
+                    ? static_cast<bf16*>(ep.q) + ((static_cast<size_t>(b) * ep.n_heads + head) * ep.R + r) * HD
+                    : static_cast<bf16*>(ep.k) + ((static_cast<size_t>(b) * ep.n_kv_heads + head) * ep.kv_stride + pos) * HD;
+    if constexpr (P == 2) {
+      *reinterpret_cast<__nv_bfloat162*>(dst + 2 * lane) = __floats2bfloat162_rn(a[0], a[1]);
+      *reinterpret_cast<__nv_bfloat162*>(dst + H2 + 2 * lane) = __floats2bfloat162_rn(c[0], c[1]);
+    } else {
+      dst[lane] = __float2bfloat16_rn(a[0]);
+      dst[H2 + lane] = __float2bfloat16_rn(c[0]);
+    }
+  }
+  if (region != 2) return;                         // uniform across the block
+  __syncthreads();
+  for (int i = threadIdx.x; i < HD * RB; i += 256) {
+    const int d = i / RB, rr = i % RB, m = m0 + rr;
+    if (m >= ep.M) continue;
+    const int b = m / ep.R, pos = ep.ctx + m - b * ep.R;
+    static_cast<bf16*>(ep.v)[((static_cast<size_t>(b) * ep.n_kv_heads + head) * HD + d) * ep.kv_stride + pos] = sv[d][rr];
+  }
+}
+
+// Paired-attention gate on the slice sums: one warp per row (N <= 256 columns, N % 4 == 0).
+__global__ void __launch_bounds__(256) splitk_gate_kernel(EpiParams ep, const float* __restrict__ part, size_t stride,
+                                                          int ldp, int splits) {
+  pdl_enter();
+  const int m = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (m >= ep.M) return;
+  float s = 0.0f;
+  for (int n = 4 * lane; n < ep.N; n += 128) {
+    const float4 a = slice_sum(part + static_cast<size_t>(m) * ldp + n, stride, splits);
+    s += silu_f(a.x) * ld_param(ep.vec, ep.bias_bf16, n) + silu_f(a.y) * ld_param(ep.vec, ep.bias_bf16, n + 1) +
+         silu_f(a.z) * ld_param(ep.vec, ep.bias_bf16, n + 2) + silu_f(a.w) * ld_param(ep.vec, ep.bias_bf16, n + 3);
+  }
+  s = warp_sum(s);
+  if (lane == 0) static_cast<float*>(ep.out)[m] = sigmoid_f(s + ld_param(ep.bias, ep.bias_bf16, 0));
 }
 
 // Phase 2: the epilogue on slice 0.
 template <int EPI>
 cudaError_t launch(const EpiParams& ep, const float* part, size_t stride, int ldp, int splits, int n_tiles_n,
                    cudaStream_t s, int* launches) {
-  if constexpr (EPI == EPI_RESID || EPI == EPI_STORE) {
+  if constexpr (EPI == EPI_QKV) {
+    if (ep.out_bf16 && (ep.head_dim == 64 || ep.head_dim == 128)) {
+      *launches = 1;
+      const dim3 grid((ep.M + 15) / 16, ep.n_heads + 2 * ep.n_kv_heads);
+      if (ep.head_dim == 64) launch_pdl(splitk_qkv_kernel<64>, grid, 256, 0, s, ep, part, stride, ldp, splits);
+      else launch_pdl(splitk_qkv_kernel<128>, grid, 256, 0, s, ep, part, stride, ldp, splits);
+      return cudaGetLastError();
+    }
+  } else if constexpr (EPI == EPI_PA_GATE) {
+    if (ep.N % 4 == 0) {
+      *launches = 1;
+      launch_pdl(splitk_gate_kernel, (ep.M + 7) / 8, 256, 0, s, ep, part, stride, ldp, splits);
+      return cudaGetLastError();
+    }
+  } else if constexpr (EPI != EPI_LMHEAD) {
     if (elem_ok(EPI, ep, ldp)) {
       *launches = 1;
       const size_t n = static_cast<size_t>(ep.M) * (ep.N / 4);

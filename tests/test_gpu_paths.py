@@ -125,3 +125,31 @@ def test_attention_f32_tiles(T, hd, Hq, Hkv, rows, ctx, causal, window, pad):
             p = np.exp(s - s.max(1, keepdims=True))
             ref = (p / p.sum(1, keepdims=True)) @ va[b, g, :, :n].T
             assert np.abs(got[b, :, h] - ref).max() < 2e-5     # fp32 scores of magnitude ~5, sums of n terms
+
+
+# split-K reductions of every epilogue (QKV per head row, GLU, fusion gate /
+# hidden / output, paired-attention gate, add, up) at row counts around their
+# 16-row blocks, both head widths, QK-norm, and the paired-attention kernels
+@pytest.mark.parametrize("hd,fusion,qk_norm,batch,rows", [(128, "gated_mlp", False, 3, 11), (64, "gated_mlp", True, 1, 1),
+                                                          (128, "paired_attn", True, 2, 24), (64, "paired_attn", False, 5, 32),
+                                                          (128, "paired_attn", False, 1, 17)])
+def test_few_row_steps_match_the_oracle(T, hd, fusion, qk_norm, batch, rows):
+    m = wl.ModelConfig(vocab=1024, d_model=1024, n_heads=1024 // hd, n_kv_heads=512 // hd, head_dim=hd, ffn=2048, n_anchor=1,
+                       n_denoise=1, fusion=fusion, fusion_rank=256, fusion_heads=4, dtype="bf16", qk_norm=qk_norm,
+                       qkv_split=hd == 128)
+    host = wl.make_weights(m, seed=3, affine_std=0.05)
+    tm = T.TadmModel(m, T.upload_weights(m, host), max_batch=batch, max_rows=rows)
+    w = wl.Workload("t", m, batch=batch, prompt_len=0, gen_len=rows, steps_per_block=4, K=4)
+    z0, z1 = (wl.random_canvas(w, batch, rows, f, s) for f, s in ((0.9, 1), (0.4, 2)))
+    cache = tm.new_cache(batch, rows)
+    logits = torch.empty((batch * rows, m.vocab), dtype=torch.float32, device="cuda")
+    tm.tadm_reset(batch)
+    tm.tadm_anchor_forward(torch.from_numpy(z0).cuda(), 4, cache)
+    tm.tadm_denoise_step(torch.from_numpy(z1).cuda(), 3, 4, 0, cache, logits=logits)
+    tm.tadm_sync_status()
+    o = O.Oracle(m, host)
+    sess = o.new_session(batch)
+    ref = o.denoise_logits(sess, z1, o.anchor_forward(sess, z0)).reshape(batch * rows, m.vocab)
+    rel = np.linalg.norm(logits.cpu().numpy() - ref) / np.linalg.norm(ref)
+    assert rel < 1.5e-2, rel          # bf16 operands, two layers and the fusion
+    tm.close()
