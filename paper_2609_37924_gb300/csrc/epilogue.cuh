@@ -183,7 +183,7 @@ __device__ __forceinline__ void epilogue_row(const EpiParams& p, int m, int n_bl
   float v[32];
   // Sources that can stage (tensor-core path) write bf16 outputs 64 columns at
   // a time through shared memory with one TMA store per warp (full lines).
-  if constexpr (Src::kStaged && (EPI == EPI_STORE || EPI == EPI_FUSION1)) {
+  if constexpr (Src::kStaged && (EPI == EPI_STORE || EPI == EPI_FUSION1 || EPI == EPI_SILU)) {
     if (src.staged()) {
       float w[32];
       for (int c = c_lo; c + 1 < c_hi; c += 2) {
@@ -213,6 +213,13 @@ __device__ __forceinline__ void epilogue_row(const EpiParams& p, int m, int n_bl
           }
           which = gate ? 0 : 1;
           x = gate ? n0 : n0 - p.d_split;
+        }
+        if constexpr (EPI == EPI_SILU) {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) {
+            v[i] = silu_f(v[i]);
+            w[i] = silu_f(w[i]);
+          }
         }
         src.store64(which, x, v, w);
       }
@@ -253,10 +260,13 @@ __device__ __forceinline__ void epilogue_row(const EpiParams& p, int m, int n_bl
       return;
     }
   }
-  // fp32 read-modify-write epilogues on the tensor-core path: the warp's 32 x 32
+  // epilogues that read an fp32 row on the tensor-core path: the warp's 32 x 32
   // accumulator chunk is transposed through its shared-memory box so that each
-  // global access instruction covers 32 consecutive columns of one row.
-  if constexpr (Src::kStaged && (EPI == EPI_RESID || EPI == EPI_FUSION2)) {
+  // global access instruction covers 32 consecutive columns of one row (with a
+  // lane per row, the 256 x 5376 up-projection of the paired-attention fusion
+  // took 28 us and its 256 x 256 mixer output 28 us, cold caches; with the
+  // row operations below the fusion, the 27 B block step went 1060 -> 1043 us).
+  if constexpr (Src::kStaged && (EPI == EPI_RESID || EPI == EPI_FUSION2 || EPI == EPI_ADD || EPI == EPI_PA_UP)) {
     if (src.has_box()) {
       const int lane = threadIdx.x & 31;
       for (int c = c_lo; c < c_hi; ++c) {
@@ -277,7 +287,8 @@ __device__ __forceinline__ void epilogue_row(const EpiParams& p, int m, int n_bl
               xv[i] = ok ? p.resid[m_i * p.ldr + n] : 0.0f;
             } else {
               xv[i] = ok ? p.base[m_i * p.ldb + n] : 0.0f;
-              gv[i] = ok ? ld_param(p.gate, p.out_bf16, static_cast<int>(m_i * p.ldg + n)) : 0.0f;
+              if constexpr (EPI == EPI_FUSION2) gv[i] = ok ? ld_param(p.gate, p.out_bf16, static_cast<int>(m_i * p.ldg + n)) : 0.0f;
+              if constexpr (EPI == EPI_PA_UP) gv[i] = ok ? static_cast<const float*>(p.gate)[m_i] * p.rowscale[m_i] : 0.0f;
             }
           }
 #pragma unroll
@@ -285,8 +296,20 @@ __device__ __forceinline__ void epilogue_row(const EpiParams& p, int m, int n_bl
             const size_t m_i = static_cast<size_t>(src.row0 + h0 + i);
             if (h0 + i < nrows && col_ok) {
               const float a = src.get(h0 + i);
-              if constexpr (EPI == EPI_RESID) p.resid[m_i * p.ldr + n] = xv[i] + a + bias;
-              else static_cast<float*>(p.out)[m_i * p.ldo + n] = xv[i] + gv[i] * (a + bias);
+              if constexpr (EPI == EPI_RESID) {
+                p.resid[m_i * p.ldr + n] = xv[i] + a + bias;
+              } else if constexpr (EPI == EPI_ADD) {
+                const float y = xv[i] + a;
+                static_cast<float*>(p.out)[m_i * p.ldo + n] = y;
+                if (p.out2) {
+                  if (p.out_bf16) static_cast<bf16*>(p.out2)[m_i * p.ldo2 + n] = __float2bfloat16_rn(y);
+                  else static_cast<float*>(p.out2)[m_i * p.ldo2 + n] = y;
+                }
+              } else if constexpr (EPI == EPI_PA_UP) {
+                static_cast<float*>(p.out)[m_i * p.ldo + n] = xv[i] + gv[i] * a;
+              } else {
+                static_cast<float*>(p.out)[m_i * p.ldo + n] = xv[i] + gv[i] * (a + bias);
+              }
             }
           }
         }

@@ -736,12 +736,12 @@ const char* gemm_tc(const GemmCall& g, cudaStream_t s) {
   a.ep.resid_tma = 0;
   a.ep.f32_tma = 0;
   a.part_tma = 0;
-  if (g.epi == EPI_RESID || g.epi == EPI_FUSION2) {
+  if (g.epi == EPI_RESID || g.epi == EPI_FUSION2 || g.epi == EPI_ADD || g.epi == EPI_PA_UP) {
     a.staged = 1;   // the boxes serve as transpose scratch, or as the source of TMA reduce-adds
     if (g.epi == EPI_RESID && (reinterpret_cast<uintptr_t>(g.ep.resid) & 15) == 0 && g.ep.ldr % 4 == 0 &&
         make_f32_map(&tc, g.ep.resid, g.M, g.N, g.ep.ldr))
       a.ep.resid_tma = 1;
-  } else if (g.ep.out_bf16 && (g.epi == EPI_STORE || g.epi == EPI_GLU)) {
+  } else if (g.ep.out_bf16 && (g.epi == EPI_STORE || g.epi == EPI_GLU || g.epi == EPI_SILU)) {
     if (aligned(g.ep.out, g.ep.ldo) && make_out_map(&tc, g.ep.out, g.M, g.N, g.ep.ldo)) a.staged = 1;
   } else if (g.ep.out_bf16 && g.epi == EPI_FUSION1 && g.ep.d_split % 64 == 0) {
     if (aligned(g.ep.out, g.ep.ldo) && aligned(g.ep.out2, g.ep.ldo2) &&

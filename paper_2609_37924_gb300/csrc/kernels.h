@@ -89,7 +89,9 @@ const char* ln_pair_rows(const float* c, const float* h, int M, int d, const voi
                          cudaStream_t s);
 const char* layernorm_rows(const float* x, int M, int d, const void* w, const void* b, int w_bf16, float eps,
                            float* out, cudaStream_t s);
-const char* rms_scale_rows(const float* x, int M, int d, float eps, float* s_out, cudaStream_t st);
+// s_out = sqrt(mean(x^2) + eps) per row, out = x / s_out (act type)
+const char* rms_divide_rows(const float* x, int M, int d, float eps, float* s_out, void* out, int act_bf16,
+                            cudaStream_t st);
 // sandwich norm: x += y / sqrt(mean(y^2) + eps) * g_post; with g_next, also
 // out = x / sqrt(mean(x^2) + eps) * g_next (the next sub-block's pre-norm, act type)
 const char* post_norm_add(float* x, const float* y, int M, int d, const void* g_post, const void* g_next, int w_bf16,
@@ -97,7 +99,9 @@ const char* post_norm_add(float* x, const float* y, int M, int d, const void* g_
 const char* scale_rows(const float* x, const float* sc, int M, int d, void* out, int act_bf16, cudaStream_t s);
 const char* concat_rows(const float* const* parts, const int* widths, int n_parts, int M, void* out,
                         int act_bf16, cudaStream_t s);
-const char* sub_rows(const float* a, const float* b, int M, int d, float* out, cudaStream_t s);
+// F = [U; Z0; Z - Z0; phi - phi0] [M, 4r] and Mout = phi - phi0 [M, r] (act type)
+const char* pa_features(const float* U, const float* Z0, const float* Z, const float* phi, const float* phi0, int M, int r,
+                        void* F, void* Mout, int act_bf16, cudaStream_t s);
 const char* rope_table(float2* tab, int n_pos, int head_dim, float theta, cudaStream_t s);
 const char* fill_canvas(int32_t* z, int ldz, const int32_t* prompt, int batch, int prompt_len, int total,
                         int mask_id, cudaStream_t s);

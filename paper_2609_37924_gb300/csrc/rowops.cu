@@ -467,15 +467,34 @@ __global__ void __launch_bounds__(256) post_norm_add_block_kernel(float* __restr
   }
 }
 
-__global__ void rms_scale_kernel(const float* __restrict__ x, int M, int d, float eps, float* __restrict__ s) {
+// s[row] = sqrt(mean(x^2) + eps) and out = x / s[row], one 256-thread block per
+// row (d % 4 == 0); the row comes back from L1 / L2 for the division.
+template <class T>
+__global__ void __launch_bounds__(256) rms_divide_kernel(const float* __restrict__ x, int d, float eps,
+                                                         float* __restrict__ s, void* __restrict__ out) {
   pdl_enter();
-  const int m = blockIdx.x * WPB + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (m >= M) return;
-  const float* xr = x + static_cast<size_t>(m) * d;
+  __shared__ float red[8];
+  const size_t base = static_cast<size_t>(blockIdx.x) * d;
   float ss = 0.0f;
-  for (int j = lane; j < d; j += 32) ss += xr[j] * xr[j];
+  for (int j = threadIdx.x * 4; j < d; j += 1024) {
+    const float4 v = *reinterpret_cast<const float4*>(x + base + j);
+    ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+  }
   ss = warp_sum(ss);
-  if (lane == 0) s[m] = sqrtf(ss / static_cast<float>(d) + eps);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
+  __syncthreads();
+  float tot = 0.0f;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) tot += red[w];
+  const float sc = sqrtf(tot / static_cast<float>(d) + eps);
+  if (threadIdx.x == 0) s[blockIdx.x] = sc;
+  for (int j = threadIdx.x * 4; j < d; j += 1024) {
+    const float4 v = *reinterpret_cast<const float4*>(x + base + j);
+    store_act<T>(out, base + j + 0, v.x / sc);
+    store_act<T>(out, base + j + 1, v.y / sc);
+    store_act<T>(out, base + j + 2, v.z / sc);
+    store_act<T>(out, base + j + 3, v.w / sc);
+  }
 }
 
 // out = x / s[row], element-wise over four columns per thread (d % 4 == 0)
@@ -494,23 +513,23 @@ __global__ void scale_rows_kernel(const float* __restrict__ x, const float* __re
   store_act<T>(out, e + 3, v.w / s);
 }
 
-// s[row] = sqrt(mean(x^2) + eps), one 256-thread block per row (few rows)
-__global__ void __launch_bounds__(256) rms_scale_block_kernel(const float* __restrict__ x, int d, float eps,
-                                                              float* __restrict__ s) {
+// Gate features of the paired-attention fusion and the up-projection's input,
+// one output element of width r per thread: M = phi - phi0, F = [U; Z0; Z - Z0; M]
+// and a copy of M (four launches of differences and concatenations before).
+template <class T>
+__global__ void pa_features_kernel(const float* __restrict__ U, const float* __restrict__ Z0, const float* __restrict__ Z,
+                                   const float* __restrict__ phi, const float* __restrict__ phi0, size_t n, int r,
+                                   void* __restrict__ F, void* __restrict__ Mout) {
   pdl_enter();
-  __shared__ float red[8];
-  const int m = blockIdx.x;
-  const float* xr = x + static_cast<size_t>(m) * d;
-  float ss = 0.0f;
-  for (int j = threadIdx.x; j < d; j += 256) ss += xr[j] * xr[j];
-  ss = warp_sum(ss);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float tot = 0.0f;
-    for (int w = 0; w < 8; ++w) tot += red[w];
-    s[m] = sqrtf(tot / static_cast<float>(d) + eps);
-  }
+  const size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x;
+  if (i >= n) return;
+  const size_t f = i / r * 4 * r + i % r;
+  const float z0 = Z0[i], m = phi[i] - phi0[i];
+  store_act<T>(F, f, U[i]);
+  store_act<T>(F, f + r, z0);
+  store_act<T>(F, f + 2 * r, Z[i] - z0);
+  store_act<T>(F, f + 3 * r, m);
+  store_act<T>(Mout, i, m);
 }
 
 struct Parts {
@@ -529,13 +548,6 @@ __global__ void concat_kernel(Parts parts, int M, int width, void* __restrict__ 
   int col = static_cast<int>(i % width), k = 0;
   while (col >= parts.w[k]) col -= parts.w[k++];
   store_act<T>(out, i, parts.p[k][static_cast<size_t>(m) * parts.w[k] + col]);
-}
-
-__global__ void sub_kernel(const float* __restrict__ a, const float* __restrict__ b, size_t n, float* __restrict__ o) {
-  pdl_enter();
-  for (size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; i < n;
-       i += static_cast<size_t>(gridDim.x) * blockDim.x)
-    o[i] = a[i] - b[i];
 }
 
 // tab[j][pos] = (cos, sin)(pos * theta^(-2j/hd)), angles evaluated in double
@@ -670,13 +682,12 @@ const char* layernorm_rows(const float* x, int M, int d, const void* w, const vo
   return err();
 }
 
-const char* rms_scale_rows(const float* x, int M, int d, float eps, float* s_out, cudaStream_t st) {
+const char* rms_divide_rows(const float* x, int M, int d, float eps, float* s_out, void* out, int act_bf16,
+                            cudaStream_t st) {
   if (M <= 0) return nullptr;
-  if (M < 1024) {   // few rows: a block per row keeps enough SMs busy
-    launch_pdl(rms_scale_block_kernel, M, 256, 0, st, x, d, eps, s_out);
-    return err();
-  }
-  launch_pdl(rms_scale_kernel, rows_grid(M), WPB * 32, 0, st, x, M, d, eps, s_out);
+  if (d % 4) return "rms_divide_rows needs d % 4 == 0";
+  if (act_bf16) launch_pdl(rms_divide_kernel<bf16>, M, 256, 0, st, x, d, eps, s_out, out);
+  else launch_pdl(rms_divide_kernel<float>, M, 256, 0, st, x, d, eps, s_out, out);
   return err();
 }
 
@@ -730,11 +741,13 @@ const char* concat_rows(const float* const* parts, const int* widths, int n_part
   return err();
 }
 
-const char* sub_rows(const float* a, const float* b, int M, int d, float* out, cudaStream_t s) {
-  const size_t n = static_cast<size_t>(M) * d;
+const char* pa_features(const float* U, const float* Z0, const float* Z, const float* phi, const float* phi0, int M, int r,
+                        void* F, void* Mout, int act_bf16, cudaStream_t s) {
+  const size_t n = static_cast<size_t>(M) * r;
   if (n == 0) return nullptr;
-  const int blocks = static_cast<int>((n + 255) / 256 < 65535 ? (n + 255) / 256 : 65535);
-  launch_pdl(sub_kernel, blocks, 256, 0, s, a, b, n, out);
+  const unsigned blocks = static_cast<unsigned>((n + 255) / 256);
+  if (act_bf16) launch_pdl(pa_features_kernel<bf16>, blocks, 256, 0, s, U, Z0, Z, phi, phi0, n, r, F, Mout);
+  else launch_pdl(pa_features_kernel<float>, blocks, 256, 0, s, U, Z0, Z, phi, phi0, n, r, F, Mout);
   return err();
 }
 

@@ -135,7 +135,7 @@ struct tadm_handle {
     size_t status, rope, rope_g, post, c, x, h_int, norm, qbuf, kv, attn, glu, f_g, f_hid, f_pre, part, conf, tok,
         split, idx;
     size_t attn_part, act, cnt;
-    size_t pa_z, pa_j, pa_mq, pa_mk, pa_mv, pa_mo, pa_r, pa_rb, pa_hid, pa_phi, pa_m, pa_dz, pa_f, pa_g, pa_mb;
+    size_t pa_z, pa_j, pa_mq, pa_mk, pa_mv, pa_mo, pa_r, pa_rb, pa_hid, pa_phi, pa_f, pa_g, pa_mb;
   } off{};
   size_t kv_slab = 0;
   int kv_stride = 0, n_part_tiles = 0;
@@ -285,8 +285,6 @@ void layout(tadm_handle* h) {
     f.pa_rb = take(M * r * es);
     f.pa_hid = take(M * 2 * r * es);
     f.pa_phi = take(M * r * 4);
-    f.pa_m = take(M * r * 4);
-    f.pa_dz = take(M * r * 4);
     f.pa_f = take(M * 4 * r * es);
     f.pa_g = take(M * 4);
     f.pa_mb = take(M * r * es);
@@ -514,13 +512,15 @@ tadm_status mixer(tadm_handle* h, const float* Z, const float* U, int B, int R, 
   return TADM_OK;
 }
 
-// Z = (X / s) W^T as fp32 [M, r]; X / s is staged in the norm buffer.
-tadm_status project_scaled(tadm_handle* h, const float* X, const float* sc, const void* W, int M, float* Z,
+// Z = (X / s) W^T as fp32 [M, r]; X / s is staged in the norm buffer.  fresh:
+// s = sqrt(mean(X^2) + 1e-6) per row is computed and kept in sc, else read.
+tadm_status project_scaled(tadm_handle* h, const float* X, float* sc, bool fresh, const void* W, int M, float* Z,
                            cudaStream_t s) {
   const tadm_config& c = h->cfg;
   const int64_t Mmax = static_cast<int64_t>(h->max_batch) * h->max_rows;
   void* norm = h->at(h->off.norm);
-  TRY(scale_rows(X, sc, M, c.d_model, norm, h->act_bf16(), s));
+  if (fresh) TRY(rms_divide_rows(X, M, c.d_model, 1e-6f, sc, norm, h->act_bf16(), s));
+  else TRY(scale_rows(X, sc, M, c.d_model, norm, h->act_bf16(), s));
   EpiParams e{};
   e.out = Z;
   e.ldo = c.fusion_rank;
@@ -538,10 +538,8 @@ tadm_status run_A(tadm_handle* h, int B, int R, int causal, void* cache, cudaStr
   TRYS(stack_fwd(h, c.n_shared, c.n_anchor, cv.h, B, R, h->ctx, causal, s));
   if (c.fusion == 1) {
     // s_C, s_H, Z0 = (C0/s_C) W_C, U = (H0/s_H) W_H, phi(Z0, U)
-    TRY(rms_scale_rows(cbuf, M, c.d_model, 1e-6f, cv.sC, s));
-    TRY(rms_scale_rows(cv.h, M, c.d_model, 1e-6f, cv.sH, s));
-    TRYS(project_scaled(h, cbuf, cv.sC, h->fw[0], M, cv.Z0, s));
-    TRYS(project_scaled(h, cv.h, cv.sH, h->fw[1], M, cv.U, s));
+    TRYS(project_scaled(h, cbuf, cv.sC, true, h->fw[0], M, cv.Z0, s));
+    TRYS(project_scaled(h, cv.h, cv.sH, true, h->fw[1], M, cv.U, s));
     TRYS(mixer(h, cv.Z0, cv.U, B, R, cv.phi0, s));
   }
   return TADM_OK;
@@ -595,26 +593,17 @@ tadm_status run_fusion(tadm_handle* h, int B, int R, const void* cache, cudaStre
   // F = [U; Z0; Z - Z0; M]; g = sigmoid(SiLU(F W_g1) W_g2 + b_g); H~ = H0 + g s_H (M W_up)
   const int r = c.fusion_rank;
   float* Z = h->at<float>(h->off.pa_z);
-  TRYS(project_scaled(h, cbuf, cv.sC, h->fw[0], M, Z, s));
+  TRYS(project_scaled(h, cbuf, cv.sC, false, h->fw[0], M, Z, s));
   float* phi = h->at<float>(h->off.pa_phi);
   TRYS(mixer(h, Z, cv.U, B, R, phi, s));
-  float* Mm = h->at<float>(h->off.pa_m);
-  float* dZ = h->at<float>(h->off.pa_dz);
-  TRY(sub_rows(phi, cv.phi0, M, r, Mm, s));
-  TRY(sub_rows(Z, cv.Z0, M, r, dZ, s));
-  const float* parts[4] = {cv.U, cv.Z0, dZ, Mm};
-  const int widths[4] = {r, r, r, r};
   void* F = h->at(h->off.pa_f);
-  TRY(concat_rows(parts, widths, 4, M, F, h->act_bf16(), s));
+  void* Mb = h->at(h->off.pa_mb);
+  TRY(pa_features(cv.U, cv.Z0, Z, phi, cv.phi0, M, r, F, Mb, h->act_bf16(), s));
   EpiParams eg{};
   eg.vec = h->fw[7];
   eg.bias = h->fw[8];
   eg.out = h->at(h->off.pa_g);
   TRYS(gemm(h, F, Mmax, 4 * r, h->fw[6], 4 * r, M, r, 4 * r, EPI_PA_GATE, eg, s));
-  const float* mparts[1] = {Mm};
-  const int mw[1] = {r};
-  void* Mb = h->at(h->off.pa_mb);
-  TRY(concat_rows(mparts, mw, 1, M, Mb, h->act_bf16(), s));
   EpiParams eu{};
   eu.base = cv.h;
   eu.ldb = d;
