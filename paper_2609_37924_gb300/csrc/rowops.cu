@@ -93,6 +93,167 @@ __global__ void embed_kernel(const int32_t* __restrict__ z, int ldz, int rows, i
   }
 }
 
+// embed_kernel with a 256-thread block per row, for few rows (32 x 2048: 10 ->
+// 6 us with the copy behind it): eight bf16 (16 bytes) per thread and step.  d % 8 == 0, 16-byte
+// aligned bf16 table, out and add; no second output.
+__global__ void __launch_bounds__(256) embed_block_kernel(const int32_t* __restrict__ z, int ldz, int rows,
+                                                          const bf16* __restrict__ E, int d, int vocab,
+                                                          float* __restrict__ out, const float* __restrict__ add,
+                                                          int add_first, const float* __restrict__ add_div) {
+  pdl_enter();
+  const int m = blockIdx.x, b = m / rows, r = m - b * rows;
+  int tok = z[static_cast<size_t>(b) * ldz + r];
+  tok = tok < 0 ? 0 : (tok >= vocab ? vocab - 1 : tok);  // never read outside E
+  const size_t ar = static_cast<size_t>(b) * (rows - add_first) + (r - add_first);
+  const float* a = add && r >= add_first ? add + ar * d : nullptr;
+  const float sc = a && add_div ? 1.0f / add_div[ar] : 1.0f;
+  const bf16* e = E + static_cast<size_t>(tok) * d;
+  float* o = out + static_cast<size_t>(m) * d;
+  for (int j = threadIdx.x * 8; j < d; j += 2048) {
+    const uint4 raw = *reinterpret_cast<const uint4*>(e + j);
+    const __nv_bfloat162* p2 = reinterpret_cast<const __nv_bfloat162*>(&raw);
+    float4 v[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const float2 x = __bfloat1622float2(p2[2 * q]), y = __bfloat1622float2(p2[2 * q + 1]);
+      v[q] = make_float4(x.x, x.y, y.x, y.y);
+      if (a) {
+        const float4 t = *reinterpret_cast<const float4*>(a + j + 4 * q);
+        v[q].x = fmaf(t.x, sc, v[q].x);
+        v[q].y = fmaf(t.y, sc, v[q].y);
+        v[q].z = fmaf(t.z, sc, v[q].z);
+        v[q].w = fmaf(t.w, sc, v[q].w);
+      }
+      *reinterpret_cast<float4*>(o + j + 4 * q) = v[q];
+    }
+  }
+}
+
+// One row of d <= 8192 columns (d % 4 == 0) held by a 256-thread block: thread
+// t has the float4 at 4 t + 1024 i.  Few-row launches are paced by the latency
+// of one row; a block per row reads it once, with every load in flight.
+constexpr int kRowVec = 8;
+__device__ __forceinline__ void load_row_block(const float* __restrict__ x, int d, float4 (&v)[kRowVec]) {
+#pragma unroll
+  for (int i = 0; i < kRowVec; ++i) {
+    const int j = 4 * threadIdx.x + 1024 * i;
+    v[i] = j < d ? *reinterpret_cast<const float4*>(x + j) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  }
+}
+// sum over the block (256 threads); every thread gets it
+__device__ __forceinline__ float block_sum256(float v, float* red) {
+  v = warp_sum(v);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  float t = 0.0f;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) t += red[w];
+  return t;
+}
+// four consecutive parameters / activations (8- or 16-byte aligned)
+__device__ __forceinline__ float4 ldw4(const void* w, int bf, int j) {
+  if (!bf) return *reinterpret_cast<const float4*>(static_cast<const float*>(w) + j);
+  const uint2 u = *reinterpret_cast<const uint2*>(static_cast<const bf16*>(w) + j);
+  const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x));
+  const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
+  return make_float4(a.x, a.y, b.x, b.y);
+}
+template <class T>
+__device__ __forceinline__ void store4(void* out, size_t i, const float4& y);
+template <>
+__device__ __forceinline__ void store4<float>(void* out, size_t i, const float4& y) {
+  *reinterpret_cast<float4*>(static_cast<float*>(out) + i) = y;
+}
+template <>
+__device__ __forceinline__ void store4<bf16>(void* out, size_t i, const float4& y) {
+  __nv_bfloat162 a = __floats2bfloat162_rn(y.x, y.y), b = __floats2bfloat162_rn(y.z, y.w);
+  *reinterpret_cast<uint2*>(static_cast<bf16*>(out) + i) =
+      make_uint2(*reinterpret_cast<uint32_t*>(&a), *reinterpret_cast<uint32_t*>(&b));
+}
+
+// rmsnorm_block_kernel for d <= 8192 with the row in registers and 8- / 16-byte
+// accesses (16-byte aligned pointers, ldo % 4 == 0)
+template <class T>
+__global__ void __launch_bounds__(256) rmsnorm_block_reg_kernel(const float* __restrict__ x, int d,
+                                                                const void* __restrict__ gain, int w_bf16, float eps,
+                                                                void* __restrict__ out, int ldo,
+                                                                const int32_t* __restrict__ rows_idx, int lo_off) {
+  pdl_enter();
+  __shared__ float red[8];
+  const int m = blockIdx.x;
+  float4 v[kRowVec];
+  load_row_block(x + static_cast<size_t>(rows_idx ? rows_idx[m] : m) * d, d, v);
+  float ss = 0.0f;
+#pragma unroll
+  for (int i = 0; i < kRowVec; ++i) ss += v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
+  const float inv = rsqrtf(block_sum256(ss, red) / static_cast<float>(d) + eps);
+#pragma unroll
+  for (int i = 0; i < kRowVec; ++i) {
+    const int j = 4 * threadIdx.x + 1024 * i;
+    if (j >= d) break;
+    const float4 g = ldw4(gain, w_bf16, j);
+    const float4 y = make_float4(v[i].x * inv * g.x, v[i].y * inv * g.y, v[i].z * inv * g.z, v[i].w * inv * g.w);
+    const size_t o = static_cast<size_t>(m) * ldo + j;
+    store4<T>(out, o, y);
+    if constexpr (sizeof(T) == 2) {
+      if (lo_off > 0)       // remainder of the split operand
+        store4<T>(out, o + lo_off,
+                  make_float4(y.x - __bfloat162float(__float2bfloat16_rn(y.x)), y.y - __bfloat162float(__float2bfloat16_rn(y.y)),
+                              y.z - __bfloat162float(__float2bfloat16_rn(y.z)), y.w - __bfloat162float(__float2bfloat16_rn(y.w))));
+    }
+  }
+}
+
+// LayerNorm of the row in v by its block: mean, then the variance about it, then out[o + j] (+ affine)
+template <class T>
+__device__ __forceinline__ void ln_row_block(const float4 (&v)[kRowVec], int d, const void* w, const void* b, int w_bf16,
+                                             float eps, void* out, size_t o, float (*red)[8]) {
+  float s = 0.0f;
+#pragma unroll
+  for (int i = 0; i < kRowVec; ++i) s += v[i].x + v[i].y + v[i].z + v[i].w;
+  const float mean = block_sum256(s, red[0]) / static_cast<float>(d);
+  float q = 0.0f;
+#pragma unroll
+  for (int i = 0; i < kRowVec; ++i) {
+    if (static_cast<int>(4 * threadIdx.x + 1024 * i) >= d) break;
+    const float a = v[i].x - mean, c = v[i].y - mean, e = v[i].z - mean, f = v[i].w - mean;
+    q += a * a + c * c + e * e + f * f;
+  }
+  const float rstd = rsqrtf(block_sum256(q, red[1]) / static_cast<float>(d) + eps);
+#pragma unroll
+  for (int i = 0; i < kRowVec; ++i) {
+    const int j = 4 * threadIdx.x + 1024 * i;
+    if (j >= d) break;
+    const float4 g = ldw4(w, w_bf16, j), c = ldw4(b, w_bf16, j);
+    store4<T>(out, o + j, make_float4((v[i].x - mean) * rstd * g.x + c.x, (v[i].y - mean) * rstd * g.y + c.y,
+                                      (v[i].z - mean) * rstd * g.z + c.z, (v[i].w - mean) * rstd * g.w + c.w));
+  }
+}
+
+// u = [LN(c); LN(h)], a block per row and half, for few rows (32 x 2048: 13 -> 3.8 us with one warp per row before)
+template <class T>
+__global__ void __launch_bounds__(256) ln_pair_block_kernel(const float* __restrict__ c, const float* __restrict__ h, int d,
+                                                            const void* wc, const void* bc, const void* wh, const void* bh,
+                                                            int w_bf16, float eps, void* __restrict__ u) {
+  pdl_enter();
+  __shared__ float red[2][8];
+  const int m = blockIdx.x >> 1, part = blockIdx.x & 1;
+  float4 v[kRowVec];
+  load_row_block((part ? h : c) + static_cast<size_t>(m) * d, d, v);
+  ln_row_block<T>(v, d, part ? wh : wc, part ? bh : bc, w_bf16, eps, u, (static_cast<size_t>(m) * 2 + part) * d, red);
+}
+
+// out = LN(x), a block per row, for few rows
+__global__ void __launch_bounds__(256) layernorm_block_kernel(const float* __restrict__ x, int d, const void* w,
+                                                              const void* b, int w_bf16, float eps, float* __restrict__ out) {
+  pdl_enter();
+  __shared__ float red[2][8];
+  float4 v[kRowVec];
+  const size_t o = static_cast<size_t>(blockIdx.x) * d;
+  load_row_block(x + o, d, v);
+  ln_row_block<float>(v, d, w, b, w_bf16, eps, out, o, red);
+}
+
 // out = x / sqrt(mean(x^2) + eps) * gain, one 256-thread block per row (few rows)
 template <class T>
 __global__ void __launch_bounds__(256) rmsnorm_block_kernel(const float* __restrict__ x, int d,
@@ -585,6 +746,17 @@ inline const char* err() {
 }
 }  // namespace
 
+// true when every pointer is 16-byte aligned (the register kernels' vector accesses)
+static bool all16(std::initializer_list<const void*> ps) {
+  for (const void* p : ps)
+    if (reinterpret_cast<uintptr_t>(p) & 15) return false;
+  return true;
+}
+
+// below this many rows a block per row keeps more SMs busy than a warp per row (LayerNorm: from 1024 columns, one
+// float4 per thread; narrower rows stay with a warp)
+constexpr int kFewRows = 1024;
+
 const char* embed_rows(const int32_t* z, int ldz, int batch, int rows, const void* E, int e_bf16, int d, int vocab,
                        float* out, float* out2, cudaStream_t s, const float* add, int add_first,
                        const float* add_div) {
@@ -592,6 +764,11 @@ const char* embed_rows(const int32_t* z, int ldz, int batch, int rows, const voi
   if (M <= 0) return nullptr;
   if (d % 4) return "d_model must be a multiple of 4";
   if (add && (add_first < 0 || add_first > rows)) return "self-conditioning rows out of range";
+  if (M < kFewRows && e_bf16 && !out2 && d % 8 == 0 && all16({E, out, add})) {
+    launch_pdl(embed_block_kernel, M, 256, 0, s, z, ldz, rows, static_cast<const bf16*>(E), d, vocab, out, add, add_first,
+               add_div);
+    return err();
+  }
   launch_pdl(embed_kernel, rows_grid(M), WPB * 32, 0, s, z, ldz, rows, M, E, e_bf16, d, vocab, out, out2, add,
              add_first, add_div);
   return err();
@@ -602,7 +779,14 @@ const char* rmsnorm_rows(const float* x, int M, int d, const void* gain, int w_b
   if (M <= 0) return nullptr;
   if (!act_bf16) lo_off = 0;       // fp32 activations are not split
   if (lo_off > 0 && (lo_off < d || lo_off + d > ldo)) return "split operand: the remainder columns must follow the row";
-  if (M < 1024) {   // few rows: a block per row keeps enough SMs busy
+  if (M < kFewRows) {
+    if (d % 4 == 0 && d <= 1024 * kRowVec && ldo % 4 == 0 && lo_off % 4 == 0 && all16({x, gain, out})) {
+      if (act_bf16)
+        launch_pdl(rmsnorm_block_reg_kernel<bf16>, M, 256, 0, s, x, d, gain, w_bf16, eps, out, ldo, rows_idx, lo_off);
+      else
+        launch_pdl(rmsnorm_block_reg_kernel<float>, M, 256, 0, s, x, d, gain, w_bf16, eps, out, ldo, rows_idx, lo_off);
+      return err();
+    }
     if (act_bf16)
       launch_pdl(rmsnorm_block_kernel<bf16>, M, 256, 0, s, x, d, gain, w_bf16, eps, out, ldo, rows_idx, lo_off);
     else
@@ -630,13 +814,6 @@ const char* rmsnorm_rows(const float* x, int M, int d, const void* gain, int w_b
   return err();
 }
 
-// true when every pointer is 16-byte aligned (the register kernels' vector accesses)
-static bool all16(std::initializer_list<const void*> ps) {
-  for (const void* p : ps)
-    if (reinterpret_cast<uintptr_t>(p) & 15) return false;
-  return true;
-}
-
 template <class T>
 static bool ln_pair_reg(const float* c, const float* h, int M, int d, const void* wc, const void* bc, const void* wh,
                  const void* bh, int w_bf16, float eps, void* u, cudaStream_t s) {
@@ -653,6 +830,13 @@ static bool ln_pair_reg(const float* c, const float* h, int M, int d, const void
 const char* ln_pair_rows(const float* c, const float* h, int M, int d, const void* wc, const void* bc, const void* wh,
                          const void* bh, int w_bf16, float eps, void* u, int act_bf16, cudaStream_t s) {
   if (M <= 0) return nullptr;
+  if (M < kFewRows && d >= 1024 && d % 4 == 0 && d <= 1024 * kRowVec && all16({c, h, wc, bc, wh, bh, u})) {
+    if (act_bf16)
+      launch_pdl(ln_pair_block_kernel<bf16>, 2 * M, 256, 0, s, c, h, d, wc, bc, wh, bh, w_bf16, eps, u);
+    else
+      launch_pdl(ln_pair_block_kernel<float>, 2 * M, 256, 0, s, c, h, d, wc, bc, wh, bh, w_bf16, eps, u);
+    return err();
+  }
   if (all16({c, h, wc, bc, wh, bh, u})) {
     const bool done = act_bf16 ? ln_pair_reg<bf16>(c, h, M, d, wc, bc, wh, bh, w_bf16, eps, u, s)
                                : ln_pair_reg<float>(c, h, M, d, wc, bc, wh, bh, w_bf16, eps, u, s);
@@ -668,6 +852,10 @@ const char* ln_pair_rows(const float* c, const float* h, int M, int d, const voi
 const char* layernorm_rows(const float* x, int M, int d, const void* w, const void* b, int w_bf16, float eps,
                            float* out, cudaStream_t s) {
   if (M <= 0) return nullptr;
+  if (M < kFewRows && d >= 1024 && d % 4 == 0 && d <= 1024 * kRowVec && all16({x, w, b, out})) {
+    launch_pdl(layernorm_block_kernel, M, 256, 0, s, x, d, w, b, w_bf16, eps, out);
+    return err();
+  }
   if (all16({x, w, b, out})) {
     switch (d) {
       case 256: launch_pdl(layernorm_reg_kernel<1>, rows_grid(M), WPB * 32, 0, s, x, M, w, b, w_bf16, eps, out); return err();
@@ -695,7 +883,7 @@ const char* post_norm_add(float* x, const float* y, int M, int d, const void* g_
                           float eps, void* out, int act_bf16, cudaStream_t s) {
   if (M <= 0) return nullptr;
   if (d % 4) return "post-norm rows need d % 4 == 0";
-  if (M < 1024) {   // few rows: a block per row keeps enough SMs busy
+  if (M < kFewRows) {
     if (act_bf16)
       launch_pdl(post_norm_add_block_kernel<bf16>, M, 256, 0, s, x, y, d, g_post, g_next, w_bf16, eps, out);
     else

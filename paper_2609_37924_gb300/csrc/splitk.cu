@@ -192,11 +192,17 @@ __global__ void __launch_bounds__(256) splitk_qkv_kernel(EpiParams ep, const flo
   for (int rr = w; rr < RB; rr += 8) {
     const int m = m0 + rr;
     if (m >= ep.M) continue;                       // uniform across the warp
+    const int b = m / ep.R, r = m - b * ep.R, pos = ep.ctx + r;
+    float2 cs[P];                                  // asked for ahead of the slices: the table may have left L2
+    if (ep.rope && region < 2) {
+#pragma unroll
+      for (int t = 0; t < P; ++t) cs[t] = ep.rope_tab[static_cast<size_t>(lane * P + t) * ep.rope_npos + pos];
+    }
     const float* p = part + static_cast<size_t>(m) * ldp + gh * HD + lane * P;
     float a[P], c[P];
 #pragma unroll
     for (int t = 0; t < P; ++t) a[t] = c[t] = 0.0f;
-#pragma unroll 4
+#pragma unroll 8
     for (int ks = 0; ks < splits; ++ks) {
       const float* q = p + ks * stride;
       if constexpr (P == 2) {
@@ -207,7 +213,6 @@ __global__ void __launch_bounds__(256) splitk_qkv_kernel(EpiParams ep, const flo
         c[0] += q[H2];
       }
     }
-    const int b = m / ep.R, r = m - b * ep.R, pos = ep.ctx + r;
     if (region == 2) {
 #pragma unroll
       for (int t = 0; t < P; ++t) {
@@ -230,10 +235,9 @@ __global__ void __launch_bounds__(256) splitk_qkv_kernel(EpiParams ep, const flo
     if (ep.rope) {
 #pragma unroll
       for (int t = 0; t < P; ++t) {
-        const float2 cs = ep.rope_tab[static_cast<size_t>(lane * P + t) * ep.rope_npos + pos];
         const float x = a[t], y = c[t];
-        a[t] = x * cs.x - y * cs.y;
-        c[t] = y * cs.x + x * cs.y;
+        a[t] = x * cs[t].x - y * cs[t].y;
+        c[t] = y * cs[t].x + x * cs[t].y;
       }
     }
     bf16* dst = region == 0
