@@ -719,6 +719,8 @@ __global__ void __launch_bounds__(192, AttnDbCfg<HD_>::MIN_BLOCKS)
   }
 }
 
+constexpr int kMaxSplits = 8;   // key ranges of one launch
+
 // Merges the split partials of one virtual row per warp, in split order:
 // m* = max m_s, O = sum 2^(m_s - m*) O_s / sum 2^(m_s - m*) l_s.
 template <int HD>
@@ -732,21 +734,35 @@ __global__ void __launch_bounds__(256) attn_combine_kernel(const float* __restri
   const int g = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (g >= n_bk * n_virt) return;
   const size_t stride = static_cast<size_t>(n_bk) * n_virt;
+  // every split's pair and row are asked for at once (splits <= kMaxSplits): the merge is one latency
+  float2 ml[kMaxSplits];
+  float src[kMaxSplits][PL];
+#pragma unroll
+  for (int s = 0; s < kMaxSplits; ++s) {
+    ml[s] = s < splits ? part_ml[s * stride + g] : make_float2(-INFINITY, 0.0f);
+    const float* p = part_o + ((s < splits ? s : 0) * stride + g) * HD + lane * PL;
+    if constexpr (PL == 4) {
+      const float4 t = *reinterpret_cast<const float4*>(p);
+      src[s][0] = t.x, src[s][1] = t.y, src[s][2] = t.z, src[s][3] = t.w;
+    } else {
+      const float2 t = *reinterpret_cast<const float2*>(p);
+      src[s][0] = t.x, src[s][1] = t.y;
+    }
+  }
   float mx = -INFINITY;
-  for (int s = 0; s < splits; ++s) mx = fmaxf(mx, part_ml[s * stride + g].x);
+#pragma unroll
+  for (int s = 0; s < kMaxSplits; ++s) mx = fmaxf(mx, ml[s].x);
   float acc[PL];
 #pragma unroll
   for (int k = 0; k < PL; ++k) acc[k] = 0.0f;
   float L = 0.0f;
-  if (mx != -INFINITY) {
-    for (int s = 0; s < splits; ++s) {
-      const float2 ml = part_ml[s * stride + g];
-      const float w = ml.x == -INFINITY ? 0.0f : ex2_approx(ml.x - mx);
-      L = fmaf(w, ml.y, L);
-      const float* src = part_o + (s * stride + g) * HD + lane * PL;
 #pragma unroll
-      for (int k = 0; k < PL; ++k) acc[k] = fmaf(w, src[k], acc[k]);
-    }
+  for (int s = 0; s < kMaxSplits; ++s) {
+    if (ml[s].x == -INFINITY) continue;             // no key of this split
+    const float w = ex2_approx(ml[s].x - mx);
+    L = fmaf(w, ml[s].y, L);
+#pragma unroll
+    for (int k = 0; k < PL; ++k) acc[k] = fmaf(w, src[s][k], acc[k]);
   }
   const float inv = L > 0.0f ? 1.0f / L : 0.0f;
   const int bk = g / n_virt, v = g - bk * n_virt;
@@ -821,7 +837,7 @@ const char* launch_tc_win(const AttnCall& a, cudaStream_t s) {
   if (a.part && a.part_bytes > 0 && !WIN) {
     const int slots = C::MIN_BLOCKS * n_sms;
     const size_t per_split = static_cast<size_t>(a.batch) * a.n_kv_heads * n_virt * (HD + 2) * sizeof(float);
-    splits = std::min(std::min(slots / base, kv_tiles / 3), 8);
+    splits = std::min(std::min(slots / base, kv_tiles / 3), kMaxSplits);
     while (splits > 1 && static_cast<size_t>(splits) * per_split > a.part_bytes) --splits;
     if (splits < 1) splits = 1;
   }

@@ -772,7 +772,7 @@ const char* gemm_tc(const GemmCall& g, cudaStream_t s) {
   // weight-streaming block steps) use 256 x 128 pair tiles instead.
   const int m_pairs = (g.M + 2 * BM - 1) / (2 * BM);
   const bool pair_ok = g_pair_mma && g.M > BM;
-  const bool narrow_kind = g.epi == EPI_RESID || g.epi == EPI_FUSION2 || (g.epi == EPI_QKV && 128 % g.ep.head_dim == 0);
+  const bool narrow_kind = g.epi == EPI_RESID || g.epi == EPI_FUSION2 || g.epi == EPI_PA_UP || (g.epi == EPI_QKV && 128 % g.ep.head_dim == 0);
   const bool narrow = pair_ok && narrow_kind && m_pairs * a.n_tiles_n * 4 <= g_num_sms;
   const int pair_units = narrow ? m_pairs * ((g.N + 127) / 128) : m_pairs * a.n_tiles_n;
   // pairs must keep >= 40% of the SMs busy to beat split-K; for the residual-add and fp32-store epilogues,
@@ -840,8 +840,12 @@ const char* gemm_tc(const GemmCall& g, cudaStream_t s) {
       return nullptr;
     }
   }
-  if (g.split_buf && !g.m_dev && !pairs_fill && tiles * 3 < g_num_sms * 2 && kblocks >= 8) {
-    int sp = std::min(std::min(g_num_sms / tiles, kblocks / 4), 16);
+  // the few-tile GEMMs of the paired-attention mixer (256 x 256 x 256: one or
+  // two CTAs, whose epilogue then walks the whole tile) split down to two
+  // k-blocks per slice: the reduction spreads the epilogue over the SMs
+  const int min_kb = tiles * 8 <= g_num_sms && (g.epi == EPI_ADD || g.epi == EPI_SILU || g.epi == EPI_PA_GATE) ? 2 : 4;
+  if (g.split_buf && !g.m_dev && !pairs_fill && tiles * 3 < g_num_sms * 2 && kblocks >= 2 * min_kb) {
+    int sp = std::min(std::min(g_num_sms / tiles, kblocks / min_kb), 16);
     const size_t per = static_cast<size_t>(g.M) * a.ldp * sizeof(float);
     while (sp > 1 && sp * per > g.split_bytes) --sp;
     if (sp > 1) {
@@ -862,6 +866,7 @@ const char* gemm_tc(const GemmCall& g, cudaStream_t s) {
     a2.n_tiles_n = (g.N + 127) / 128;
     cudaError_t e = g.epi == EPI_RESID  ? launch_epi_pair<EPI_RESID, 128>(ta, tbh, tc, tc2, a2, pair_units, s)
                     : g.epi == EPI_QKV  ? launch_epi_pair<EPI_QKV, 128>(ta, tbh, tc, tc2, a2, pair_units, s)
+                    : g.epi == EPI_PA_UP ? launch_epi_pair<EPI_PA_UP, 128>(ta, tbh, tc, tc2, a2, pair_units, s)
                                         : launch_epi_pair<EPI_FUSION2, 128>(ta, tbh, tc, tc2, a2, pair_units, s);
     if (e != cudaSuccess) return cudaGetErrorString(e);
     const_cast<GemmCall&>(g).launched = 1;

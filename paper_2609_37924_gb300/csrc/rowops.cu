@@ -95,11 +95,12 @@ __global__ void embed_kernel(const int32_t* __restrict__ z, int ldz, int rows, i
 
 // embed_kernel with a 256-thread block per row, for few rows (32 x 2048: 10 ->
 // 6 us with the copy behind it): eight bf16 (16 bytes) per thread and step.  d % 8 == 0, 16-byte
-// aligned bf16 table, out and add; no second output.
+// aligned bf16 table, outputs and add.
 __global__ void __launch_bounds__(256) embed_block_kernel(const int32_t* __restrict__ z, int ldz, int rows,
                                                           const bf16* __restrict__ E, int d, int vocab,
-                                                          float* __restrict__ out, const float* __restrict__ add,
-                                                          int add_first, const float* __restrict__ add_div) {
+                                                          float* __restrict__ out, float* __restrict__ out2,
+                                                          const float* __restrict__ add, int add_first,
+                                                          const float* __restrict__ add_div) {
   pdl_enter();
   const int m = blockIdx.x, b = m / rows, r = m - b * rows;
   int tok = z[static_cast<size_t>(b) * ldz + r];
@@ -125,6 +126,7 @@ __global__ void __launch_bounds__(256) embed_block_kernel(const int32_t* __restr
         v[q].w = fmaf(t.w, sc, v[q].w);
       }
       *reinterpret_cast<float4*>(o + j + 4 * q) = v[q];
+      if (out2) *reinterpret_cast<float4*>(out2 + static_cast<size_t>(m) * d + j + 4 * q) = v[q];
     }
   }
 }
@@ -764,9 +766,9 @@ const char* embed_rows(const int32_t* z, int ldz, int batch, int rows, const voi
   if (M <= 0) return nullptr;
   if (d % 4) return "d_model must be a multiple of 4";
   if (add && (add_first < 0 || add_first > rows)) return "self-conditioning rows out of range";
-  if (M < kFewRows && e_bf16 && !out2 && d % 8 == 0 && all16({E, out, add})) {
-    launch_pdl(embed_block_kernel, M, 256, 0, s, z, ldz, rows, static_cast<const bf16*>(E), d, vocab, out, add, add_first,
-               add_div);
+  if (M < kFewRows && e_bf16 && d % 8 == 0 && all16({E, out, out2, add})) {
+    launch_pdl(embed_block_kernel, M, 256, 0, s, z, ldz, rows, static_cast<const bf16*>(E), d, vocab, out, out2, add,
+               add_first, add_div);
     return err();
   }
   launch_pdl(embed_kernel, rows_grid(M), WPB * 32, 0, s, z, ldz, rows, M, E, e_bf16, d, vocab, out, out2, add,

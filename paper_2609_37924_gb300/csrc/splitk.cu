@@ -171,16 +171,15 @@ bool elem_ok(int epi, const EpiParams& ep, int ldp) {
   }
 }
 
-// QKV epilogue on the slice sums: a block takes 16 rows of one head, a warp
-// two of them; a lane holds the rotate-half pairs (i, i + HD / 2) of HD / 64
+// QKV epilogue on the slice sums: a block takes 8 rows of one head, one per
+// warp; a lane holds the rotate-half pairs (i, i + HD / 2) of HD / 64
 // consecutive dims i, so partials, Q and K move in whole lines.  V rows cross
-// shared memory and leave transposed, 16 positions (one 32-byte sector) of a
-// dim at a time.
+// shared memory and leave transposed, 8 positions of a dim at a time.
 template <int HD>
 __global__ void __launch_bounds__(256) splitk_qkv_kernel(EpiParams ep, const float* __restrict__ part, size_t stride,
                                                          int ldp, int splits) {
   pdl_enter();
-  constexpr int P = HD / 64, H2 = HD / 2, RB = 16;
+  constexpr int P = HD / 64, H2 = HD / 2, RB = 8;
   __shared__ bf16 sv[HD][RB + 2];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int gh = blockIdx.y, m0 = blockIdx.x * RB;
@@ -284,7 +283,7 @@ cudaError_t launch(const EpiParams& ep, const float* part, size_t stride, int ld
   if constexpr (EPI == EPI_QKV) {
     if (ep.out_bf16 && (ep.head_dim == 64 || ep.head_dim == 128)) {
       *launches = 1;
-      const dim3 grid((ep.M + 15) / 16, ep.n_heads + 2 * ep.n_kv_heads);
+      const dim3 grid((ep.M + 7) / 8, ep.n_heads + 2 * ep.n_kv_heads);
       if (ep.head_dim == 64) launch_pdl(splitk_qkv_kernel<64>, grid, 256, 0, s, ep, part, stride, ldp, splits);
       else launch_pdl(splitk_qkv_kernel<128>, grid, 256, 0, s, ep, part, stride, ldp, splits);
       return cudaGetLastError();

@@ -458,13 +458,19 @@ tadm_status stack_fwd(tadm_handle* h, int first, int n, float* x, int B, int R, 
 // S: c = embed(z) then L_S layers (c lives in the workspace).
 // `add` (optional): the self-conditioning signal of rows add_first .. R-1 of
 // each sequence, fp32 [B * (R - add_first), d], added to their embedding
-// (divided by add_div[row] when add_div is given).
+// (divided by add_div[row] when add_div is given).  copy (optional): also
+// receives c, from the embedding itself when S has no layers (run_A's input).
 tadm_status run_S(tadm_handle* h, const int32_t* z, int ldz, int B, int R, int causal, cudaStream_t s,
-                  const float* add = nullptr, int add_first = 0, const float* add_div = nullptr) {
+                  const float* add = nullptr, int add_first = 0, const float* add_div = nullptr, float* copy = nullptr) {
   const tadm_config& c = h->cfg;
   float* cbuf = h->at<float>(h->off.c);
-  TRY(embed_rows(z, ldz, B, R, h->embed, c.dtype, c.d_model, c.vocab, cbuf, nullptr, s, add, add_first, add_div));
-  return stack_fwd(h, 0, c.n_shared, cbuf, B, R, h->ctx, causal, s);
+  TRY(embed_rows(z, ldz, B, R, h->embed, c.dtype, c.d_model, c.vocab, cbuf, c.n_shared == 0 ? copy : nullptr, s, add,
+                 add_first, add_div));
+  TRYS(stack_fwd(h, 0, c.n_shared, cbuf, B, R, h->ctx, causal, s));
+  if (copy && c.n_shared > 0 &&
+      cudaMemcpyAsync(copy, cbuf, static_cast<size_t>(B) * R * c.d_model * 4, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
+    return fail(h, TADM_ERR_CUDA, "copy c -> h failed");
+  return TADM_OK;
 }
 
 // Mixer phi(Z, U) of the paired-attention fusion (App. C.1); writes phi (fp32 [M, r]).
@@ -527,14 +533,13 @@ tadm_status project_scaled(tadm_handle* h, const float* X, float* sc, bool fresh
   return gemm(h, norm, Mmax, c.d_model, W, c.d_model, M, c.fusion_rank, c.d_model, EPI_STORE, e, s, true);
 }
 
-// A: h = A(c) into the cache (plus the refresh-only quantities of App. C.1).
+// A: h = A(c) in place in the cache, where run_S left a copy of c (plus the
+// refresh-only quantities of App. C.1).
 tadm_status run_A(tadm_handle* h, int B, int R, int causal, void* cache, cudaStream_t s) {
   const tadm_config& c = h->cfg;
   const int M = B * R;
   CacheView cv = cache_view(c, cache, B, R);
   const float* cbuf = h->at<float>(h->off.c);
-  if (cudaMemcpyAsync(cv.h, cbuf, static_cast<size_t>(M) * c.d_model * 4, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-    return fail(h, TADM_ERR_CUDA, "copy c -> h failed");
   TRYS(stack_fwd(h, c.n_shared, c.n_anchor, cv.h, B, R, h->ctx, causal, s));
   if (c.fusion == 1) {
     // s_C, s_H, Z0 = (C0/s_C) W_C, U = (H0/s_H) W_H, phi(Z0, U)
@@ -653,7 +658,7 @@ tadm_status fresh_pass(tadm_handle* h, const int32_t* z, int ldz, int B, int R, 
   const tadm_config& c = h->cfg;
   if (h->max_ctx <= 0) return fail(h, TADM_ERR_STATE, "handle was created without KV context (max_ctx = 0)");
   if (h->ctx + R > h->max_ctx) return fail(h, TADM_ERR_STATE, "context full: %d + %d > %d", h->ctx, R, h->max_ctx);
-  TRYS(run_S(h, z, ldz, B, R, 1, s));
+  TRYS(run_S(h, z, ldz, B, R, 1, s, nullptr, 0, nullptr, h->at<float>(h->off.h_int)));
   void* cache = h->at(h->off.h_int);
   TRYS(run_A(h, B, R, 1, cache, s));
   if (c.fusion == 1) {
@@ -1016,7 +1021,7 @@ tadm_status tadm_anchor_forward(tadm_handle* h, const int32_t* x_t, int batch, i
   TRYS(check_ready(h, batch, rows));
   if (!x_t || !h_cache) return fail(h, TADM_ERR_INVALID_ARG, "NULL pointer");
   h->last_stream = stream;
-  TRYS(run_S(h, x_t, rows, batch, rows, 0, stream));
+  TRYS(run_S(h, x_t, rows, batch, rows, 0, stream, nullptr, 0, nullptr, static_cast<float*>(h_cache)));
   TRYS(run_A(h, batch, rows, 0, h_cache, stream));
   h->counters.anchor_layers += h->cfg.n_anchor;
   h->counters.anchor_calls += 1;
@@ -1142,7 +1147,7 @@ tadm_status generate_loop(tadm_handle* h, const int32_t* prompt, int batch, int 
         TRYS(fresh_pass(h, out, total, batch, prompt_len, s));
         break;
       case 1:  // anchor refresh: h_cache <- A(S(z))
-        TRYS(run_S(h, z, total, batch, R, 0, s));
+        TRYS(run_S(h, z, total, batch, R, 0, s, nullptr, 0, nullptr, static_cast<float*>(cache)));
         TRYS(run_A(h, batch, R, 0, cache, s));
         h->counters.anchor_layers += c.n_anchor;
         h->counters.anchor_calls += 1;
@@ -1313,7 +1318,7 @@ tadm_status tadm_generate_remdm(tadm_handle* h, const int32_t* prompt, int batch
   TRY(fill_canvas(out, total, prompt, batch, prompt_len, total, mask, s));
   void* cache = h->at(h->off.h_int);
   for (int n = 0; n < steps; ++n) {
-    TRYS(run_S(h, out, total, batch, R, 0, s));
+    TRYS(run_S(h, out, total, batch, R, 0, s, nullptr, 0, nullptr, n % K == 0 ? static_cast<float*>(cache) : nullptr));
     if (n % K == 0) {                          // Alg. 1 refresh test (T - i) mod K = 0
       TRYS(run_A(h, batch, R, 0, cache, s));
       h->counters.anchor_layers += c.n_anchor;
@@ -1457,7 +1462,8 @@ tadm_status tadm_generate_entropy_bound(tadm_handle* h, const int32_t* prompt, i
   void* cache = h->at(h->off.h_int);
   for (int i = 0; i < steps; ++i) {
     const int n = steps - i;                      // Alg. 2's n = T .. 1
-    TRYS(run_S(h, out, total, batch, R, 0, s, self_cond && i > 0 ? sig : nullptr, prompt_len, zs));
+    TRYS(run_S(h, out, total, batch, R, 0, s, self_cond && i > 0 ? sig : nullptr, prompt_len, zs,
+               i % K == 0 ? static_cast<float*>(cache) : nullptr));
     if (i % K == 0) {                             // Alg. 1 refresh test (T - i) mod K = 0
       TRYS(run_A(h, batch, R, 0, cache, s));
       h->counters.anchor_layers += c.n_anchor;
