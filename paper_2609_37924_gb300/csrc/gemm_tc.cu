@@ -141,6 +141,7 @@ struct TcArgs {
   int part_tma;            // split-K partials go through them too (tmC: the 3-D map [splits][M][ldp])
   int b_split;             // >0: B tile = 128 rows at n*128 and 128 rows at b_split + n*128
   int n_tiles_n;
+  int m_fast;              // tile = n * (row blocks) + m instead of m * n_tiles_n + n
   int kb_wrap;             // > 0: split hi + lo operand of kb_wrap k-blocks per half: k-block kb reads A's
                            // k-block (kb odd ? kb_wrap : 0) + kb / 2 and B's k-block kb / 2, so that the two
                            // reads of a B tile follow each other (the second one hits L2)
@@ -150,8 +151,12 @@ struct TcArgs {
   EpiParams ep;
 };
 
-// Tiles run N-fastest: the CTAs in flight share A tiles (activations, the
-// large operand) through L2, and every weight matrix of the model fits in L2.
+// Tile order (m_fast): the CTAs in flight share the tiles of the larger operand
+// through L2, so that it is read from HBM once.  Activations larger than the
+// weights (whole canvases): N-fastest.  Weights larger than the activations
+// (few rows, the output head): M-fastest; N-fastest read the 524 MB head of the
+// block model once per 256 rows (1500 x 2048 x 128000: 648 -> 547 us; a layer of 1024-row block steps 174 ->
+// 169 us).
 // While the MMA warp fills an accumulator, its epilogue warps ask L2 for the
 // fp32 rows that their epilogue will read (h, base): each lane its own row's
 // share of the tile's columns, so the epilogue does not wait on DRAM latency.
@@ -161,6 +166,16 @@ struct TcArgs {
 // 83).  The residual epilogue needs no prefetch: its TMA reduce-adds are
 // performed at L2 and nothing waits for them (with one from the epilogue
 // lanes the layers are 0.7 % slower).
+__device__ __forceinline__ void tile_coords(const TcArgs& a, int tile, int num_m, int& nb, int& mb) {
+  if (a.m_fast) {
+    nb = tile / num_m;
+    mb = tile - nb * num_m;
+  } else {
+    mb = tile / a.n_tiles_n;
+    nb = tile - mb * a.n_tiles_n;
+  }
+}
+
 template <int EPI>
 __device__ __forceinline__ void prefetch_epilogue_inputs(const TcArgs& a, int m, int nb, int part, int nsplit,
                                                          int ncols = BN) {
@@ -233,9 +248,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   if (args.b_early && warp == 0 && lane == 0) {
     const int tile = blockIdx.x / args.splits, kb0 = (blockIdx.x % args.splits) * args.kb_per_split;
     pre = min(STAGES, min(kblocks, kb0 + args.kb_per_split) - kb0);
+    int nb, mb;
+    tile_coords(args, tile, (args.M + BM - 1) / BM, nb, mb);
     for (int s = 0; s < pre; ++s) {
       mbar_arrive_expect_tx(&full[s], STAGE_BYTES);
-      load_b(s, kb0 + s, tile % args.n_tiles_n);
+      load_b(s, kb0 + s, nb);
     }
   }
   pdl_enter();
@@ -254,7 +271,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       for (int s = 0; s < STAGES; ++s) issued[s] = 0;
       for (int unit = blockIdx.x; unit < units && !*abort_flag; unit += gridDim.x) {
         const int tile = unit / args.splits, ks = unit % args.splits;
-        const int nb = tile % args.n_tiles_n, mb = tile / args.n_tiles_n;
+        int nb, mb;
+        tile_coords(args, tile, num_m, nb, mb);
         const int kb0 = ks * args.kb_per_split, kb1 = min(kblocks, kb0 + args.kb_per_split);
         bool ok = true;
         for (int kb = kb0; kb < kb1; ++kb) {
@@ -322,7 +340,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     uint32_t acc_phase = 0;
     for (int unit = blockIdx.x; unit < units; unit += gridDim.x) {
       const int tile = unit / args.splits, ks = unit % args.splits;
-      const int nb = tile % args.n_tiles_n, mb = tile / args.n_tiles_n;
+      int nb, mb;
+      tile_coords(args, tile, num_m, nb, mb);
       if (args.splits == 1 && part < nsplit)
         prefetch_epilogue_inputs<EPI>(args, mb * BM + quad * 32 + lane, nb, part, nsplit);
       if (!warp_wait_bounded(&tfull[acc], acc_phase, abort_flag, args.status)) break;
@@ -450,9 +469,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   if (args.b_early && warp == 0 && lane == 0) {
     const int tile = u0 / args.splits, kb0 = (u0 % args.splits) * args.kb_per_split;
     pre = min(P_STAGES, min(kblocks, kb0 + args.kb_per_split) - kb0);
+    int nb, mb2;
+    tile_coords(args, tile, (args.M + 2 * BM - 1) / (2 * BM), nb, mb2);
     for (int s = 0; s < pre; ++s) {
       if (leader) mbar_arrive_expect_tx(&full[s], 2 * P_STAGE_BYTES);
-      load_b(s, kb0 + s, tile % args.n_tiles_n);
+      load_b(s, kb0 + s, nb);
     }
   }
   pdl_enter();
@@ -468,8 +489,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       uint32_t phase = 0;
       for (int unit = u0; unit < units && !*abort_flag; unit += ustep) {
         const int tile = unit / args.splits, ks = unit % args.splits;
-        const int nb = tile % args.n_tiles_n;
-        const int mb = 2 * (tile / args.n_tiles_n) + static_cast<int>(rank);   // this CTA's 128-row block
+        int nb, mb2;
+        tile_coords(args, tile, num_m2, nb, mb2);
+        const int mb = 2 * mb2 + static_cast<int>(rank);   // this CTA's 128-row block
         const int kb0 = ks * args.kb_per_split, kb1 = min(kblocks, kb0 + args.kb_per_split);
         bool ok = true;
         for (int kb = kb0; kb < kb1; ++kb) {
@@ -540,8 +562,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
     uint32_t acc_phase = 0;
     for (int unit = u0; unit < units; unit += ustep) {
       const int tile = unit / args.splits, ks = unit % args.splits;
-      const int nb = tile % args.n_tiles_n;
-      const int mb = 2 * (tile / args.n_tiles_n) + static_cast<int>(rank);
+      int nb, mb2;
+      tile_coords(args, tile, num_m2, nb, mb2);
+      const int mb = 2 * mb2 + static_cast<int>(rank);
       if (args.splits == 1 && part < nsplit)
         prefetch_epilogue_inputs<EPI>(args, mb * BM + quad * 32 + lane, nb, part, nsplit, PBN);
       if (!warp_wait_bounded(&tfull[acc], acc_phase, abort_flag, args.status)) break;
@@ -719,6 +742,7 @@ const char* gemm_tc(const GemmCall& g, cudaStream_t s) {
   a.b_split = glu ? g.N : 0;
   a.n_tiles_n = glu ? (g.N + BN / 2 - 1) / (BN / 2) : (g.N + BN - 1) / BN;
   a.kb_wrap = g.k_b > 0 ? g.k_b / BK : 0;
+  a.m_fast = b_rows * k_b > static_cast<int64_t>(g.M) * g.K;
   if (glu && g.N % (BN / 2)) return "GLU GEMM needs the FFN width to be a multiple of 128";
   if (g.epi == EPI_QKV && BN % g.ep.head_dim) return "head_dim must divide 256";
   if (g.epi == EPI_PA_GATE && g.N > BN) return "gate GEMM needs N <= 256";
