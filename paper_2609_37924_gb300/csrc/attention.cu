@@ -1125,7 +1125,7 @@ __global__ void __launch_bounds__(128) attn_bf16_kernel(const bf16* __restrict__
 // contiguous in the dimension their product runs over); thread (ty, tx) owns
 // rows ty and ty + 8 and keys (then dims) tx + 16 j, so every float4 read
 // feeds four FMAs per partner row.  The online softmax runs once per tile.
-// 4 x 4 heads x 128 rows, hd 64: 93 -> 15.7 us (one warp per query row, a warp
+// 4 x 4 heads x 128 rows, hd 64: 93 -> 12.6 us (one warp per query row, a warp
 // reduction and two uncoalesced V reads per key).
 constexpr int FQ = 16, FK = 64, FNT = 128;
 
@@ -1283,14 +1283,22 @@ cudaError_t launch_bf16(const AttnCall& a, cudaStream_t s) {
 
 template <int HD>
 cudaError_t launch_f32(const AttnCall& a, cudaStream_t s) {
-  constexpr int smem = F32Cfg<HD>::FLOATS * 4;
-  static bool attr = false;
-  if (!attr) {
-    const cudaError_t e = cudaFuncSetAttribute(attn_f32_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  constexpr int need = F32Cfg<HD>::FLOATS * 4, alone = 120 * 1024;
+  static int n_sms = 0;
+  if (n_sms == 0) {
+    const cudaError_t e = cudaFuncSetAttribute(attn_f32_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               std::max(need, alone));
     if (e != cudaSuccess) return e;
-    attr = true;
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    n_sms = n > 0 ? n : 1;
   }
   dim3 grid((a.rows + FQ - 1) / FQ, a.n_heads, a.batch);
+  // a launch of at most one block per SM asks for more than half of an SM's
+  // shared memory: its blocks start while the predecessor's last ones run and
+  // would otherwise share the first SMs that come free
+  const int smem = static_cast<int64_t>(grid.x) * grid.y * grid.z <= n_sms ? std::max(need, alone) : need;
   const int vec = a.kv_stride % 4 == 0 && ((reinterpret_cast<uintptr_t>(a.k) | reinterpret_cast<uintptr_t>(a.v)) & 15) == 0;
   launch_pdl(attn_f32_kernel<HD>, grid, FNT, smem, s, static_cast<const float*>(a.q), static_cast<const float*>(a.k),
              static_cast<const float*>(a.v), static_cast<float*>(a.o), a.n_heads, a.n_kv_heads, a.rows, a.ctx, a.kv_stride,

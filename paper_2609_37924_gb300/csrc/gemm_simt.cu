@@ -6,21 +6,26 @@
 // tiles would leave SMs idle).  The GEMMs of this path are a few hundred rows
 // by a few hundred columns, so a launch is paced by the latency of one
 // block's K loop, not by FMA throughput: K advances 64 at a time through a
-// three-stage cp.async ring, and the block's four 64-thread groups each take
-// 16 of the 64 columns of every stage (a split of K inside the block); their
-// partial tiles are summed in group order through shared memory.  Weights
-// (b_weights) start loading ahead of the grid dependency.  Rows of the stage
-// are padded to 68 floats: the 8 column (4 row) addresses of a warp's float4
-// reads fall into different banks.
-// 512 rows: the residual projections (N 256, K 256 and 1024) 95 -> 15.6 us a
-// launch, QKV (N 768, K 256) 36 -> 14.8 us, cold caches (before: 64 x 64
-// tiles, 16 columns of K per synchronous step, 32 to 96 blocks).
+// cp.async ring, and the block's thread groups (four of 64 threads, or eight
+// warps for 16-row tiles) each take their share of the 64 columns of every
+// stage for the whole tile (a split of K inside the block; 4 x 8 outputs per
+// thread either way); the partial tiles are summed in group order through
+// shared memory.  Weights (b_weights) start loading ahead of the grid
+// dependency.  Rows of the stage are padded to 68 floats: the eight column
+// addresses of a quarter-warp's float4 reads fall into different banks.
+// 16-row tiles run six stages, one block per SM: a launch that starts while
+// its predecessor's last blocks run otherwise packs three blocks onto the
+// first SMs that come free (W_down of 512 rows took 37 us in a generation and
+// 15 alone).  512 rows in a generation: W_down (N 256, K 1024) 14.4 us, W_o 4.9,
+// QKV (N 768, K 256) 12.4, GLU (N 2 x 1024, K 256) 22, fusion hidden (N 1280, K
+// 512) 38; with 64 x 64 tiles and 16 columns of K per synchronous step the
+// residual projections took 95 us a launch, QKV 36, GLU 38.
 // EPI_GLU tiles hold 32 gate and 32 up columns; EPI_QKV needs head_dim <= 64.
 #include "kernels.h"
 
 namespace tadm {
 namespace {
-constexpr int TN = 64, TK = 64, LDK = TK + 4, STAGES = 3, GROUPS = 4, NT = 64 * GROUPS;
+constexpr int TN = 64, TK = 64, LDK = TK + 4, NT = 256;
 
 struct SmemSrc {
   static constexpr bool kStaged = false;
@@ -43,13 +48,17 @@ template <int N>
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 template <int TM>
-struct SimtCfg { static constexpr int FLOATS = STAGES * (TM + TN) * LDK; };
+struct SimtCfg {
+  static constexpr int STAGES = TM == 16 ? 6 : 3, GROUPS = TM == 16 ? 8 : 4;
+  static constexpr int FLOATS = STAGES * (TM + TN) * LDK;
+};
 
 // VEC: rows of A and B are 16-byte aligned and K % 4 == 0 (16-byte copies); otherwise 4-byte copies.
 template <int EPI, int TM, bool VEC>
-__global__ void __launch_bounds__(NT) gemm_simt_kernel(const float* __restrict__ A, const float* __restrict__ B, int M,
+__global__ void __launch_bounds__(NT, TM == 16 ? 1 : 2) gemm_simt_kernel(const float* __restrict__ A, const float* __restrict__ B, int M,
                                                        int K, int lda, int ldb, int tiles_n, int n_rows_b, int b_split,
                                                        int b_early, EpiParams ep) {
+  constexpr int STAGES = SimtCfg<TM>::STAGES, GROUPS = SimtCfg<TM>::GROUPS, TG = NT / GROUPS, KC = TK / GROUPS;
   extern __shared__ __align__(16) float smem[];
   const int tid = threadIdx.x, m0 = blockIdx.x / tiles_n * TM, nb = blockIdx.x % tiles_n;
   const int ksteps = (K + TK - 1) / TK;
@@ -86,10 +95,10 @@ __global__ void __launch_bounds__(NT) gemm_simt_kernel(const float* __restrict__
     }
     cp_commit();
   }
-  // group g owns columns 16 g .. 16 g + 15 of every stage; within it thread
-  // (ty, tx) owns rows ty + 8 i and columns tx + 8 j of the tile
-  constexpr int RM = TM / 8;
-  const int g = tid / 64, t = tid % 64, ty = t / 8, tx = t % 8;
+  // group g owns columns KC g .. KC g + KC - 1 of every stage; its thread
+  // (ty, tx) owns rows ty + TY i and columns tx + 8 j of the tile
+  constexpr int TY = TG / 8, RM = TM / TY;
+  const int g = tid / TG, t = tid % TG, ty = t / 8, tx = t % 8;
   float acc[RM][8];
 #pragma unroll
   for (int i = 0; i < RM; ++i)
@@ -103,13 +112,14 @@ __global__ void __launch_bounds__(NT) gemm_simt_kernel(const float* __restrict__
       load_a(ks + STAGES - 1);
     }
     cp_commit();
-    const float* a0 = sA + (ks % STAGES) * TM * LDK + ty * LDK + 16 * g;
-    const float* b0 = sB + (ks % STAGES) * TN * LDK + tx * LDK + 16 * g;
+    const float* a0 = sA + (ks % STAGES) * TM * LDK + ty * LDK + KC * g;
+    const float* b0 = sB + (ks % STAGES) * TN * LDK + tx * LDK + KC * g;
 #pragma unroll
-    for (int kk = 0; kk < 16; kk += 4) {
-      float4 a[RM], b[8];
+    for (int kk = 0; kk < KC; kk += 4) {
+      float4 a[RM];
 #pragma unroll
-      for (int i = 0; i < RM; ++i) a[i] = *reinterpret_cast<const float4*>(a0 + 8 * i * LDK + kk);
+      for (int i = 0; i < RM; ++i) a[i] = *reinterpret_cast<const float4*>(a0 + TY * i * LDK + kk);
+      float4 b[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) b[j] = *reinterpret_cast<const float4*>(b0 + 8 * j * LDK + kk);
 #pragma unroll
@@ -132,7 +142,7 @@ __global__ void __launch_bounds__(NT) gemm_simt_kernel(const float* __restrict__
 #pragma unroll
   for (int i = 0; i < RM; ++i)
 #pragma unroll
-    for (int j = 0; j < 8; ++j) sC[g * TILE + (ty + 8 * i) * LDC + tx + 8 * j] = acc[i][j];
+    for (int j = 0; j < 8; ++j) sC[g * TILE + (ty + TY * i) * LDC + tx + 8 * j] = acc[i][j];
   __syncthreads();
   for (int e = tid; e < TM * TN; e += NT) {
     const int o = (e / TN) * LDC + e % TN;
