@@ -206,56 +206,6 @@ __global__ void __launch_bounds__(256) rmsnorm_block_reg_kernel(const float* __r
   }
 }
 
-// LayerNorm of the row in v by its block: mean, then the variance about it, then out[o + j] (+ affine)
-template <class T>
-__device__ __forceinline__ void ln_row_block(const float4 (&v)[kRowVec], int d, const void* w, const void* b, int w_bf16,
-                                             float eps, void* out, size_t o, float (*red)[8]) {
-  float s = 0.0f;
-#pragma unroll
-  for (int i = 0; i < kRowVec; ++i) s += v[i].x + v[i].y + v[i].z + v[i].w;
-  const float mean = block_sum256(s, red[0]) / static_cast<float>(d);
-  float q = 0.0f;
-#pragma unroll
-  for (int i = 0; i < kRowVec; ++i) {
-    if (static_cast<int>(4 * threadIdx.x + 1024 * i) >= d) break;
-    const float a = v[i].x - mean, c = v[i].y - mean, e = v[i].z - mean, f = v[i].w - mean;
-    q += a * a + c * c + e * e + f * f;
-  }
-  const float rstd = rsqrtf(block_sum256(q, red[1]) / static_cast<float>(d) + eps);
-#pragma unroll
-  for (int i = 0; i < kRowVec; ++i) {
-    const int j = 4 * threadIdx.x + 1024 * i;
-    if (j >= d) break;
-    const float4 g = ldw4(w, w_bf16, j), c = ldw4(b, w_bf16, j);
-    store4<T>(out, o + j, make_float4((v[i].x - mean) * rstd * g.x + c.x, (v[i].y - mean) * rstd * g.y + c.y,
-                                      (v[i].z - mean) * rstd * g.z + c.z, (v[i].w - mean) * rstd * g.w + c.w));
-  }
-}
-
-// u = [LN(c); LN(h)], a block per row and half, for few rows (32 x 2048: 13 -> 3.8 us with one warp per row before)
-template <class T>
-__global__ void __launch_bounds__(256) ln_pair_block_kernel(const float* __restrict__ c, const float* __restrict__ h, int d,
-                                                            const void* wc, const void* bc, const void* wh, const void* bh,
-                                                            int w_bf16, float eps, void* __restrict__ u) {
-  pdl_enter();
-  __shared__ float red[2][8];
-  const int m = blockIdx.x >> 1, part = blockIdx.x & 1;
-  float4 v[kRowVec];
-  load_row_block((part ? h : c) + static_cast<size_t>(m) * d, d, v);
-  ln_row_block<T>(v, d, part ? wh : wc, part ? bh : bc, w_bf16, eps, u, (static_cast<size_t>(m) * 2 + part) * d, red);
-}
-
-// out = LN(x), a block per row, for few rows
-__global__ void __launch_bounds__(256) layernorm_block_kernel(const float* __restrict__ x, int d, const void* w,
-                                                              const void* b, int w_bf16, float eps, float* __restrict__ out) {
-  pdl_enter();
-  __shared__ float red[2][8];
-  float4 v[kRowVec];
-  const size_t o = static_cast<size_t>(blockIdx.x) * d;
-  load_row_block(x + o, d, v);
-  ln_row_block<float>(v, d, w, b, w_bf16, eps, out, o, red);
-}
-
 // out = x / sqrt(mean(x^2) + eps) * gain, one 256-thread block per row (few rows)
 template <class T>
 __global__ void __launch_bounds__(256) rmsnorm_block_kernel(const float* __restrict__ x, int d,
@@ -498,6 +448,66 @@ __global__ void __launch_bounds__(WPB * 32) ln_pair_reg_kernel(const float* __re
       store8<T>(u, static_cast<size_t>(m) * 2 * d + part * d + j, y);
     }
   }
+}
+
+// LayerNorm of a row of d = 256 NCH columns by a 256-thread block: every thread
+// loads eight consecutive columns of chunk threadIdx / 32, the row crosses
+// shared memory, and warp 0 takes mean and variance in ln_row_reg's order, so
+// that a row's result does not depend on how many rows the launch has.
+template <class T, int NCH>
+__device__ __forceinline__ void ln_row_block(const float* __restrict__ xr, const void* w, const void* b, int w_bf16,
+                                             float eps, void* out, size_t o) {
+  constexpr int d = 256 * NCH;
+  __shared__ __align__(16) float row[d];
+  __shared__ float stat[2];
+  float v[8], wv[8], bv[8], y[8];
+  const int j = 8 * threadIdx.x;
+  const bool on = j < d;                            // d <= 2048: one chunk per warp
+  if (on) {
+    const float4 a = *reinterpret_cast<const float4*>(xr + j), c = *reinterpret_cast<const float4*>(xr + j + 4);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    v[4] = c.x; v[5] = c.y; v[6] = c.z; v[7] = c.w;
+    *reinterpret_cast<float4*>(row + j) = a;
+    *reinterpret_cast<float4*>(row + j + 4) = c;
+    ldw8(w, w_bf16, j, wv);
+    ldw8(b, w_bf16, j, bv);
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    float r[NCH][8], mean, rstd;
+    ln_row_reg<NCH>(row, threadIdx.x, eps, r, mean, rstd);
+    if (threadIdx.x == 0) {
+      stat[0] = mean;
+      stat[1] = rstd;
+    }
+  }
+  __syncthreads();
+  if (!on) return;
+  const float mean = stat[0], rstd = stat[1];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) y[i] = (v[i] - mean) * rstd * wv[i] + bv[i];
+  store8<T>(out, o + j, y);
+}
+
+// u = [LN(c); LN(h)], a block per row and half, for few rows (32 x 2048: 13 -> 3.8 us with one warp per row before)
+template <class T, int NCH>
+__global__ void __launch_bounds__(256) ln_pair_block_kernel(const float* __restrict__ c, const float* __restrict__ h,
+                                                            const void* wc, const void* bc, const void* wh, const void* bh,
+                                                            int w_bf16, float eps, void* __restrict__ u) {
+  pdl_enter();
+  constexpr int d = 256 * NCH;
+  const int m = blockIdx.x >> 1, part = blockIdx.x & 1;
+  ln_row_block<T, NCH>((part ? h : c) + static_cast<size_t>(m) * d, part ? wh : wc, part ? bh : bc, w_bf16, eps, u,
+                       (static_cast<size_t>(m) * 2 + part) * d);
+}
+
+// out = LN(x), a block per row, for few rows
+template <int NCH>
+__global__ void __launch_bounds__(256) layernorm_block_kernel(const float* __restrict__ x, const void* w, const void* b,
+                                                              int w_bf16, float eps, float* __restrict__ out) {
+  pdl_enter();
+  const size_t o = static_cast<size_t>(blockIdx.x) * 256 * NCH;
+  ln_row_block<float, NCH>(x + o, w, b, w_bf16, eps, out, o);
 }
 
 // layernorm_kernel for d = 256 NCH with the row in registers
@@ -755,8 +765,8 @@ static bool all16(std::initializer_list<const void*> ps) {
   return true;
 }
 
-// below this many rows a block per row keeps more SMs busy than a warp per row (LayerNorm: from 1024 columns, one
-// float4 per thread; narrower rows stay with a warp)
+// below this many rows a block per row keeps more SMs busy than a warp per row (LayerNorm: the widths of the register
+// kernels from 1024 columns; narrower rows leave most of a block idle)
 constexpr int kFewRows = 1024;
 
 const char* embed_rows(const int32_t* z, int ldz, int batch, int rows, const void* E, int e_bf16, int d, int vocab,
@@ -832,11 +842,10 @@ static bool ln_pair_reg(const float* c, const float* h, int M, int d, const void
 const char* ln_pair_rows(const float* c, const float* h, int M, int d, const void* wc, const void* bc, const void* wh,
                          const void* bh, int w_bf16, float eps, void* u, int act_bf16, cudaStream_t s) {
   if (M <= 0) return nullptr;
-  if (M < kFewRows && d >= 1024 && d % 4 == 0 && d <= 1024 * kRowVec && all16({c, h, wc, bc, wh, bh, u})) {
-    if (act_bf16)
-      launch_pdl(ln_pair_block_kernel<bf16>, 2 * M, 256, 0, s, c, h, d, wc, bc, wh, bh, w_bf16, eps, u);
-    else
-      launch_pdl(ln_pair_block_kernel<float>, 2 * M, 256, 0, s, c, h, d, wc, bc, wh, bh, w_bf16, eps, u);
+  if (M < kFewRows && (d == 1024 || d == 2048) && all16({c, h, wc, bc, wh, bh, u})) {
+    auto go = [&](auto k) { launch_pdl(k, 2 * M, 256, 0, s, c, h, wc, bc, wh, bh, w_bf16, eps, u); };
+    if (d == 1024) act_bf16 ? go(ln_pair_block_kernel<bf16, 4>) : go(ln_pair_block_kernel<float, 4>);
+    else act_bf16 ? go(ln_pair_block_kernel<bf16, 8>) : go(ln_pair_block_kernel<float, 8>);
     return err();
   }
   if (all16({c, h, wc, bc, wh, bh, u})) {
@@ -854,8 +863,9 @@ const char* ln_pair_rows(const float* c, const float* h, int M, int d, const voi
 const char* layernorm_rows(const float* x, int M, int d, const void* w, const void* b, int w_bf16, float eps,
                            float* out, cudaStream_t s) {
   if (M <= 0) return nullptr;
-  if (M < kFewRows && d >= 1024 && d % 4 == 0 && d <= 1024 * kRowVec && all16({x, w, b, out})) {
-    launch_pdl(layernorm_block_kernel, M, 256, 0, s, x, d, w, b, w_bf16, eps, out);
+  if (M < kFewRows && (d == 1024 || d == 2048) && all16({x, w, b, out})) {
+    if (d == 1024) launch_pdl(layernorm_block_kernel<4>, M, 256, 0, s, x, w, b, w_bf16, eps, out);
+    else launch_pdl(layernorm_block_kernel<8>, M, 256, 0, s, x, w, b, w_bf16, eps, out);
     return err();
   }
   if (all16({x, w, b, out})) {
