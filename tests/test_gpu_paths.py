@@ -153,3 +153,32 @@ def test_few_row_steps_match_the_oracle(T, hd, fusion, qk_norm, batch, rows):
     rel = np.linalg.norm(logits.cpu().numpy() - ref) / np.linalg.norm(ref)
     assert rel < 1.5e-2, rel          # bf16 operands, two layers and the fusion
     tm.close()
+
+
+# pipelined hd-64 attention (launches of more 128-row tiles than SMs; P in
+# tensor memory): odd row counts, tiles with idle softmax warps, a context,
+# causal limits inside and between key tiles, a KV group of two heads, few keys
+@pytest.mark.parametrize("B,Hq,Hkv,rows,ctx,causal", [(4, 12, 12, 450, 0, False), (7, 12, 12, 129, 40, False),
+                                                      (4, 16, 16, 333, 70, True), (16, 20, 10, 40, 24, False),
+                                                      (3, 16, 8, 500, 131, True), (40, 4, 4, 100, 0, True)])
+def test_attention_pipelined_hd64(T, B, Hq, Hkv, rows, ctx, causal):
+    hd, n = 64, ctx + rows
+    stride = (n + 7) // 8 * 8
+    assert ((Hq // Hkv) * rows + 127) // 128 * Hkv * B > 152
+    g = torch.Generator(device="cuda").manual_seed(rows)
+    q = (2.0 * torch.randn((B, Hq, rows, hd), generator=g, device="cuda")).to(torch.bfloat16)
+    k = torch.randn((B, Hkv, stride, hd), generator=g, device="cuda").to(torch.bfloat16)
+    v = torch.randn((B, Hkv, hd, stride), generator=g, device="cuda").to(torch.bfloat16)
+    o = torch.full((B * rows, Hq * hd), float("nan"), dtype=torch.bfloat16, device="cuda")
+    T.tadm_attention(q, k, v, o, Hq, Hkv, rows, ctx, causal, 1)
+    rep = Hq // Hkv
+    kd, vd = k[:, :, :n].double().repeat_interleave(rep, 1), v[..., :n].double().transpose(2, 3).repeat_interleave(rep, 1)
+    s = q.double() @ kd.transpose(2, 3) / 8.0
+    if causal:
+        pos = ctx + torch.arange(rows, device="cuda")[:, None]
+        s = s.masked_fill(torch.arange(n, device="cuda")[None, :] > pos, -float("inf"))
+    ref = (torch.softmax(s, -1) @ vd).transpose(1, 2).reshape(B * rows, Hq * hd)
+    err = (o.double() - ref).abs()
+    assert torch.isfinite(o.float()).all()
+    # bf16 P (relative 2^-9 each, at most 2^-8 of the largest |V|) and the bf16 result
+    assert (err <= 2.0 ** -8 * ref.abs() + 2.0 ** -8 * v.float().abs().max()).all()
