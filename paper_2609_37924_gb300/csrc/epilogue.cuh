@@ -389,7 +389,8 @@ __device__ __forceinline__ void epilogue_row(const EpiParams& p, int m, int n_bl
     }
   } else if constexpr (EPI == EPI_GLU) {
     const int half = ncols / 2;
-    const int g_lo = part * (half / 32) / nsplit, g_hi = (part + 1) * (half / 32) / nsplit;
+    int g_lo = part * (half / 32) / nsplit;
+    const int g_hi = (part + 1) * (half / 32) / nsplit;
     if constexpr (Src::kStaged) {
       if (src.staged()) {
         float w[32], u[32];
@@ -412,9 +413,10 @@ __device__ __forceinline__ void epilogue_row(const EpiParams& p, int m, int n_bl
 #pragma unroll
             for (int i = 0; i < 32; ++i) w[i] = silu_f(w[i]) * u[i];
           }
-          src.store64(0, n_blk * half + 32 * c, v, w);
+          if (n_blk * half + 32 * c < p.N && src.row0 < p.M) src.store64(0, n_blk * half + 32 * c, v, w);
         }
-        return;
+        if (((g_hi - g_lo) & 1) == 0) return;
+        g_lo = g_hi - 1;   // an odd chunk left (192-wide tiles): row stores
       }
     }
     for (int c = g_lo; c < g_hi; ++c) {

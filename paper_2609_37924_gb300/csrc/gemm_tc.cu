@@ -392,13 +392,14 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 // bytes); the MMA thread's commits release empty[s] and signal tfull[a] in
 // both CTAs; every epilogue warp of both CTAs releases an accumulator on the
 // even CTA's tempty[a].
-// PBN: columns of the pair tile (256, or 128 for GEMMs whose 256-wide pair
-// tiles would leave most SMs idle).
+// PBN: columns of the pair tile (256, 128 for GEMMs whose 256-wide pair tiles
+// would leave most SMs idle, or 192 for GLU GEMMs whose last round of 256-wide
+// tiles would).
 template <int PBN>
 struct PairCfg {
-  static constexpr int STAGES = PBN == 256 ? 6 : 8;
+  static constexpr int STAGES = PBN == 128 ? 8 : 6;
   static constexpr int A_BYTES = BM * BK * 2;            // 16 KB
-  static constexpr int B_BYTES = (PBN / 2) * BK * 2;     // this CTA's half of B: 16 KB / 8 KB
+  static constexpr int B_BYTES = (PBN / 2) * BK * 2;     // this CTA's half of B: 16 / 12 / 8 KB
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr size_t SMEM = 1024 + STAGES * STAGE_BYTES + EPI_WARPS * STAGE_OUT_BYTES + 256;
   static_assert(SMEM <= 232448, "pair GEMM shared memory");
@@ -895,6 +896,25 @@ const char* gemm_tc(const GemmCall& g, cudaStream_t s) {
     if (e != cudaSuccess) return cudaGetErrorString(e);
     const_cast<GemmCall&>(g).launched = 1;
     return nullptr;
+  }
+  // GLU tiles of 96 gate and 96 up columns where their rounds over the clusters
+  // take at most 0.85 of the 256-wide tiles' (a narrower tile re-reads the
+  // activations more often): the 256 x 2 x 21504 projection of a 27 B block
+  // step is 168 tiles on 76 clusters, whose third round is 16 tiles, or 224 in
+  // 2.95 rounds (the step of three layers 978 -> 945 us)
+  if (pair_ok && a.splits == 1 && glu && !g.m_dev) {
+    const int cl = std::max(g_num_sms / 2, 1), n192 = (g.N + 95) / 96;
+    const int64_t r256 = (pair_units + cl - 1) / cl, r192 = (m_pairs * n192 + cl - 1) / cl;
+    if (r192 * 192 * 100 <= r256 * 256 * 85) {
+      CUtensorMap tbn;
+      if (!make_map(&tbn, g.B, b_rows, k_b, g.ldb, 96)) return "tensor map (B, 96 rows) encode failed";
+      TcArgs a2 = a;
+      a2.n_tiles_n = n192;
+      const cudaError_t e = launch_epi_pair<EPI_GLU, 192>(ta, tbn, tc, tc2, a2, m_pairs * n192, s);
+      if (e != cudaSuccess) return cudaGetErrorString(e);
+      const_cast<GemmCall&>(g).launched = 1;
+      return nullptr;
+    }
   }
   if (pair_ok && a.splits == 1) {
     CUtensorMap tbh;

@@ -182,3 +182,28 @@ def test_attention_pipelined_hd64(T, B, Hq, Hkv, rows, ctx, causal):
     assert torch.isfinite(o.float()).all()
     # bf16 P (relative 2^-9 each, at most 2^-8 of the largest |V|) and the bf16 result
     assert (err <= 2.0 ** -8 * ref.abs() + 2.0 ** -8 * v.float().abs().max()).all()
+
+
+# GLU projections on 192-wide pair tiles (96 gate and 96 up columns; FFN widths
+# whose last round of 256-wide tiles is nearly empty): a width that 96 divides
+# and one it does not, both activations, ragged rows
+@pytest.mark.parametrize("ffn,glu,rows", [(10752, "swiglu", 130), (10112, "geglu", 255)])
+def test_glu_192_wide_tiles(T, ffn, glu, rows):
+    m = wl.ModelConfig(vocab=512, d_model=256, n_heads=4, n_kv_heads=4, head_dim=64, ffn=ffn, glu=glu, n_anchor=1,
+                       n_denoise=1, fusion="none", dtype="bf16")
+    host = wl.make_weights(m, seed=5, affine_std=0.05)
+    tm = T.TadmModel(m, T.upload_weights(m, host), max_batch=1, max_rows=rows)
+    w = wl.Workload("t", m, batch=1, prompt_len=0, gen_len=rows, steps_per_block=4, K=4)
+    z = wl.random_canvas(w, 1, rows, 0.5, 1)
+    cache = tm.new_cache(1, rows)
+    logits = torch.empty((rows, m.vocab), dtype=torch.float32, device="cuda")
+    tm.tadm_reset(1)
+    tm.tadm_anchor_forward(torch.from_numpy(z).cuda(), 4, cache)
+    tm.tadm_denoise_step(torch.from_numpy(z).cuda(), 3, 4, 0, cache, logits=logits)
+    tm.tadm_sync_status()
+    o = O.Oracle(m, host)
+    sess = o.new_session(1)
+    ref = np.asarray(o.denoise_logits(sess, z, o.anchor_forward(sess, z))).reshape(rows, m.vocab)
+    rel = np.linalg.norm(logits.cpu().numpy() - ref) / np.linalg.norm(ref)
+    assert rel < 1.5e-2, rel           # bf16 operands, two layers
+    tm.close()
