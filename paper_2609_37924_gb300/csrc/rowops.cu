@@ -180,10 +180,15 @@ __global__ void __launch_bounds__(256) rmsnorm_block_reg_kernel(const float* __r
                                                                 const void* __restrict__ gain, int w_bf16, float eps,
                                                                 void* __restrict__ out, int ldo,
                                                                 const int32_t* __restrict__ rows_idx, int lo_off) {
-  pdl_enter();
   __shared__ float red[8];
   const int m = blockIdx.x;
-  float4 v[kRowVec];
+  float4 v[kRowVec], gw[kRowVec];
+#pragma unroll
+  for (int i = 0; i < kRowVec; ++i) {               // weights: read while the previous kernel finishes
+    const int j = 4 * threadIdx.x + 1024 * i;
+    if (j < d) gw[i] = ldw4(gain, w_bf16, j);
+  }
+  pdl_enter();
   load_row_block(x + static_cast<size_t>(rows_idx ? rows_idx[m] : m) * d, d, v);
   float ss = 0.0f;
 #pragma unroll
@@ -193,7 +198,7 @@ __global__ void __launch_bounds__(256) rmsnorm_block_reg_kernel(const float* __r
   for (int i = 0; i < kRowVec; ++i) {
     const int j = 4 * threadIdx.x + 1024 * i;
     if (j >= d) break;
-    const float4 g = ldw4(gain, w_bf16, j);
+    const float4 g = gw[i];
     const float4 y = make_float4(v[i].x * inv * g.x, v[i].y * inv * g.y, v[i].z * inv * g.z, v[i].w * inv * g.w);
     const size_t o = static_cast<size_t>(m) * ldo + j;
     store4<T>(out, o, y);
@@ -463,14 +468,17 @@ __device__ __forceinline__ void ln_row_block(const float* __restrict__ xr, const
   float v[8], wv[8], bv[8], y[8];
   const int j = 8 * threadIdx.x;
   const bool on = j < d;                            // d <= 2048: one chunk per warp
+  if (on) {                                         // weights: read while the previous kernel finishes
+    ldw8(w, w_bf16, j, wv);
+    ldw8(b, w_bf16, j, bv);
+  }
+  pdl_enter();
   if (on) {
     const float4 a = *reinterpret_cast<const float4*>(xr + j), c = *reinterpret_cast<const float4*>(xr + j + 4);
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
     v[4] = c.x; v[5] = c.y; v[6] = c.z; v[7] = c.w;
     *reinterpret_cast<float4*>(row + j) = a;
     *reinterpret_cast<float4*>(row + j + 4) = c;
-    ldw8(w, w_bf16, j, wv);
-    ldw8(b, w_bf16, j, bv);
   }
   __syncthreads();
   if (threadIdx.x < 32) {
@@ -494,7 +502,6 @@ template <class T, int NCH>
 __global__ void __launch_bounds__(256) ln_pair_block_kernel(const float* __restrict__ c, const float* __restrict__ h,
                                                             const void* wc, const void* bc, const void* wh, const void* bh,
                                                             int w_bf16, float eps, void* __restrict__ u) {
-  pdl_enter();
   constexpr int d = 256 * NCH;
   const int m = blockIdx.x >> 1, part = blockIdx.x & 1;
   ln_row_block<T, NCH>((part ? h : c) + static_cast<size_t>(m) * d, part ? wh : wc, part ? bh : bc, w_bf16, eps, u,
@@ -505,7 +512,6 @@ __global__ void __launch_bounds__(256) ln_pair_block_kernel(const float* __restr
 template <int NCH>
 __global__ void __launch_bounds__(256) layernorm_block_kernel(const float* __restrict__ x, const void* w, const void* b,
                                                               int w_bf16, float eps, float* __restrict__ out) {
-  pdl_enter();
   const size_t o = static_cast<size_t>(blockIdx.x) * 256 * NCH;
   ln_row_block<float, NCH>(x + o, w, b, w_bf16, eps, out, o);
 }

@@ -109,47 +109,62 @@ __device__ __forceinline__ float4 slice_sum(const float* p, size_t stride, int s
 // columns of one row over the slices in slice order, then runs the epilogue on
 // them, with coalesced 16-byte accesses.  Same sums in the same order as the
 // two-phase path below, so the result does not depend on which one ran.
+// The epilogue's other inputs (residual, base, gate, bias) are read ahead of the
+// grid dependency: their writers ran before the GEMM whose partials this kernel
+// waits for, and that GEMM writes nothing else.
 template <int EPI>
 __global__ void __launch_bounds__(256) splitk_elem_kernel(EpiParams ep, const float* __restrict__ part, size_t stride,
                                                           int ldp, int splits) {
-  pdl_enter();
   const int n4 = ep.N / 4;
   const size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x;
-  if (i >= static_cast<size_t>(ep.M) * n4) return;
-  const int m = static_cast<int>(i / n4), n = static_cast<int>(i % n4) * 4;
+  const bool on = i < static_cast<size_t>(ep.M) * n4;
+  const int m = on ? static_cast<int>(i / n4) : 0, n = on ? static_cast<int>(i % n4) * 4 : 0;
   const size_t row = static_cast<size_t>(m);
+  float4 x = make_float4(0.0f, 0.0f, 0.0f, 0.0f), b = x, g = x;
+  float gs = 0.0f;
+  if constexpr (EPI == EPI_RESID || EPI == EPI_FUSION1 || EPI == EPI_FUSION2) {
+    if (on && ep.bias) b = ld4(ep.bias, ep.bias_bf16, n);
+  }
+  if constexpr (EPI == EPI_RESID) {
+    if (on) x = ld4(ep.resid, 0, row * ep.ldr + n);
+  } else if constexpr (EPI == EPI_ADD || EPI == EPI_FUSION2 || EPI == EPI_PA_UP) {
+    if (on) x = ld4(ep.base, 0, row * ep.ldb + n);
+    if constexpr (EPI == EPI_FUSION2)
+      if (on) g = ld4(ep.gate, ep.out_bf16, row * ep.ldg + n);
+    if constexpr (EPI == EPI_PA_UP)
+      if (on) gs = static_cast<const float*>(ep.gate)[m] * ep.rowscale[m];
+  }
+  pdl_enter();
+  if (!on) return;
   if constexpr (EPI == EPI_GLU) {   // a tile's 256 columns: 128 gate columns, then their up columns
     const float* p = part + row * ldp + (n / 128) * 256 + n % 128;
-    const float4 g = slice_sum(p, stride, splits), u = slice_sum(p + 128, stride, splits);
+    const float4 ga = slice_sum(p, stride, splits), u = slice_sum(p + 128, stride, splits);
     const bool tanh = ep.glu != 0;
     st4(ep.out, ep.out_bf16, row * ep.ldo + n,
-        mul4(map4(g, [&](float x) { return tanh ? gelu_tanh_f(x) : silu_f(x); }), u));
+        mul4(map4(ga, [&](float v) { return tanh ? gelu_tanh_f(v) : silu_f(v); }), u));
     return;
   }
   float4 a = slice_sum(part + row * ldp + n, stride, splits);
   if constexpr (EPI == EPI_RESID || EPI == EPI_FUSION1 || EPI == EPI_FUSION2) {
-    if (ep.bias) a = add4(a, ld4(ep.bias, ep.bias_bf16, n));
+    if (ep.bias) a = add4(a, b);
   }
   if constexpr (EPI == EPI_RESID) {
-    float4* r = reinterpret_cast<float4*>(ep.resid + row * ep.ldr + n);
-    *r = add4(*r, a);
+    st4(ep.resid, 0, row * ep.ldr + n, add4(x, a));
   } else if constexpr (EPI == EPI_STORE) {
     st4(ep.out, ep.out_bf16, row * ep.ldo + n, a);
   } else if constexpr (EPI == EPI_SILU) {
-    st4(ep.out, ep.out_bf16, row * ep.ldo + n, map4(a, [](float x) { return silu_f(x); }));
+    st4(ep.out, ep.out_bf16, row * ep.ldo + n, map4(a, [](float v) { return silu_f(v); }));
   } else if constexpr (EPI == EPI_ADD) {
-    a = add4(ld4(ep.base, 0, row * ep.ldb + n), a);
+    a = add4(x, a);
     st4(ep.out, 0, row * ep.ldo + n, a);
     if (ep.out2) st4(ep.out2, ep.out_bf16, row * ep.ldo2 + n, a);
   } else if constexpr (EPI == EPI_FUSION1) {
-    if (n < ep.d_split) st4(ep.out, ep.out_bf16, row * ep.ldo + n, map4(a, [](float x) { return sigmoid_f(x); }));
-    else st4(ep.out2, ep.out_bf16, row * ep.ldo2 + n - ep.d_split, map4(a, [](float x) { return gelu_erf_f(x); }));
+    if (n < ep.d_split) st4(ep.out, ep.out_bf16, row * ep.ldo + n, map4(a, [](float v) { return sigmoid_f(v); }));
+    else st4(ep.out2, ep.out_bf16, row * ep.ldo2 + n - ep.d_split, map4(a, [](float v) { return gelu_erf_f(v); }));
   } else if constexpr (EPI == EPI_FUSION2) {
-    st4(ep.out, 0, row * ep.ldo + n,
-        add4(ld4(ep.base, 0, row * ep.ldb + n), mul4(ld4(ep.gate, ep.out_bf16, row * ep.ldg + n), a)));
+    st4(ep.out, 0, row * ep.ldo + n, add4(x, mul4(g, a)));
   } else if constexpr (EPI == EPI_PA_UP) {
-    const float gs = static_cast<const float*>(ep.gate)[m] * ep.rowscale[m];
-    st4(ep.out, 0, row * ep.ldo + n, add4(ld4(ep.base, 0, row * ep.ldb + n), map4(a, [&](float x) { return gs * x; })));
+    st4(ep.out, 0, row * ep.ldo + n, add4(x, map4(a, [&](float v) { return gs * v; })));
   }
 }
 
@@ -178,7 +193,6 @@ bool elem_ok(int epi, const EpiParams& ep, int ldp) {
 template <int HD>
 __global__ void __launch_bounds__(256) splitk_qkv_kernel(EpiParams ep, const float* __restrict__ part, size_t stride,
                                                          int ldp, int splits) {
-  pdl_enter();
   constexpr int P = HD / 64, H2 = HD / 2, RB = 8;
   __shared__ bf16 sv[HD][RB + 2];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -187,16 +201,15 @@ __global__ void __launch_bounds__(256) splitk_qkv_kernel(EpiParams ep, const flo
   if (gh < ep.n_heads) { region = 0; head = gh; }
   else if (gh < ep.n_heads + ep.n_kv_heads) { region = 1; head = gh - ep.n_heads; }
   const void* gain = region == 0 ? ep.q_gain : region == 1 ? ep.k_gain : nullptr;
+  const int rr = w, m = m0 + rr;
+  const int b = m / ep.R, r = m - b * ep.R, pos = ep.ctx + r;
+  float2 cs[P];                                    // constant table, often no longer in L2: read while the GEMM runs
 #pragma unroll
-  for (int rr = w; rr < RB; rr += 8) {
-    const int m = m0 + rr;
-    if (m >= ep.M) continue;                       // uniform across the warp
-    const int b = m / ep.R, r = m - b * ep.R, pos = ep.ctx + r;
-    float2 cs[P];                                  // asked for ahead of the slices: the table may have left L2
-    if (ep.rope && region < 2) {
-#pragma unroll
-      for (int t = 0; t < P; ++t) cs[t] = ep.rope_tab[static_cast<size_t>(lane * P + t) * ep.rope_npos + pos];
-    }
+  for (int t = 0; t < P; ++t)
+    cs[t] = ep.rope && region < 2 && m < ep.M ? ep.rope_tab[static_cast<size_t>(lane * P + t) * ep.rope_npos + pos]
+                                              : make_float2(1.0f, 0.0f);
+  pdl_enter();
+  if (m < ep.M) {                                  // uniform across the warp
     const float* p = part + static_cast<size_t>(m) * ldp + gh * HD + lane * P;
     float a[P], c[P];
 #pragma unroll
@@ -218,7 +231,6 @@ __global__ void __launch_bounds__(256) splitk_qkv_kernel(EpiParams ep, const flo
         sv[lane * P + t][rr] = __float2bfloat16_rn(a[t]);
         sv[H2 + lane * P + t][rr] = __float2bfloat16_rn(c[t]);
       }
-      continue;
     }
     if (gain) {
       float ss = 0.0f;
@@ -231,7 +243,7 @@ __global__ void __launch_bounds__(256) splitk_qkv_kernel(EpiParams ep, const flo
         c[t] *= inv * ld_param(gain, ep.bias_bf16, H2 + lane * P + t);
       }
     }
-    if (ep.rope) {
+    if (ep.rope && region < 2) {
 #pragma unroll
       for (int t = 0; t < P; ++t) {
         const float x = a[t], y = c[t];
@@ -242,12 +254,14 @@ __global__ void __launch_bounds__(256) splitk_qkv_kernel(EpiParams ep, const flo
     bf16* dst = region == 0
                     ? static_cast<bf16*>(ep.q) + ((static_cast<size_t>(b) * ep.n_heads + head) * ep.R + r) * HD
                     : static_cast<bf16*>(ep.k) + ((static_cast<size_t>(b) * ep.n_kv_heads + head) * ep.kv_stride + pos) * HD;
-    if constexpr (P == 2) {
-      *reinterpret_cast<__nv_bfloat162*>(dst + 2 * lane) = __floats2bfloat162_rn(a[0], a[1]);
-      *reinterpret_cast<__nv_bfloat162*>(dst + H2 + 2 * lane) = __floats2bfloat162_rn(c[0], c[1]);
-    } else {
-      dst[lane] = __float2bfloat16_rn(a[0]);
-      dst[H2 + lane] = __float2bfloat16_rn(c[0]);
+    if (region < 2) {
+      if constexpr (P == 2) {
+        *reinterpret_cast<__nv_bfloat162*>(dst + 2 * lane) = __floats2bfloat162_rn(a[0], a[1]);
+        *reinterpret_cast<__nv_bfloat162*>(dst + H2 + 2 * lane) = __floats2bfloat162_rn(c[0], c[1]);
+      } else {
+        dst[lane] = __float2bfloat16_rn(a[0]);
+        dst[H2 + lane] = __float2bfloat16_rn(c[0]);
+      }
     }
   }
   if (region != 2) return;                         // uniform across the block
