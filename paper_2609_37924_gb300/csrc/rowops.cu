@@ -278,9 +278,12 @@ __global__ void __launch_bounds__(WPB * 32) rmsnorm_reg_kernel(const float* __re
                                                                const bf16* __restrict__ gain, float eps,
                                                                bf16* __restrict__ out, int ldo,
                                                                const int32_t* __restrict__ rows_idx, int lo_off) {
-  pdl_enter();
   constexpr int d = 256 * NCH;
   const int m = blockIdx.x * WPB + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  uint4 gr[NCH];                                    // weights: read while the previous kernel finishes
+#pragma unroll
+  for (int c = 0; c < NCH; ++c) gr[c] = *reinterpret_cast<const uint4*>(gain + (c * 32 + lane) * 8);
+  pdl_enter();
   if (m >= M) return;
   const float* xr = x + static_cast<size_t>(rows_idx ? rows_idx[m] : m) * d;
   float v[NCH][8];
@@ -301,8 +304,7 @@ __global__ void __launch_bounds__(WPB * 32) rmsnorm_reg_kernel(const float* __re
 #pragma unroll
   for (int c = 0; c < NCH; ++c) {
     const int j = (c * 32 + lane) * 8;
-    const uint4 graw = *reinterpret_cast<const uint4*>(gain + j);
-    const __nv_bfloat162* g2 = reinterpret_cast<const __nv_bfloat162*>(&graw);
+    const __nv_bfloat162* g2 = reinterpret_cast<const __nv_bfloat162*>(&gr[c]);
     uint32_t packed[4], packed_lo[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
