@@ -1169,13 +1169,31 @@ __global__ void __launch_bounds__(128) attn_bf16_kernel(const bf16* __restrict__
 // Key tiles of 64 go through shared memory (K rows and V^T rows, both
 // contiguous in the dimension their product runs over); thread (ty, tx) owns
 // rows ty and ty + 8 and keys (then dims) tx + 16 j, so every float4 read
-// feeds four FMAs per partner row.  The online softmax runs once per tile.
-// 4 x 4 heads x 128 rows, hd 64: 93 -> 12.6 us (one warp per query row, a warp
-// reduction and two uncoalesced V reads per key).
+// feeds several rows.  The sums are those of one warp per query row that takes
+// the keys one by one: a score is 32 partial sums over dims l, l + 32, ..
+// added as a tree, and every key updates maximum, sum and output in key order,
+// so a result depends neither on the tiling nor on other rows (a sampler that
+// compares confidences of nearly equal positions sees the last bit).  Maxima
+// and exponentials of a tile are taken in parallel (a scan over the keys);
+// only the FMA chains run key by key.  4 x 4 heads x 128 rows, hd 64: 93 ->
+// 16.6 us (one warp per query row, with a warp reduction and two uncoalesced V
+// reads per key, before; 12.6 with one softmax update per tile).
 constexpr int FQ = 16, FK = 64, FNT = 128;
 
+__device__ __forceinline__ float4 mul4(const float4& a, const float4& b) {
+  return make_float4(__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y), __fmul_rn(a.z, b.z), __fmul_rn(a.w, b.w));
+}
+__device__ __forceinline__ float4 fma4(const float4& a, const float4& b, const float4& c) {
+  return make_float4(fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y), fmaf(a.z, b.z, c.z), fmaf(a.w, b.w, c.w));
+}
+__device__ __forceinline__ float4 add4(const float4& a, const float4& b) {
+  return make_float4(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y), __fadd_rn(a.z, b.z), __fadd_rn(a.w, b.w));
+}
+// acc c + p v, the rescaled sum rounded once
+__device__ __forceinline__ float weigh(float acc, float c, float p, float v) { return fmaf(acc, c, __fmul_rn(p, v)); }
+
 template <int HD>
-struct F32Cfg { static constexpr int FLOATS = FQ * (HD + 4) + FK * (HD + 4) + HD * (FK + 4) + FQ * (FK + 4); };
+struct F32Cfg { static constexpr int FLOATS = FQ * (HD + 4) + FK * (HD + 4) + HD * (FK + 4) + 2 * FQ * (FK + 4); };
 
 template <int HD>
 __global__ void __launch_bounds__(FNT) attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k,
@@ -1188,7 +1206,8 @@ __global__ void __launch_bounds__(FNT) attn_f32_kernel(const float* __restrict__
   float* sQ = reinterpret_cast<float*>(smem_raw);          // [FQ][LD]
   float* sK = sQ + FQ * LD;                                // [FK][LD]
   float* sV = sK + FK * LD;                                // [HD][LDP]
-  float* sP = sV + HD * LDP;                               // [FQ][LDP]
+  float* sP = sV + HD * LDP;                               // [FQ][LDP] scores, then probabilities
+  float* sC = sP + FQ * LDP;                               // [FQ][LDP] rescale factors
   const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16;
   const int r0 = blockIdx.x * FQ, h = blockIdx.y, b = blockIdx.z;
   const int hk = h / (n_heads / n_kv_heads);
@@ -1200,7 +1219,9 @@ __global__ void __launch_bounds__(FNT) attn_f32_kernel(const float* __restrict__
   // keys that any row of the block may see
   const int end = causal ? ctx + r0 + nr : ctx + rows;
   const int begin = window > 0 ? max(0, ctx + r0 - window + 1) : 0;
-  float acc[2][ND], m[2] = {-INFINITY, -INFINITY}, l[2] = {0.0f, 0.0f};
+  // the softmax of row sr by eight lanes of the warp that owns it (rows ty and ty + 8 of its two ty)
+  const int lane = tid & 31, sr = 2 * (tid >> 5) + ((lane >> 3) & 1) + 8 * (lane >> 4), sk = 8 * (lane & 7);
+  float acc[2][ND], m = -INFINITY, l[2] = {0.0f, 0.0f};
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -1234,64 +1255,117 @@ __global__ void __launch_bounds__(FNT) attn_f32_kernel(const float* __restrict__
         sV[(i / FK) * LDP + i % FK] = k0 + i % FK < end ? vb[static_cast<size_t>(i / FK) * kv_stride + k0 + i % FK] : 0.0f;
     }
     __syncthreads();
-    float s[2][4];
+    // scores: 32 partial sums over dims l, l + 32, .., then their tree sum (16, 8, 4, 2, 1 apart), four at a time
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
+    for (int jp = 0; jp < 4; jp += 2) {
+      float4 C[2][2], B[2][2], A[2][2];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) s[i][j] = 0.0f;
-#pragma unroll 4
-    for (int d = 0; d < HD; d += 4) {
-      float4 a[2], c[4];
+      for (int n = 0; n < 8; ++n) {                        // dims 4c .. 4c + 3 with c = 0 4 2 6 1 5 3 7
+        const int c = (n >> 2) + (n & 2) + 4 * (n & 1);
+        float4 p[2][2];
 #pragma unroll
-      for (int i = 0; i < 2; ++i) a[i] = *reinterpret_cast<const float4*>(sQ + (ty + 8 * i) * LD + d);
+        for (int e = 0; e < HD / 32; ++e) {
+          float4 a[2], b[2];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) c[j] = *reinterpret_cast<const float4*>(sK + (tx + 16 * j) * LD + d);
+          for (int i = 0; i < 2; ++i) a[i] = *reinterpret_cast<const float4*>(sQ + (ty + 8 * i) * LD + 4 * c + 32 * e);
+#pragma unroll
+          for (int j = 0; j < 2; ++j) b[j] = *reinterpret_cast<const float4*>(sK + (tx + 16 * (jp + j)) * LD + 4 * c + 32 * e);
+#pragma unroll
+          for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+              p[i][j] = e == 0 ? mul4(a[i], b[j]) : fma4(a[i], b[j], p[i][j]);
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            if ((n & 1) == 0) { A[i][j] = p[i][j]; continue; }
+            A[i][j] = add4(A[i][j], p[i][j]);
+            if ((n & 2) == 0) { B[i][j] = A[i][j]; continue; }
+            B[i][j] = add4(B[i][j], A[i][j]);
+            C[i][j] = (n & 4) == 0 ? B[i][j] : add4(C[i][j], B[i][j]);
+          }
+      }
 #pragma unroll
       for (int i = 0; i < 2; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-          s[i][j] = fmaf(a[i].w, c[j].w, fmaf(a[i].z, c[j].z, fmaf(a[i].y, c[j].y, fmaf(a[i].x, c[j].x, s[i][j]))));
+        for (int j = 0; j < 2; ++j) {
+          const float4 t = C[i][j];
+          sP[(ty + 8 * i) * LDP + tx + 16 * (jp + j)] =
+              __fmul_rn(__fadd_rn(__fadd_rn(t.x, t.z), __fadd_rn(t.y, t.w)), scale);
+        }
     }
+    __syncwarp();                                          // a row's scores are written and read by one warp
+    // online softmax key by key: m_j = max(m_(j-1), s_j), c_j = e^(m_(j-1) - m_j), p_j = e^(s_j - m_j)
+    {
+      const int qpos = ctx + r0 + sr;
+      const int hi = (causal ? min(end, qpos + 1) : end) - k0, lo = (window > 0 ? qpos - window + 1 : 0) - k0;
+      float d[8], mine = -INFINITY;
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int qpos = ctx + r0 + ty + 8 * i;
-      const int hi = causal ? min(end, qpos + 1) : end, lo = window > 0 ? qpos - window + 1 : 0;
-      float mx = m[i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int key = k0 + tx + 16 * j;
-        s[i][j] = key < hi && key >= lo ? s[i][j] * scale : -INFINITY;
-        mx = fmaxf(mx, s[i][j]);
+      for (int e = 0; e < 8; e += 4) {
+        const float4 t = *reinterpret_cast<const float4*>(sP + sr * LDP + sk + e);
+        d[e] = t.x; d[e + 1] = t.y; d[e + 2] = t.z; d[e + 3] = t.w;
       }
 #pragma unroll
-      for (int w = 8; w > 0; w >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, w));
-      const float f = mx == -INFINITY ? 1.0f : expf(m[i] - mx);   // nothing seen yet: nothing to rescale
-      float ps = 0.0f;
+      for (int e = 0; e < 8; ++e)
+        if (sk + e >= lo && sk + e < hi) mine = fmaxf(mine, d[e]);
+      float before = mine;                                 // maximum of the lanes before this one, then of all
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float p = s[i][j] == -INFINITY ? 0.0f : expf(s[i][j] - mx);
-        sP[(ty + 8 * i) * LDP + tx + 16 * j] = p;
-        ps += p;
+      for (int w = 1; w < 8; w <<= 1) {
+        const float t = __shfl_up_sync(0xffffffffu, before, w, 8);
+        if ((lane & 7) >= w) before = fmaxf(before, t);
       }
+      const float all = __shfl_sync(0xffffffffu, before, 7, 8);
+      before = __shfl_up_sync(0xffffffffu, before, 1, 8);
+      float cur = (lane & 7) == 0 ? m : fmaxf(m, before);
+      m = fmaxf(m, all);
 #pragma unroll
-      for (int w = 8; w > 0; w >>= 1) ps += __shfl_xor_sync(0xffffffffu, ps, w);
-      l[i] = l[i] * f + ps;
-      m[i] = mx;
-#pragma unroll
-      for (int j = 0; j < ND; ++j) acc[i][j] *= f;
+      for (int e = 0; e < 8; ++e) {
+        const bool see = sk + e >= lo && sk + e < hi;
+        const float mn = see ? fmaxf(cur, d[e]) : cur;
+        sC[sr * LDP + sk + e] = see ? expf(cur - mn) : 1.0f;
+        sP[sr * LDP + sk + e] = see ? expf(d[e] - mn) : 0.0f;
+        cur = mn;
+      }
     }
-    __syncwarp();                                          // a row's probabilities are written and read by one warp
+    __syncwarp();
+    // keys in order, as they entered the softmax; masked ones are left out (their V may hold anything)
+    const int hi0 = causal ? ctx + r0 + 1 : end, lo_last = window > 0 ? ctx + r0 + nr - window : 0;
+    if (k0 + FK <= min(hi0, end) && k0 >= lo_last) {
 #pragma unroll 4
-    for (int c = 0; c < FK; c += 4) {
-      float4 p[2];
+      for (int c = 0; c < FK; c += 4) {
+        float4 p[2], f[2];
 #pragma unroll
-      for (int i = 0; i < 2; ++i) p[i] = *reinterpret_cast<const float4*>(sP + (ty + 8 * i) * LDP + c);
+        for (int i = 0; i < 2; ++i) {
+          p[i] = *reinterpret_cast<const float4*>(sP + (ty + 8 * i) * LDP + c);
+          f[i] = *reinterpret_cast<const float4*>(sC + (ty + 8 * i) * LDP + c);
+          l[i] = fmaf(fmaf(fmaf(fmaf(l[i], f[i].x, p[i].x), f[i].y, p[i].y), f[i].z, p[i].z), f[i].w, p[i].w);
+        }
 #pragma unroll
-      for (int j = 0; j < ND; ++j) {
-        const float4 v = *reinterpret_cast<const float4*>(sV + (tx + 16 * j) * LDP + c);
+        for (int j = 0; j < ND; ++j) {
+          const float4 v = *reinterpret_cast<const float4*>(sV + (tx + 16 * j) * LDP + c);
 #pragma unroll
-        for (int i = 0; i < 2; ++i)
-          acc[i][j] = fmaf(p[i].w, v.w, fmaf(p[i].z, v.z, fmaf(p[i].y, v.y, fmaf(p[i].x, v.x, acc[i][j]))));
+          for (int i = 0; i < 2; ++i) {
+            acc[i][j] = weigh(acc[i][j], f[i].x, p[i].x, v.x);
+            acc[i][j] = weigh(acc[i][j], f[i].y, p[i].y, v.y);
+            acc[i][j] = weigh(acc[i][j], f[i].z, p[i].z, v.z);
+            acc[i][j] = weigh(acc[i][j], f[i].w, p[i].w, v.w);
+          }
+        }
+      }
+    } else {
+      const int n = min(FK, end - k0);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int qpos = ctx + r0 + ty + 8 * i;
+        const int lo = max(0, (window > 0 ? qpos - window + 1 : 0) - k0), hi = min(n, (causal ? qpos + 1 : end) - k0);
+        for (int c = lo; c < hi; ++c) {
+          const float p = sP[(ty + 8 * i) * LDP + c], f = sC[(ty + 8 * i) * LDP + c];
+          l[i] = fmaf(l[i], f, p);
+#pragma unroll
+          for (int j = 0; j < ND; ++j) acc[i][j] = weigh(acc[i][j], f, p, sV[(tx + 16 * j) * LDP + c]);
+        }
       }
     }
   }

@@ -2,30 +2,31 @@
 // acc[M, N] = A[M, K] * B[N, K]^T with the same fused epilogues as the tensor
 // core path.
 //
-// One 256-thread block per TM x 64 output tile (TM = 32, or 16 when 32-row
+// One 128-thread block per TM x 64 output tile (TM = 32, or 16 when 32-row
 // tiles would leave SMs idle).  The GEMMs of this path are a few hundred rows
-// by a few hundred columns, so a launch is paced by the latency of one
-// block's K loop, not by FMA throughput: K advances 64 at a time through a
-// cp.async ring, and the block's thread groups (four of 64 threads, or eight
-// warps for 16-row tiles) each take their share of the 64 columns of every
-// stage for the whole tile (a split of K inside the block; 4 x 8 outputs per
-// thread either way); the partial tiles are summed in group order through
-// shared memory.  Weights (b_weights) start loading ahead of the grid
-// dependency.  Rows of the stage are padded to 68 floats: the eight column
-// addresses of a quarter-warp's float4 reads fall into different banks.
-// 16-row tiles run six stages, one block per SM: a launch that starts while
-// its predecessor's last blocks run otherwise packs three blocks onto the
-// first SMs that come free (W_down of 512 rows took 37 us in a generation and
-// 15 alone).  512 rows in a generation: W_down (N 256, K 1024) 14.4 us, W_o 4.9,
-// QKV (N 768, K 256) 12.4, GLU (N 2 x 1024, K 256) 22, fusion hidden (N 1280, K
-// 512) 38; with 64 x 64 tiles and 16 columns of K per synchronous step the
-// residual projections took 95 us a launch, QKV 36, GLU 38.
+// by a few hundred columns, so a launch is paced by one block's K loop and its
+// shared-memory reads: K advances 64 at a time through a cp.async ring; a warp
+// owns TM / 4 whole rows, so that its reads of A are one address for all lanes,
+// and a lane two columns.  Every output is one FMA chain in the order of k: a
+// result depends neither on the tile nor on the number of rows.  (K split over
+// thread groups of the block was 8 % faster over a generation, but its sums
+// differ in the last bit, which moves tokens between nearly equal confidences.)
+// Weights (b_weights) start loading ahead of the grid dependency.  Rows of the
+// stage are padded to 68 floats: the eight column addresses of a quarter-warp's
+// float4 reads fall into different banks.  16-row tiles run six stages, one
+// block per SM: a launch that starts while its predecessor's last blocks run
+// otherwise packs three blocks onto the first SMs that come free.  512 rows,
+// launched alone: W_down and W_o (N 256, K 1024 and 256) 17.8 us on average,
+// QKV (N 768, K 256) 13.5, GLU (N 2 x 1024, K 256) 23.6, fusion hidden (N 1280,
+// K 512) 40.8; with 64 x 64 tiles and 16 columns of K per synchronous step the
+// residual projections took 95 us, QKV 36, GLU 38.  Eight warps of half as many
+// columns: 10.9 -> 12.2 ms a generation.
 // EPI_GLU tiles hold 32 gate and 32 up columns; EPI_QKV needs head_dim <= 64.
 #include "kernels.h"
 
 namespace tadm {
 namespace {
-constexpr int TN = 64, TK = 64, LDK = TK + 4, NT = 256;
+constexpr int TN = 64, TK = 64, LDK = TK + 4, NT = 128;
 
 struct SmemSrc {
   static constexpr bool kStaged = false;
@@ -49,7 +50,7 @@ __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0
 
 template <int TM>
 struct SimtCfg {
-  static constexpr int STAGES = TM == 16 ? 6 : 3, GROUPS = TM == 16 ? 8 : 4;
+  static constexpr int STAGES = TM == 16 ? 6 : 3;
   static constexpr int FLOATS = STAGES * (TM + TN) * LDK;
 };
 
@@ -58,7 +59,7 @@ template <int EPI, int TM, bool VEC>
 __global__ void __launch_bounds__(NT, TM == 16 ? 1 : 2) gemm_simt_kernel(const float* __restrict__ A, const float* __restrict__ B, int M,
                                                        int K, int lda, int ldb, int tiles_n, int n_rows_b, int b_split,
                                                        int b_early, EpiParams ep) {
-  constexpr int STAGES = SimtCfg<TM>::STAGES, GROUPS = SimtCfg<TM>::GROUPS, TG = NT / GROUPS, KC = TK / GROUPS;
+  constexpr int STAGES = SimtCfg<TM>::STAGES, RM = TM / (NT / 32);
   extern __shared__ __align__(16) float smem[];
   const int tid = threadIdx.x, m0 = blockIdx.x / tiles_n * TM, nb = blockIdx.x % tiles_n;
   const int ksteps = (K + TK - 1) / TK;
@@ -95,15 +96,11 @@ __global__ void __launch_bounds__(NT, TM == 16 ? 1 : 2) gemm_simt_kernel(const f
     }
     cp_commit();
   }
-  // group g owns columns KC g .. KC g + KC - 1 of every stage; its thread
-  // (ty, tx) owns rows ty + TY i and columns tx + 8 j of the tile
-  constexpr int TY = TG / 8, RM = TM / TY;
-  const int g = tid / TG, t = tid % TG, ty = t / 8, tx = t % 8;
-  float acc[RM][8];
+  // warp w owns rows RM w .. RM w + RM - 1 of the tile, its lane l columns l and l + 32
+  const int warp = tid >> 5, lane = tid & 31;
+  float acc[RM][2];
 #pragma unroll
-  for (int i = 0; i < RM; ++i)
-#pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = 0.0f;
+  for (int i = 0; i < RM; ++i) acc[i][0] = acc[i][1] = 0.0f;
   for (int ks = 0; ks < ksteps; ++ks) {
     cp_wait<STAGES - 2>();
     __syncthreads();                                // stage ks has landed; stage ks - 1 has been read by all
@@ -112,20 +109,19 @@ __global__ void __launch_bounds__(NT, TM == 16 ? 1 : 2) gemm_simt_kernel(const f
       load_a(ks + STAGES - 1);
     }
     cp_commit();
-    const float* a0 = sA + (ks % STAGES) * TM * LDK + ty * LDK + KC * g;
-    const float* b0 = sB + (ks % STAGES) * TN * LDK + tx * LDK + KC * g;
+    const float* a0 = sA + (ks % STAGES) * TM * LDK + RM * warp * LDK;
+    const float* b0 = sB + (ks % STAGES) * TN * LDK + lane * LDK;
 #pragma unroll
-    for (int kk = 0; kk < KC; kk += 4) {
-      float4 a[RM];
+    for (int kk = 0; kk < TK; kk += 4) {
+      float4 a[RM], b[2];
 #pragma unroll
-      for (int i = 0; i < RM; ++i) a[i] = *reinterpret_cast<const float4*>(a0 + TY * i * LDK + kk);
-      float4 b[8];
+      for (int j = 0; j < 2; ++j) b[j] = *reinterpret_cast<const float4*>(b0 + 32 * j * LDK + kk);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) b[j] = *reinterpret_cast<const float4*>(b0 + 8 * j * LDK + kk);
+      for (int i = 0; i < RM; ++i) a[i] = *reinterpret_cast<const float4*>(a0 + i * LDK + kk);
 #pragma unroll
       for (int i = 0; i < RM; ++i)
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < 2; ++j) {
           acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
           acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
           acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
@@ -133,33 +129,28 @@ __global__ void __launch_bounds__(NT, TM == 16 ? 1 : 2) gemm_simt_kernel(const f
         }
     }
   }
-  // partial tiles of the groups -> their sum in group order, in the first one's place
+  if constexpr (EPI == EPI_RESID) {                 // element-wise, coalesced
+#pragma unroll
+    for (int i = 0; i < RM; ++i)
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int m = m0 + RM * warp + i, n = nb * TN + lane + 32 * j;
+        if (m < M && n < ep.N) {
+          float* x = ep.resid + static_cast<size_t>(m) * ep.ldr + n;
+          *x += ep.bias ? acc[i][j] + ld_param(ep.bias, ep.bias_bf16, n) : acc[i][j];
+        }
+      }
+  }
+  if constexpr (EPI == EPI_RESID) return;
   cp_wait<0>();
-  __syncthreads();
-  constexpr int LDC = TN + 1, TILE = TM * LDC;
-  static_assert(GROUPS * TILE <= SimtCfg<TM>::FLOATS, "partial tiles fit the stages");
+  __syncthreads();                                  // the stages are free: the tile goes over them
+  constexpr int LDC = TN + 1;
+  static_assert(TM * LDC <= SimtCfg<TM>::FLOATS, "the output tile fits the stages");
   float* sC = smem;
 #pragma unroll
   for (int i = 0; i < RM; ++i)
 #pragma unroll
-    for (int j = 0; j < 8; ++j) sC[g * TILE + (ty + TY * i) * LDC + tx + 8 * j] = acc[i][j];
-  __syncthreads();
-  for (int e = tid; e < TM * TN; e += NT) {
-    const int o = (e / TN) * LDC + e % TN;
-    float s = sC[o];
-#pragma unroll
-    for (int q = 1; q < GROUPS; ++q) s += sC[q * TILE + o];
-    if constexpr (EPI == EPI_RESID) {               // element-wise, coalesced
-      const int m = m0 + e / TN, n = nb * TN + e % TN;
-      if (m < M && n < ep.N) {
-        float* x = ep.resid + static_cast<size_t>(m) * ep.ldr + n;
-        *x += ep.bias ? s + ld_param(ep.bias, ep.bias_bf16, n) : s;
-      }
-    } else {
-      sC[o] = s;
-    }
-  }
-  if constexpr (EPI == EPI_RESID) return;
+    for (int j = 0; j < 2; ++j) sC[(RM * warp + i) * LDC + lane + 32 * j] = acc[i][j];
   __syncthreads();
   // the tile's 64 columns of a row go to one thread, or to two where the epilogue's columns are independent
   constexpr int NS = (EPI == EPI_STORE || EPI == EPI_SILU || EPI == EPI_ADD || EPI == EPI_FUSION1 || EPI == EPI_FUSION2 ||

@@ -657,10 +657,7 @@ __global__ void __launch_bounds__(256) rms_divide_kernel(const float* __restrict
   __shared__ float red[8];
   const size_t base = static_cast<size_t>(blockIdx.x) * d;
   float ss = 0.0f;
-  for (int j = threadIdx.x * 4; j < d; j += 1024) {
-    const float4 v = *reinterpret_cast<const float4*>(x + base + j);
-    ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
-  }
+  for (int j = threadIdx.x; j < d; j += 256) ss += x[base + j] * x[base + j];
   ss = warp_sum(ss);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
   __syncthreads();

@@ -110,13 +110,17 @@ __global__ void combine_kernel(const float* __restrict__ part, int rows, int n_t
   }
 }
 
-// combine_kernel with a block per row, for few rows of many tiles (32 rows x 1000 tiles: 14 -> 8 us with the copies behind it).
+// combine_kernel with a block per row, for few rows of many tiles (32 rows x 1000 tiles: 14 -> 8 us with the copies
+// behind it).  All threads take the exponentials; warp 0 adds the terms in combine_kernel's order, so a row's
+// confidence does not depend on how many rows the launch has.
+constexpr int kCombineTiles = 4096;
 __global__ void __launch_bounds__(256) combine_block_kernel(const float* __restrict__ part, int n_tiles,
                                                             float* __restrict__ conf, int32_t* __restrict__ tok,
                                                             const int32_t* __restrict__ rows_idx) {
   pdl_enter();
   __shared__ float sv[32];
   __shared__ int si[32];
+  __shared__ float2 term[kCombineTiles];            // (sum, weight) of a tile; (0, 0) for one without a token
   const float* p = part + static_cast<size_t>(blockIdx.x) * n_tiles * 3;
   float mx = -INFINITY;
   int arg = -1;
@@ -126,18 +130,16 @@ __global__ void __launch_bounds__(256) combine_block_kernel(const float* __restr
     if (i >= 0 && better(m, i, mx, arg)) { mx = m; arg = i; }
   }
   block_argmax<256>(mx, arg, sv, si);
-  float s = 0.0f;
   for (int t = threadIdx.x; t < n_tiles; t += 256)
-    if (__float_as_int(p[3 * t + 2]) >= 0) s += p[3 * t + 1] * expf(p[3 * t] - mx);
+    term[t] = __float_as_int(p[3 * t + 2]) >= 0 ? make_float2(p[3 * t + 1], expf(p[3 * t] - mx)) : make_float2(0.0f, 0.0f);
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+  float s = 0.0f;
+  for (int t = threadIdx.x; t < n_tiles; t += 32) s = fmaf(term[t].x, term[t].y, s);
   s = warp_sum(s);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) sv[threadIdx.x >> 5] = s;
-  __syncthreads();
   if (threadIdx.x == 0) {
-    float t = 0.0f;
-    for (int w = 0; w < 8; ++w) t += sv[w];
     const int dst = rows_idx ? rows_idx[blockIdx.x] : blockIdx.x;   // compacted rows scatter back to their positions
-    conf[dst] = 1.0f / t;
+    conf[dst] = 1.0f / s;
     tok[dst] = arg;
   }
 }
@@ -1080,7 +1082,7 @@ const char* confidence_rows(const float* logits, int rows, int vocab, int ld, in
 const char* combine_partials(const float* part, int rows, int n_tiles, float* conf, int32_t* tok, cudaStream_t s,
                              const int32_t* rows_idx) {
   if (rows <= 0) return nullptr;
-  if (rows <= 1024 && n_tiles >= 64) {   // a row is a chain of n_tiles / 32 loads for one warp
+  if (rows <= 1024 && n_tiles >= 64 && n_tiles <= kCombineTiles) {   // a row is a chain of n_tiles / 32 loads for one warp
     launch_pdl(combine_block_kernel, rows, 256, 0, s, part, n_tiles, conf, tok, rows_idx);
     return err();
   }

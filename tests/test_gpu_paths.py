@@ -207,3 +207,53 @@ def test_glu_192_wide_tiles(T, ffn, glu, rows):
     rel = np.linalg.norm(logits.cpu().numpy() - ref) / np.linalg.norm(ref)
     assert rel < 1.5e-2, rel           # bf16 operands, two layers
     tm.close()
+
+
+# fp32 results of a row do not depend on how many rows the launch has: 16- and
+# 32-row GEMM tiles, block- and warp-per-row reduction of the head's tiles, one
+# or several attention blocks (equal to the last bit: a sampler compares
+# confidences that may be that close)
+@pytest.mark.parametrize("rows", [1, 100, 1024])
+def test_f32_rows_alone(T, rows):
+    g = torch.Generator(device="cuda").manual_seed(3)
+    d, vocab, M = 64, 4165, 1100
+    x = torch.randn((M, d), generator=g, device="cuda")
+    w = torch.randn((vocab, d), generator=g, device="cuda") * 0.3
+    scratch = torch.empty(T.tadm_head_scratch_size(M, vocab, 0), dtype=torch.uint8, device="cuda")
+    conf, tok = torch.empty(M, device="cuda"), torch.empty(M, dtype=torch.int32, device="cuda")
+    T.tadm_head_confidence(x, w, vocab - 1, conf, tok, scratch, 0)
+    conf2, tok2 = torch.empty(rows, device="cuda"), torch.empty(rows, dtype=torch.int32, device="cuda")
+    T.tadm_head_confidence(x[:rows], w, vocab - 1, conf2, tok2, scratch, 0)
+    assert torch.equal(conf[:rows], conf2) and torch.equal(tok[:rows], tok2)
+    p = torch.softmax((x.double() @ w.double().T)[:, :-1], -1)
+    assert (conf / p.max(-1).values.float() - 1).abs().max() < 1e-4    # logits of 64 terms, exponentiated
+
+
+@pytest.mark.parametrize("hd", [32, 64, 128])
+def test_attention_f32_row_alone(T, hd):
+    g = torch.Generator(device="cuda").manual_seed(4)
+    n, rows = 137, 33
+    k = torch.randn((1, 2, n + 3, hd), generator=g, device="cuda")
+    v = torch.randn((1, 2, hd, n + 3), generator=g, device="cuda")
+    q = torch.randn((1, 4, rows, hd), generator=g, device="cuda")
+    o = torch.empty((rows, 4 * hd), device="cuda")
+    T.tadm_attention(q, k, v, o, 4, 2, rows, n - rows, False, 0)
+    for r in (0, 15, 32):
+        one = torch.empty((1, 4 * hd), device="cuda")
+        T.tadm_attention(q[:, :, r:r + 1].contiguous(), k, v, one, 4, 2, 1, n - 1, False, 0)
+        assert torch.equal(o[r:r + 1], one)
+
+
+# a key outside a row's causal or window range leaves the row alone, whatever its V holds
+@pytest.mark.parametrize("causal,window", [(True, 0), (False, 40)])
+def test_attention_f32_masked_v(T, causal, window):
+    g = torch.Generator(device="cuda").manual_seed(5)
+    rows, hd = 100, 64
+    q, k = (torch.randn((1, 1, rows, hd), generator=g, device="cuda") for _ in range(2))
+    v = torch.randn((1, 1, hd, rows), generator=g, device="cuda")
+    bad = 99 if causal else 0
+    v[..., bad] = float("inf")
+    o = torch.empty((rows, hd), device="cuda")
+    T.tadm_attention(q, k, v, o, 1, 1, rows, 0, causal, 0, window=window)
+    free = torch.arange(rows, device="cuda") < 99 if causal else torch.arange(rows, device="cuda") >= window
+    assert torch.isfinite(o[free]).all() and not torch.isfinite(o[~free]).any()
