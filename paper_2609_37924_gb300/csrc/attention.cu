@@ -459,12 +459,12 @@ __global__ void __launch_bounds__(192, AttnTcCfg<HD, TKV>::MIN_BLOCKS)
 // hd 64 to the 64 TMEM columns left, two keys per column: a P V MMA then reads
 // only V from shared memory (16 of 48 cycles of operand reads for 32 of MMA)
 // and the softmax needs no proxy fence (two layers of 16 x 1024 rows:
-// 757 -> 748 us).  The MMA thread
-// issues S(i) as soon as the softmax has released its S buffer (tile i - 2),
-// then O += P(i-1) V(i-1): while the softmax threads exponentiate tile i,
-// the tensor pipe already computes S(i+1).  Ordering facts the softmax relies
-// on (tcgen05 operations of one thread complete in issue order): P V(i-2) is
-// issued before S(i), so when S(i) is complete the P buffer of tile i and
+// 757 -> 748 us).  The MMA warp issues S(i), then O += P(i-1) V(i-1): while
+// the softmax warps exponentiate tile i, the tensor pipe already computes
+// S(i+1).  Ordering facts (tcgen05 operations of one thread complete in issue
+// order): P V(i-2) is issued after p_full(i-2), when every softmax warp has
+// read S(i-2), and before S(i), so S(i) needs no wait for its buffer (an extra
+// barrier for it cost 2.4 of 29.2 us over 16 x 2032 keys at hd 128); when S(i) is complete, the P buffer of tile i and
 // the O accumulator up to tile i-2 are settled; a rescale of O at tile i
 // waits for P V(i-1) on o_full.
 template <int HD_>
@@ -503,12 +503,11 @@ __global__ void __launch_bounds__(192, AttnDbCfg<HD_>::MIN_BLOCKS)
   uint64_t* kv_full = bars + 1;        // [NST]
   uint64_t* kv_empty = bars + 5;       // [NST]
   uint64_t* s_full = bars + 9;         // [2]
-  uint64_t* s_free = bars + 11;        // [2]
-  uint64_t* p_full = bars + 13;        // [2]
-  uint64_t* o_full = bars + 15;        // one completion per P V
-  uint64_t* drain = bars + 16;
-  uint64_t* o_done = bars + 17;        // the last P V is complete
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 18);
+  uint64_t* p_full = bars + 11;        // [2]
+  uint64_t* o_full = bars + 13;        // one completion per P V
+  uint64_t* drain = bars + 14;
+  uint64_t* o_done = bars + 15;        // the last P V is complete
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 16);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -528,7 +527,6 @@ __global__ void __launch_bounds__(192, AttnDbCfg<HD_>::MIN_BLOCKS)
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(&s_full[s], 1);
-      mbar_init(&s_free[s], act_warps);
       mbar_init(&p_full[s], act_warps);
     }
     mbar_init(o_full, 1);
@@ -582,10 +580,9 @@ __global__ void __launch_bounds__(192, AttnDbCfg<HD_>::MIN_BLOCKS)
       const uint64_t q0 = sdesc_kmajor_sw128(smem_u32(sQ));
       for (int i = 0; ok && i <= n_tiles; ++i) {
         if (i < n_tiles) {
-          // S(i) = Q K(i)^T into S buffer i & 1, once the softmax has released it (tile i - 2)
+          // S(i) = Q K(i)^T into S buffer i & 1, which the softmax has read (p_full of tile i - 2)
           const int st = i % NST, sb = i & 1;
           if (!warp_wait_bounded(&kv_full[st], (i / NST) & 1, abort_flag, args.status)) break;
-          if (i >= 2 && !warp_wait_bounded(&s_free[sb], ((i - 2) >> 1) & 1, abort_flag, args.status)) break;
           tc_fence_after();
           const uint64_t k0 = sdesc_kmajor_sw128(smem_u32(sK + st * C::K_BYTES));
 #pragma unroll
@@ -663,9 +660,6 @@ __global__ void __launch_bounds__(192, AttnDbCfg<HD_>::MIN_BLOCKS)
       tmem_ld32_nowait(t_s + 32, rb);
       tmem_wait_ld(ra);
       tmem_bind(rb);
-      // S is in registers: its TMEM buffer goes back to the MMA thread (S(i+2)) at once
-      tc_fence_before();
-      warp_arrive(&s_free[sb]);
       // pass 1: row max over the tile (both halves stay in registers for pass 2)
       float mxa[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
       if (masked) max64<true>(ra, rb, 0, lim, mxa);
@@ -722,12 +716,9 @@ __global__ void __launch_bounds__(192, AttnDbCfg<HD_>::MIN_BLOCKS)
       f2_unpack(ps2[1], b0, b1);
       l_run += (a0 + a1) + (b0 + b1);
       m_ref = m_new;
-      if constexpr (C::P_TMEM) {
-        tmem_wait_st();
-        tc_fence_before();
-      } else {
-        fence_proxy_async_smem();
-      }
+      if constexpr (C::P_TMEM) tmem_wait_st();
+      else fence_proxy_async_smem();
+      tc_fence_before();
       warp_arrive(&p_full[sb]);
     }
     // o_done, not o_full: at this point P V(n-2) may still be running as well
