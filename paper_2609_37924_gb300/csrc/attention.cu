@@ -167,11 +167,10 @@ __global__ void __launch_bounds__(192, AttnTcCfg<HD, TKV>::MIN_BLOCKS)
   uint64_t* kv_full = bars + 1;       // [2]
   uint64_t* kv_empty = bars + 3;      // [2]
   uint64_t* s_full = bars + 5;
-  uint64_t* s_free = bars + 6;
-  uint64_t* p_full = bars + 7;
-  uint64_t* o_full = bars + 8;
-  uint64_t* drain = bars + 10;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 11);
+  uint64_t* p_full = bars + 6;
+  uint64_t* o_full = bars + 7;
+  uint64_t* drain = bars + 8;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 9);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -198,7 +197,6 @@ __global__ void __launch_bounds__(192, AttnTcCfg<HD, TKV>::MIN_BLOCKS)
       mbar_init(&kv_empty[s], 1);
     }
     mbar_init(s_full, 1);
-    mbar_init(s_free, act_warps);
     mbar_init(p_full, act_warps);
     mbar_init(o_full, 1);
     mbar_init(drain, 1);
@@ -252,7 +250,6 @@ __global__ void __launch_bounds__(192, AttnTcCfg<HD, TKV>::MIN_BLOCKS)
       for (int i = 0; ok && i < n_tiles; ++i) {
         const int st = i & 1;
         if (!warp_wait_bounded(&kv_full[st], (i >> 1) & 1, abort_flag, args.status)) break;
-        if (i > 0 && !warp_wait_bounded(s_free, (i - 1) & 1, abort_flag, args.status)) break;
         tc_fence_after();
         const uint64_t k0 = sdesc_kmajor_sw128(smem_u32(sK + st * C::K_BYTES));
         const uint64_t v0 = sdesc_kmajor_sw128(smem_u32(sV + st * C::V_BYTES));
@@ -261,8 +258,8 @@ __global__ void __launch_bounds__(192, AttnTcCfg<HD, TKV>::MIN_BLOCKS)
           umma_bf16(t_s, q0 + (((kk >> 2) * 16384 + (kk & 3) * 32) >> 4),
                     k0 + (((kk >> 2) * (TKV * 128) + (kk & 3) * 32) >> 4), idesc_s, kk != 0);
         umma_commit(s_full);
-        // P of tile i is in shared memory and any rescale of O by the softmax
-        // threads is complete: O += P V
+        // P of tile i is in shared memory, S has been read (S(i+1) needs no wait of
+        // its own) and any rescale of O by the softmax threads is complete: O += P V
         if (!warp_wait_bounded(p_full, i & 1, abort_flag, args.status)) break;
         tc_fence_after();
 #pragma unroll
@@ -387,7 +384,6 @@ __global__ void __launch_bounds__(192, AttnTcCfg<HD, TKV>::MIN_BLOCKS)
       m_ref = m_new;
       tc_fence_before();
       fence_proxy_async_smem();
-      warp_arrive(s_free);
       warp_arrive(p_full);
     }
     const size_t bk = static_cast<size_t>(b) * args.n_kv_heads + hk;
