@@ -6,13 +6,15 @@
 //   warp 0      one thread issues TMA loads of A / B tiles into a 4-stage
 //               shared-memory ring (128-byte swizzle);
 //   warp 1      allocates 512 TMEM columns (two 128 x 256 fp32 accumulators)
-//               and one thread issues tcgen05.mma (M=128, N=256, K=16);
+//               and issues tcgen05.mma (M=128, N=256, K=16) converged, one
+//               elected lane;
 //   warps 2..9  epilogue: tcgen05.ld the accumulator rows (one TMEM lane per
 //               thread; two warps per lane quadrant, each taking half of the
 //               256 columns) and run the fused epilogue of epilogue.cuh, while
 //               the MMA warp fills the other accumulator.
 // GEMMs of more than 128 rows run the CTA-pair variant (gemm_tc2_kernel:
-// 256 x 256 tiles, tcgen05.mma.cta_group::2, six stages), with split-K for
+// 256 x 256 tiles, 192 or 128 wide where those leave SMs idle,
+// tcgen05.mma.cta_group::2, six to eight stages), with split-K for
 // the weight-streaming residual / fp32-store GEMMs whose tiles cannot fill
 // the SMs; other GEMMs that need split-K run this kernel.
 // Every mbarrier wait is bounded (mbar_wait_bounded): a role that gives up
