@@ -456,9 +456,10 @@ __global__ void __launch_bounds__(192, AttnTcCfg<HD, TKV>::MIN_BLOCKS)
 // hd 128, launches within one CTA per SM: four stages of 32 KB and P fill the
 // shared memory.  hd 128, larger launches of long rows: two stages, so that two
 // CTAs share an SM, and P(i) in the columns of S(i), which its thread has read
-// (8 prompts x 16 heads x 512 causal rows: 28 us; 40 with attn_tc_kernel's
+// (8 prompts x 16 heads x 512 causal rows: 27 us; 40 with attn_tc_kernel's
 // 128-key tiles, one CTA per SM, 33 with four stages; 2 x 32 heads x 2048
-// rows: 147 -> 122).  The error against 64 bits is attn_tc_kernel's.
+// rows: 147 -> 120).  Largest error against 64 bits as with attn_tc_kernel
+// (2^-7.3 of sum p |v|), 2-norm within 2 % of it.
 // The MMA warp issues S(i), then O += P(i-1) V(i-1): while the softmax warps
 // exponentiate tile i, the tensor pipe already computes S(i+1).  Ordering facts
 // (tcgen05 operations of one thread complete in issue order): P V(i-2) is
@@ -660,23 +661,12 @@ __global__ void __launch_bounds__(192, AttnDbCfg<HD_, NST_>::MIN_BLOCKS)
       const int lim = kv_hi - i * TKV;                                // visible keys of this tile
       const bool masked = __any_sync(0xffffffffu, lim < TKV);
       uint32_t ra[32], rb[32];
-      float mxa[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-      if (C::P_OVER_S && i == 0 && n_tiles > 1) {
-        // the reference max comes from 128 keys, as with attn_tc_kernel's tiles: more rows hold their maximum as an exact
-        // P = 1 (from 64 keys, the 2-norm of the error grows by up to 2 %)
-        if (!warp_wait_bounded(&s_full[1], 0, abort_flag, args.status)) { ok = false; break; }
-        tc_fence_after();
-        tmem_ld32_nowait(t_s + TKV, ra);
-        tmem_ld32_nowait(t_s + TKV + 32, rb);
-        tmem_wait_ld(ra);
-        tmem_bind(rb);
-        max64<true>(ra, rb, 0, lim - TKV, mxa);
-      }
       tmem_ld32_nowait(t_s, ra);
       tmem_ld32_nowait(t_s + 32, rb);
       tmem_wait_ld(ra);
       tmem_bind(rb);
       // pass 1: row max over the tile (both halves stay in registers for pass 2)
+      float mxa[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
       if (masked) max64<true>(ra, rb, 0, lim, mxa);
       else max64<false>(ra, rb, 0, 64, mxa);
       const float m_tile = fmax3(fmaxf(mxa[0], mxa[1]), mxa[2], mxa[3]) * args.scale_log2;
