@@ -448,48 +448,40 @@ __global__ void __launch_bounds__(192, AttnTcCfg<HD, TKV>::MIN_BLOCKS)
 
 // ------------------------------------------------------------ pipelined variant
 // The same computation without key splits or a window, with the tensor pipe
-// and the softmax overlapped: 64-key tiles, S double-buffered in TMEM (S0, S1,
-// then O) and P double-buffered.  hd 64: four K / V stages, two CTAs per SM, P
-// in the TMEM columns behind O, two keys per column: a P V MMA then reads only
-// V from shared memory (16 of 48 cycles of operand reads for 32 of MMA) and the
-// softmax needs no proxy fence (two layers of 16 x 1024 rows: 757 -> 748 us).
-// hd 128, launches within one CTA per SM: four stages of 32 KB and P fill the
-// shared memory.  hd 128, larger launches of long rows: two stages, so that two
-// CTAs share an SM, and P(i) in the columns of S(i), which its thread has read
-// (8 prompts x 16 heads x 512 causal rows: 27 us; 40 with attn_tc_kernel's
-// 128-key tiles, one CTA per SM, 33 with four stages; 2 x 32 heads x 2048
-// rows: 147 -> 120).  Largest error against 64 bits as with attn_tc_kernel
-// (2^-7.3 of sum p |v|), 2-norm within 2 % of it.
-// The MMA warp issues S(i), then O += P(i-1) V(i-1): while the softmax warps
-// exponentiate tile i, the tensor pipe already computes S(i+1).  Ordering facts
-// (tcgen05 operations of one thread complete in issue order): P V(i-2) is
-// issued after p_full(i-2), when every softmax warp has read S(i-2), and before
-// S(i), so S(i) needs no wait for its buffer (an extra barrier for it cost 2.4
-// of 29.2 us over 16 x 2032 keys at hd 128); where P lies over S, S(i) waits on
-// o_full for P V(i-2), which reads those columns.  When S(i) is complete, the P
-// buffer of tile i and the O accumulator up to tile i-2 are settled; a rescale
-// of O at tile i waits for P V(i-1) on o_full.
-template <int HD_, int NST_>
+// and the softmax overlapped: 64-key tiles, S double-buffered in TMEM (S0,
+// S1, then O: 2 * 64 + hd of the 256 columns; two CTAs per SM for hd 64, one
+// for hd 128, whose four stages of 32 KB fill the shared memory) and P
+// double-buffered, four K / V stages.  P goes to shared memory for hd 128; for
+// hd 64 to the 64 TMEM columns left, two keys per column: a P V MMA then reads
+// only V from shared memory (16 of 48 cycles of operand reads for 32 of MMA)
+// and the softmax needs no proxy fence (two layers of 16 x 1024 rows:
+// 757 -> 748 us).  The MMA warp issues S(i), then O += P(i-1) V(i-1): while
+// the softmax warps exponentiate tile i, the tensor pipe already computes
+// S(i+1).  Ordering facts (tcgen05 operations of one thread complete in issue
+// order): P V(i-2) is issued after p_full(i-2), when every softmax warp has
+// read S(i-2), and before S(i), so S(i) needs no wait for its buffer (an extra
+// barrier for it cost 2.4 of 29.2 us over 16 x 2032 keys at hd 128); when S(i) is complete, the P buffer of tile i and
+// the O accumulator up to tile i-2 are settled; a rescale of O at tile i
+// waits for P V(i-1) on o_full.
+template <int HD_>
 struct AttnDbCfg {
-  static constexpr int HD = HD_, TKV = 64, STAGES = NST_;
-  static constexpr bool P_TMEM = HD == 64 || NST_ == 2, P_OVER_S = P_TMEM && HD != 64;
-  static constexpr int MIN_BLOCKS = P_TMEM ? 2 : 1;
+  static constexpr int HD = HD_, TKV = 64, STAGES = 4;
+  static constexpr int MIN_BLOCKS = HD == 64 ? 2 : 1;
   static constexpr int Q_BYTES = HD / 64 * 16384;     // HD/64 swizzle atoms of 128 rows x 64 dims
   static constexpr int K_BYTES = HD / 64 * TKV * 128; // HD/64 atoms of 64 keys x 64 dims
   static constexpr int V_BYTES = HD * 128;            // HD dims x 64 keys (V^T)
+  static constexpr bool P_TMEM = HD == 64;            // P0 at columns 192 .. 223, P1 at 224 .. 255
   static constexpr int P_BYTES = P_TMEM ? 0 : 16384;  // 128 rows x 64 keys
   static constexpr int SMEM = Q_BYTES + STAGES * (K_BYTES + V_BYTES) + 2 * P_BYTES + 256;
   static constexpr int TMEM_COLS = 256;               // S0 [0, 64), S1 [64, 128), O [128, 128 + HD)
-  static constexpr int P_COL = P_OVER_S ? 0 : 192, P_STEP = P_OVER_S ? TKV : 32;   // P in TMEM: columns of buffer 0, distance of 1
-  static_assert(NST_ == 2 || NST_ == 4, "barriers");
   static_assert(2 * TKV + HD <= TMEM_COLS, "TMEM columns");
 };
 
-template <int HD_, int NST_>
-__global__ void __launch_bounds__(192, AttnDbCfg<HD_, NST_>::MIN_BLOCKS)
+template <int HD_>
+__global__ void __launch_bounds__(192, AttnDbCfg<HD_>::MIN_BLOCKS)
     attn_db_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                    const AttnTcArgs args) {
-  using C = AttnDbCfg<HD_, NST_>;
+  using C = AttnDbCfg<HD_>;
   constexpr int HD = C::HD, TKV = C::TKV, NST = C::STAGES;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = smem_raw;
@@ -566,7 +558,7 @@ __global__ void __launch_bounds__(192, AttnDbCfg<HD_, NST_>::MIN_BLOCKS)
           tma_load_3d(sK + st * C::K_BYTES + s * (TKV * 128), &tmK, &kv_full[st], 64 * s, i * TKV, z);
         tma_load_3d(sV + st * C::V_BYTES, &tmV, &kv_full[st], i * TKV, 0, z);
         ++issued[st];
-        if (i + NST < n_tiles) {     // the stage ring holds tiles i .. i + NST - 1; L2 fetches tile i + NST meanwhile
+        if (i + NST < n_tiles) {     // the stage ring holds tiles i .. i+3; L2 fetches tile i+4 meanwhile
           for (int s = 0; s < HD / 64; ++s) tma_prefetch_3d(&tmK, 64 * s, (i + NST) * TKV, z);
           tma_prefetch_3d(&tmV, (i + NST) * TKV, 0, z);
         }
@@ -587,7 +579,6 @@ __global__ void __launch_bounds__(192, AttnDbCfg<HD_, NST_>::MIN_BLOCKS)
           // S(i) = Q K(i)^T into S buffer i & 1, which the softmax has read (p_full of tile i - 2)
           const int st = i % NST, sb = i & 1;
           if (!warp_wait_bounded(&kv_full[st], (i / NST) & 1, abort_flag, args.status)) break;
-          if (C::P_OVER_S && i >= 2 && !warp_wait_bounded(o_full, i & 1, abort_flag, args.status)) break;   // P V(i-2)
           tc_fence_after();
           const uint64_t k0 = sdesc_kmajor_sw128(smem_u32(sK + st * C::K_BYTES));
 #pragma unroll
@@ -605,7 +596,7 @@ __global__ void __launch_bounds__(192, AttnDbCfg<HD_, NST_>::MIN_BLOCKS)
           if constexpr (C::P_TMEM) {
 #pragma unroll
             for (int kk = 0; kk < TKV / 16; ++kk)
-              umma_bf16_ts(t_o, tmem + C::P_COL + pb * C::P_STEP + 8 * kk, v0 + 2 * kk, idesc_o, (j != 0) || (kk != 0));
+              umma_bf16_ts(t_o, tmem + 2 * TKV + HD + pb * (TKV / 2) + 8 * kk, v0 + 2 * kk, idesc_o, (j != 0) || (kk != 0));
           } else {
             const uint64_t p0 = sdesc_kmajor_sw128(smem_u32(sP + pb * C::P_BYTES));
 #pragma unroll
@@ -705,7 +696,7 @@ __global__ void __launch_bounds__(192, AttnDbCfg<HD_, NST_>::MIN_BLOCKS)
           exp32_regs<false>(ra, sc2, negm2, 64, ps2, pk);
           exp32_regs<false>(rb, sc2, negm2, 64, ps2, pk + 16);
         }
-        tmem_st32(tmem + lane_off + C::P_COL + sb * C::P_STEP, pk);
+        tmem_st32(t_o + lane_off + HD + sb * (TKV / 2), pk);
       } else {
         uint8_t* prow = sP + sb * C::P_BYTES + row * 128;
         if (masked) {
@@ -904,8 +895,8 @@ const char* launch_tc_win(const AttnCall& a, cudaStream_t s) {
   return nullptr;
 }
 
-// The pipelined kernels: where no key split is wanted (the CTAs of the launch
-// fill the SMs) and no window hides keys.  TADM_ATTN_DB=0 keeps
+// The pipelined hd-64 kernel: whenever no key split is wanted (the CTAs of
+// the launch fill the SMs) and no window hides keys.  TADM_ATTN_DB=0 keeps
 // attn_tc_kernel for every shape.
 bool attn_db_enabled() {
   static const bool on = [] {
@@ -915,9 +906,9 @@ bool attn_db_enabled() {
   return on;
 }
 
-template <int HD, int NST>
+template <int HD>
 const char* launch_db(const AttnCall& a, cudaStream_t s) {
-  using C = AttnDbCfg<HD, NST>;
+  using C = AttnDbCfg<HD>;
   if (!encoder()) return "cuTensorMapEncodeTiled is unavailable";
   const int kv_len = a.ctx + a.rows;
   CUtensorMap mk, mv;
@@ -928,7 +919,7 @@ const char* launch_db(const AttnCall& a, cudaStream_t s) {
     return "attention tensor map encode failed";
   static bool attr = false;
   if (!attr) {
-    if (cudaFuncSetAttribute(attn_db_kernel<HD, NST>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM) != cudaSuccess)
+    if (cudaFuncSetAttribute(attn_db_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM) != cudaSuccess)
       return "attention smem attribute failed";
     attr = true;
   }
@@ -937,7 +928,7 @@ const char* launch_db(const AttnCall& a, cudaStream_t s) {
   AttnTcArgs args{static_cast<const bf16*>(a.q), a.rows, a.ctx, kv_len, a.n_heads, a.n_kv_heads, a.causal, 0,
                   1.4426950408889634f / sqrtf(static_cast<float>(C::HD)), static_cast<bf16*>(a.o),
                   n_vtiles, 1, 0, nullptr, nullptr, a.status};
-  launch_pdl(attn_db_kernel<HD, NST>, dim3(n_vtiles, a.n_kv_heads, a.batch), 192, C::SMEM, s, mk, mv, args);
+  launch_pdl(attn_db_kernel<HD>, dim3(n_vtiles, a.n_kv_heads, a.batch), 192, C::SMEM, s, mk, mv, args);
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? nullptr : cudaGetErrorString(e);
 }
@@ -1437,25 +1428,20 @@ const char* attention(const AttnCall& a, cudaStream_t s) {
       cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev);
       const int ctas = ((a.n_heads / a.n_kv_heads) * a.rows + TQ - 1) / TQ * a.n_kv_heads * a.batch;
       const bool window_cuts = a.window > 0 && a.window < a.ctx + a.rows;
-      if (attn_db_enabled() && !window_cuts && ctas > n_sms) return launch_db<64, 4>(a, s);
+      if (attn_db_enabled() && !window_cuts && ctas > n_sms) return launch_db<64>(a, s);
       return launch_tc<64, 128>(a, s);
     }
     if (a.head_dim == 128) {
       if (!tc) return launch_bf16<128>(a, s) == cudaSuccess ? nullptr : "attention launch failed";
-      // the pipelined kernel at one CTA per SM when the launch fills 80-100 % of the SMs in one wave, at two CTAs per
-      // SM for larger launches of long rows; larger launches of short rows stay with attn_tc_kernel at two CTAs per SM
-      // (32 sequences x 32 rows over 1056 keys: 30.9 against 32.6 us), smaller ones split the keys
+      // one CTA per SM: the pipelined kernel when the launch fills 80-100 % of the SMs in one wave (larger
+      // launches run attn_tc_kernel two CTAs per SM, smaller ones split the keys)
       int dev = 0, n_sms = 0;
       cudaGetDevice(&dev);
       cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev);
-      const int n_virt = (a.n_heads / a.n_kv_heads) * a.rows;
-      const int ctas = (n_virt + TQ - 1) / TQ * a.n_kv_heads * a.batch;
+      const int ctas = ((a.n_heads / a.n_kv_heads) * a.rows + TQ - 1) / TQ * a.n_kv_heads * a.batch;
       const bool window_cuts = a.window > 0 && a.window < a.ctx + a.rows;
-      if (attn_db_enabled() && !window_cuts && 5 * ctas >= 4 * n_sms) {
-        if (ctas <= n_sms) return launch_db<128, 4>(a, s);
-        if (n_virt >= 2 * TQ) return launch_db<128, 2>(a, s);
-      }
-      return n_virt < 2 * TQ ? launch_tc<128, 64>(a, s) : launch_tc<128, 128>(a, s);
+      if (attn_db_enabled() && !window_cuts && 5 * ctas >= 4 * n_sms && ctas <= n_sms) return launch_db<128>(a, s);
+      return (a.n_heads / a.n_kv_heads) * a.rows < 2 * TQ ? launch_tc<128, 64>(a, s) : launch_tc<128, 128>(a, s);
     }
     return "bf16 attention supports head_dim 64 and 128";
   }
