@@ -649,7 +649,7 @@ __global__ void __launch_bounds__(256) post_norm_add_block_kernel(float* __restr
 }
 
 // s[row] = sqrt(mean(x^2) + eps) and out = x / s[row], one 256-thread block per
-// row (d % 4 == 0); the row comes back from L1 / L2 for the division.
+// row for few rows (d % 4 == 0); the row comes back from L1 / L2 for the division.
 template <class T>
 __global__ void __launch_bounds__(256) rms_divide_kernel(const float* __restrict__ x, int d, float eps,
                                                          float* __restrict__ s, void* __restrict__ out) {
@@ -667,6 +667,27 @@ __global__ void __launch_bounds__(256) rms_divide_kernel(const float* __restrict
   const float sc = sqrtf(tot / static_cast<float>(d) + eps);
   if (threadIdx.x == 0) s[blockIdx.x] = sc;
   for (int j = threadIdx.x * 4; j < d; j += 1024) {
+    const float4 v = *reinterpret_cast<const float4*>(x + base + j);
+    store_act<T>(out, base + j + 0, v.x / sc);
+    store_act<T>(out, base + j + 1, v.y / sc);
+    store_act<T>(out, base + j + 2, v.z / sc);
+    store_act<T>(out, base + j + 3, v.w / sc);
+  }
+}
+
+// rms_divide_kernel with a warp per row for many rows; lane l adds the squares of columns l, l + 32, ...
+template <class T>
+__global__ void __launch_bounds__(WPB * 32) rms_divide_warp_kernel(const float* __restrict__ x, int M, int d, float eps,
+                                                                   float* __restrict__ s, void* __restrict__ out) {
+  pdl_enter();
+  const int m = blockIdx.x * WPB + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (m >= M) return;
+  const size_t base = static_cast<size_t>(m) * d;
+  float ss = 0.0f;
+  for (int j = lane; j < d; j += 32) ss += x[base + j] * x[base + j];
+  const float sc = sqrtf(warp_sum(ss) / static_cast<float>(d) + eps);
+  if (lane == 0) s[m] = sc;
+  for (int j = lane * 4; j < d; j += 128) {
     const float4 v = *reinterpret_cast<const float4*>(x + base + j);
     store_act<T>(out, base + j + 0, v.x / sc);
     store_act<T>(out, base + j + 1, v.y / sc);
@@ -891,8 +912,13 @@ const char* rms_divide_rows(const float* x, int M, int d, float eps, float* s_ou
                             cudaStream_t st) {
   if (M <= 0) return nullptr;
   if (d % 4) return "rms_divide_rows needs d % 4 == 0";
-  if (act_bf16) launch_pdl(rms_divide_kernel<bf16>, M, 256, 0, st, x, d, eps, s_out, out);
-  else launch_pdl(rms_divide_kernel<float>, M, 256, 0, st, x, d, eps, s_out, out);
+  if (M < kFewRows) {
+    if (act_bf16) launch_pdl(rms_divide_kernel<bf16>, M, 256, 0, st, x, d, eps, s_out, out);
+    else launch_pdl(rms_divide_kernel<float>, M, 256, 0, st, x, d, eps, s_out, out);
+    return err();
+  }
+  if (act_bf16) launch_pdl(rms_divide_warp_kernel<bf16>, rows_grid(M), WPB * 32, 0, st, x, M, d, eps, s_out, out);
+  else launch_pdl(rms_divide_warp_kernel<float>, rows_grid(M), WPB * 32, 0, st, x, M, d, eps, s_out, out);
   return err();
 }
 
