@@ -274,20 +274,32 @@ __global__ void __launch_bounds__(256) splitk_qkv_kernel(EpiParams ep, const flo
   }
 }
 
-// Paired-attention gate on the slice sums: one warp per row (N <= 256 columns, N % 4 == 0).
+// Paired-attention gate on the slice sums: one warp per row (N <= 256 columns,
+// N % 4 == 0).  The lanes sum the slices and take the SiLU, whole lines at a
+// time; one lane adds the products in column order, as the epilogue of an
+// unsplit GEMM does, so that the gate's order of sums is the same on both
+// paths (256 dependent FMAs, under 1 us).
+constexpr int kGateCols = 256;
 __global__ void __launch_bounds__(256) splitk_gate_kernel(EpiParams ep, const float* __restrict__ part, size_t stride,
                                                           int ldp, int splits) {
+  __shared__ float2 term[8][kGateCols];             // (SiLU of the column, its weight)
   pdl_enter();
   const int m = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (m >= ep.M) return;
-  float s = 0.0f;
+  if (m >= ep.M) return;                            // uniform across the warp
+  float2* t = term[threadIdx.x >> 5];
   for (int n = 4 * lane; n < ep.N; n += 128) {
     const float4 a = slice_sum(part + static_cast<size_t>(m) * ldp + n, stride, splits);
-    s += silu_f(a.x) * ld_param(ep.vec, ep.bias_bf16, n) + silu_f(a.y) * ld_param(ep.vec, ep.bias_bf16, n + 1) +
-         silu_f(a.z) * ld_param(ep.vec, ep.bias_bf16, n + 2) + silu_f(a.w) * ld_param(ep.vec, ep.bias_bf16, n + 3);
+    t[n] = make_float2(silu_f(a.x), ld_param(ep.vec, ep.bias_bf16, n));
+    t[n + 1] = make_float2(silu_f(a.y), ld_param(ep.vec, ep.bias_bf16, n + 1));
+    t[n + 2] = make_float2(silu_f(a.z), ld_param(ep.vec, ep.bias_bf16, n + 2));
+    t[n + 3] = make_float2(silu_f(a.w), ld_param(ep.vec, ep.bias_bf16, n + 3));
   }
-  s = warp_sum(s);
-  if (lane == 0) static_cast<float*>(ep.out)[m] = sigmoid_f(s + ld_param(ep.bias, ep.bias_bf16, 0));
+  __syncwarp();
+  if (lane != 0) return;
+  float s = 0.0f;
+#pragma unroll 16
+  for (int n = 0; n < ep.N; ++n) s = fmaf(t[n].x, t[n].y, s);
+  static_cast<float*>(ep.out)[m] = sigmoid_f(s + ld_param(ep.bias, ep.bias_bf16, 0));
 }
 
 // Phase 2: the epilogue on slice 0.
@@ -303,7 +315,7 @@ cudaError_t launch(const EpiParams& ep, const float* part, size_t stride, int ld
       return cudaGetLastError();
     }
   } else if constexpr (EPI == EPI_PA_GATE) {
-    if (ep.N % 4 == 0) {
+    if (ep.N % 4 == 0 && ep.N <= kGateCols) {
       *launches = 1;
       launch_pdl(splitk_gate_kernel, (ep.M + 7) / 8, 256, 0, s, ep, part, stride, ldp, splits);
       return cudaGetLastError();

@@ -63,8 +63,10 @@ def digests(T, name):
     return out
 
 
-# s_C and s_H of 1024 and more rows: one warp adds a row's squares
-@pytest.mark.parametrize("name,what", [("paired_2688", "scales")])
+# s_C and s_H of 1024 and more rows (one warp adds a row's squares); the gate of
+# a split GEMM (its products added in column order; 2688 rows leave the mixer's
+# GEMMs unsplit)
+@pytest.mark.parametrize("name,what", [("paired_2688", "scales"), ("paired_2688", "fused")])
 def test_step_bits(T, name, what):
     with open(GOLDEN) as f:
         assert digests(T, name)[what] == json.load(f)[name][what]
