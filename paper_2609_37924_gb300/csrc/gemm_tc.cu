@@ -867,12 +867,10 @@ const char* gemm_tc(const GemmCall& g, cudaStream_t s) {
       return nullptr;
     }
   }
-  // the few-tile GEMMs of the paired-attention mixer (256 x 256 x 256: one or
-  // two CTAs, whose epilogue then walks the whole tile) split down to two
-  // k-blocks per slice: the reduction spreads the epilogue over the SMs
-  const int min_kb = tiles * 8 <= g_num_sms && (g.epi == EPI_ADD || g.epi == EPI_SILU || g.epi == EPI_PA_GATE) ? 2 : 4;
-  if (g.split_buf && !g.m_dev && !pairs_fill && tiles * 3 < g_num_sms * 2 && kblocks >= 2 * min_kb) {
-    int sp = std::min(std::min(g_num_sms / tiles, kblocks / min_kb), 16);
+  // at least four k-blocks a slice (with two for the paired-attention mixer's few-tile GEMMs the 27 B block step took
+  // 924 us and not 943, but its fused latents moved: their sums were cut in other places)
+  if (g.split_buf && !g.m_dev && !pairs_fill && tiles * 3 < g_num_sms * 2 && kblocks >= 8) {
+    int sp = std::min(std::min(g_num_sms / tiles, kblocks / 4), 16);
     const size_t per = static_cast<size_t>(g.M) * a.ldp * sizeof(float);
     while (sp > 1 && sp * per > g.split_bytes) --sp;
     if (sp > 1) {

@@ -24,6 +24,8 @@ BASE = dict(vocab=1024, d_model=512, n_heads=4, n_kv_heads=2, head_dim=128, ffn=
             fusion_rank=256, fusion_heads=4, dtype="bf16")
 STEPS = {  # name: (model, batch, rows)
     "paired_2688": (dict(fusion="paired_attn"), 21, 128),
+    "paired_64": (dict(fusion="paired_attn"), 2, 32),
+    "paired_256": (dict(fusion="paired_attn"), 8, 32),
 }
 
 
@@ -65,8 +67,9 @@ def digests(T, name):
 
 # s_C and s_H of 1024 and more rows (one warp adds a row's squares); the gate of
 # a split GEMM (its products added in column order; 2688 rows leave the mixer's
-# GEMMs unsplit)
-@pytest.mark.parametrize("name,what", [("paired_2688", "scales"), ("paired_2688", "fused")])
+# GEMMs unsplit); the K slices of the mixer's GEMMs of few rows
+@pytest.mark.parametrize("name,what", [("paired_2688", "scales"), ("paired_2688", "fused"), ("paired_64", "fused"),
+                                       ("paired_256", "fused")])
 def test_step_bits(T, name, what):
     with open(GOLDEN) as f:
         assert digests(T, name)[what] == json.load(f)[name][what]
