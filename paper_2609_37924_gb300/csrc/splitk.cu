@@ -195,6 +195,7 @@ __global__ void __launch_bounds__(256) splitk_qkv_kernel(EpiParams ep, const flo
                                                          int ldp, int splits) {
   constexpr int P = HD / 64, H2 = HD / 2, RB = 8;
   __shared__ bf16 sv[HD][RB + 2];
+  __shared__ __align__(16) float sr[RB][HD];       // a warp's row, for QK-norm
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int gh = blockIdx.y, m0 = blockIdx.x * RB;
   int region = 2, head = gh - ep.n_heads - ep.n_kv_heads;
@@ -233,10 +234,22 @@ __global__ void __launch_bounds__(256) splitk_qkv_kernel(EpiParams ep, const flo
       }
     }
     if (gain) {
-      float ss = 0.0f;
+      // squares in column order, as the epilogue of an unsplit GEMM adds them: the row crosses shared memory and every
+      // lane runs the same chain (hd dependent FMAs on broadcast reads)
+      float* row = sr[w];
 #pragma unroll
-      for (int t = 0; t < P; ++t) ss = fmaf(a[t], a[t], fmaf(c[t], c[t], ss));
-      const float inv = rsqrtf(warp_sum(ss) / static_cast<float>(HD) + ep.qk_eps);
+      for (int t = 0; t < P; ++t) {
+        row[lane * P + t] = a[t];
+        row[H2 + lane * P + t] = c[t];
+      }
+      __syncwarp();
+      float ss = 0.0f;
+#pragma unroll 8
+      for (int n = 0; n < HD; n += 4) {
+        const float4 x = *reinterpret_cast<const float4*>(row + n);
+        ss = fmaf(x.w, x.w, fmaf(x.z, x.z, fmaf(x.y, x.y, fmaf(x.x, x.x, ss))));
+      }
+      const float inv = rsqrtf(ss / static_cast<float>(HD) + ep.qk_eps);
 #pragma unroll
       for (int t = 0; t < P; ++t) {
         a[t] *= inv * ld_param(gain, ep.bias_bf16, lane * P + t);

@@ -26,6 +26,8 @@ STEPS = {  # name: (model, batch, rows)
     "paired_2688": (dict(fusion="paired_attn"), 21, 128),
     "paired_64": (dict(fusion="paired_attn"), 2, 32),
     "paired_256": (dict(fusion="paired_attn"), 8, 32),
+    "qk_norm_64": (dict(qk_norm=True), 2, 32),
+    "qk_norm_hd64_96": (dict(qk_norm=True, n_heads=8, n_kv_heads=4, head_dim=64), 3, 32),
 }
 
 
@@ -67,9 +69,10 @@ def digests(T, name):
 
 # s_C and s_H of 1024 and more rows (one warp adds a row's squares); the gate of
 # a split GEMM (its products added in column order; 2688 rows leave the mixer's
-# GEMMs unsplit); the K slices of the mixer's GEMMs of few rows
+# GEMMs unsplit); the K slices of the mixer's GEMMs of few rows; the squares of
+# QK-norm behind a split QKV projection (column by column)
 @pytest.mark.parametrize("name,what", [("paired_2688", "scales"), ("paired_2688", "fused"), ("paired_64", "fused"),
-                                       ("paired_256", "fused")])
+                                       ("paired_256", "fused"), ("qk_norm_64", "h"), ("qk_norm_hd64_96", "h")])
 def test_step_bits(T, name, what):
     with open(GOLDEN) as f:
         assert digests(T, name)[what] == json.load(f)[name][what]
