@@ -756,36 +756,34 @@ const char* gemm_tc(const GemmCall& g, cudaStream_t s) {
   a.ep.M = g.M;
   a.ep.N = g.N;
   a.ep.n_tiles = a.n_tiles_n * (g.epi == EPI_LMHEAD ? 2 : 1);   // one partial per column half
-  // bf16 outputs of the plain, GLU and fusion-gate epilogues go out through TMA stores
+  // Outputs go out through TMA stores (bf16: plain, GLU, SiLU and fusion-gate epilogues; fp32: plain epilogue, the
+  // head's logits and the residual's reduce-adds) where base and row stride allow a map and the last column ends on
+  // 16 bytes: TMA clips to 16 bytes, not to elements, and columns past N are the caller's.  Otherwise row stores.
   CUtensorMap tc{}, tc2{};
   a.staged = 0;
-  auto aligned = [](const void* p, int ld) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && ld % 8 == 0; };
+  auto tma_ok = [](const void* p, int ld, int n, int es) {
+    return p && (reinterpret_cast<uintptr_t>(p) & 15) == 0 && ld % (16 / es) == 0 && n % (16 / es) == 0;
+  };
   a.ep.resid_tma = 0;
   a.ep.f32_tma = 0;
   a.part_tma = 0;
   if (g.epi == EPI_RESID || g.epi == EPI_FUSION2 || g.epi == EPI_ADD || g.epi == EPI_PA_UP) {
     a.staged = 1;   // the boxes serve as transpose scratch, or as the source of TMA reduce-adds
-    if (g.epi == EPI_RESID && (reinterpret_cast<uintptr_t>(g.ep.resid) & 15) == 0 && g.ep.ldr % 4 == 0 &&
-        make_f32_map(&tc, g.ep.resid, g.M, g.N, g.ep.ldr))
+    if (g.epi == EPI_RESID && tma_ok(g.ep.resid, g.ep.ldr, g.N, 4) && make_f32_map(&tc, g.ep.resid, g.M, g.N, g.ep.ldr))
       a.ep.resid_tma = 1;
   } else if (g.ep.out_bf16 && (g.epi == EPI_STORE || g.epi == EPI_GLU || g.epi == EPI_SILU)) {
-    if (aligned(g.ep.out, g.ep.ldo) && make_out_map(&tc, g.ep.out, g.M, g.N, g.ep.ldo)) a.staged = 1;
+    if (tma_ok(g.ep.out, g.ep.ldo, g.N, 2) && make_out_map(&tc, g.ep.out, g.M, g.N, g.ep.ldo)) a.staged = 1;
   } else if (g.ep.out_bf16 && g.epi == EPI_FUSION1 && g.ep.d_split % 64 == 0) {
-    if (aligned(g.ep.out, g.ep.ldo) && aligned(g.ep.out2, g.ep.ldo2) &&
+    if (tma_ok(g.ep.out, g.ep.ldo, g.ep.d_split, 2) && tma_ok(g.ep.out2, g.ep.ldo2, g.N - g.ep.d_split, 2) &&
         make_out_map(&tc, g.ep.out, g.M, g.ep.d_split, g.ep.ldo) &&
         make_out_map(&tc2, g.ep.out2, g.M, g.N - g.ep.d_split, g.ep.ldo2))
       a.staged = 1;
   }
-  // fp32 outputs of the plain epilogue and the head's logits: TMA stores of
-  // 32 x 32 boxes, where the last column ends on 16 bytes (N % 4 == 0: TMA
-  // clips to 16 bytes, and columns past N are the caller's)
   const float* f32_out = g.epi == EPI_STORE && !g.ep.out_bf16 ? static_cast<const float*>(g.ep.out)
                          : g.epi == EPI_LMHEAD                ? g.ep.logits
                                                               : nullptr;
   const int f32_ld = g.epi == EPI_STORE ? g.ep.ldo : g.ep.ld_logits;
-  if (f32_out && (reinterpret_cast<uintptr_t>(f32_out) & 15) == 0 && f32_ld % 4 == 0 && g.N % 4 == 0 &&
-      make_f32_map(&tc, f32_out, g.M, g.N, f32_ld))
-    a.ep.f32_tma = 1;
+  if (tma_ok(f32_out, f32_ld, g.N, 4) && make_f32_map(&tc, f32_out, g.M, g.N, f32_ld)) a.ep.f32_tma = 1;
   const int tiles = ((g.M + BM - 1) / BM) * a.n_tiles_n;
   // split-K when the tiles cannot fill the SMs and K is long: fixed-order
   // reduction afterwards, so results do not depend on the split

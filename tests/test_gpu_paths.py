@@ -42,6 +42,23 @@ def test_gemm_fp32_store_edges(T, M, N, K, ldc):
     assert (got[:, N:] == 7.0).all() and (flat[M * ldc:] == 7.0).all().item()
 
 
+# bf16 outputs likewise (N % 8 == 0 and ldc % 8 == 0), on both tile kernels:
+# columns past N of a wider matrix are the caller's
+@pytest.mark.parametrize("M", [33, 257])
+@pytest.mark.parametrize("N,K,ldc", [(301, 72, 304), (300, 136, 304), (304, 64, 312), (36, 64, 40), (260, 64, 264), (1, 8, 8),
+                                     (301, 72, 301)])
+def test_gemm_bf16_store_edges(T, M, N, K, ldc):
+    A, a = bf16_tensor((M, K), 8)
+    B, b = bf16_tensor((N, K), 9)
+    flat = torch.full((M * ldc + 8,), 7.0, dtype=torch.bfloat16, device="cuda")
+    C = flat[:M * ldc].view(M, ldc)
+    T.tadm_gemm(A, B, C[:, :N], dtype=1)
+    got, ref = C.cpu().to(torch.float64).numpy(), a @ b.T
+    # fp32 accumulation of K exact bf16 products, then one rounding to 8 bits
+    assert (np.abs(got[:, :N] - ref) <= 2.0 ** -8 * np.abs(ref) + 1e-5 * np.abs(a).max() * np.abs(b).max() * np.sqrt(K)).all()
+    assert (got[:, N:] == 7.0).all() and (flat[M * ldc:] == 7.0).all().item()
+
+
 def _nucleus_ok(logits, mask, top_p, u, tok, tol=2e-5):
     """tok is the inverse-CDF draw of the nucleus, up to fp32 rounding of the cumulative mass at its edges."""
     q = np.exp(logits.astype(np.float64) - np.delete(logits, mask).max())
