@@ -548,12 +548,13 @@ __global__ void __launch_bounds__(NT) remdm_sample_smem_kernel(const float* __re
     for (int v = tid; v < vocab; v += NT) {
       const float q = v == mask_id ? 0.0f : expf(qs[v] - mx);
       qs[v] = q;
-      s3[0] += q;
+      s3[0] += q > 0.0f ? q : 0.0f;                // a NaN holds no mass (nor does it pass a threshold below)
     }
     block_sum3<NT>(s3, red, flip);                 // its barrier also publishes qs
     const float total = s3[0], target = top_p * total;
     // mass(lo) >= target > mass(hi), mass(t) = sum of q >= t
-    uint32_t lo = __float_as_uint(fmaxf(0.99f * (1.0f - top_p) * total / static_cast<float>(vocab), 0.0f)), hi = 0x3F800001u;
+    uint32_t lo = __float_as_uint(fmaxf(0.99f * (1.0f - top_p) * total / static_cast<float>(vocab), 0.0f));
+    uint32_t hi = target > 0.0f ? 0x3F800001u : lo;   // a row without mass has no bracket (the search needs mass(hi) < target)
     float mass_hi = 0.0f, mass_hi_all = 0.0f;      // mass(hi); mass above the collected tokens
     bool collected = false;                        // the tokens of the bracket are in c
     float c[kNucCand / NT];

@@ -97,6 +97,25 @@ def test_remdm_nucleus_draws(T, V, R, top_p):
             assert _nucleus_ok(logits[b * R + r], mask, top_p, u[b, r, 2], got[b, r]), (b, r, got[b, r])
 
 
+# a NaN logit holds no mass and is never drawn; a row without any mass (every
+# weight e^(l - max) is 0 or NaN) draws nothing and ends (token -1)
+@pytest.mark.parametrize("V", [1001, 30522])
+def test_remdm_rows_with_nan_and_inf(T, V):
+    B, R, mask, top_p, seed, step = 1, 48, V - 1, 0.5, 78, 2
+    rng = np.random.default_rng(V)
+    logits = (0.5 * rng.standard_normal((R, V))).astype(np.float32)
+    logits[:, 5::97] = np.nan
+    logits[3] = -np.inf
+    logits[4, 7] = np.inf
+    zt = torch.full((B, R), mask, dtype=torch.int32, device="cuda")
+    act = torch.empty(R, dtype=torch.int32, device="cuda")
+    T.tadm_remdm_update(zt, torch.from_numpy(logits).cuda(), 0, mask, 0.0, 1.0, top_p, seed, step, act)
+    got, u = zt.cpu().numpy()[0], wl.remdm_uniforms(seed, step, B, R)[0, :, 2]
+    assert got[3] == got[4] == -1
+    for r in set(range(R)) - {3, 4}:
+        assert _nucleus_ok(np.where(np.isnan(logits[r]), -np.inf, logits[r]), mask, top_p, u[r], got[r]), (r, got[r])
+
+
 def f32_tensor(shape, seed):
     x = wl.normal(seed, 98, int(np.prod(shape)), 0.0, 1.0, "f32").reshape(shape)
     return torch.from_numpy(x).cuda(), x.astype(np.float64)
