@@ -1390,16 +1390,15 @@ cudaError_t launch_bf16(const AttnCall& a, cudaStream_t s) {
 template <int HD>
 cudaError_t launch_f32(const AttnCall& a, cudaStream_t s) {
   constexpr int need = F32Cfg<HD>::FLOATS * 4, alone = 120 * 1024;
-  static int n_sms = 0;
-  if (n_sms == 0) {
-    const cudaError_t e = cudaFuncSetAttribute(attn_f32_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               std::max(need, alone));
-    if (e != cudaSuccess) return e;
-    int dev = 0, n = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    n_sms = n > 0 ? n : 1;
-  }
+  int dev = 0;
+  const int n_sms = current_sms(&dev);
+  static PerDevice ready;
+  cudaError_t e = cudaSuccess;
+  if (ready.get(dev, [&] {
+        e = cudaFuncSetAttribute(attn_f32_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, std::max(need, alone));
+        return e == cudaSuccess ? 1 : 0;
+      }) <= 0)
+    return e;
   dim3 grid((a.rows + FQ - 1) / FQ, a.n_heads, a.batch);
   // a launch of at most one block per SM asks for more than half of an SM's
   // shared memory: its blocks start while the predecessor's last ones run and

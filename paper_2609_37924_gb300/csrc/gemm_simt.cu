@@ -162,14 +162,16 @@ __global__ void __launch_bounds__(NT, TM == 16 ? 1 : 2) gemm_simt_kernel(const f
 }
 
 template <int EPI, int TM, bool VEC>
-cudaError_t launch_tile(const GemmCall& g, int tiles_n, int b_split, int n_rows_b, const EpiParams& ep, cudaStream_t s) {
+cudaError_t launch_tile(const GemmCall& g, int dev, int tiles_n, int b_split, int n_rows_b, const EpiParams& ep,
+                        cudaStream_t s) {
   constexpr int smem = SimtCfg<TM>::FLOATS * 4;
-  static bool attr = false;
-  if (!attr) {
-    const cudaError_t e = cudaFuncSetAttribute(gemm_simt_kernel<EPI, TM, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static PerDevice ready;
+  cudaError_t e = cudaSuccess;
+  if (ready.get(dev, [&] {
+        e = cudaFuncSetAttribute(gemm_simt_kernel<EPI, TM, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        return e == cudaSuccess ? 1 : 0;
+      }) <= 0)
+    return e;
   const unsigned grid = static_cast<unsigned>(tiles_n) * static_cast<unsigned>((g.M + TM - 1) / TM);
   launch_pdl(gemm_simt_kernel<EPI, TM, VEC>, grid, NT, smem, s, static_cast<const float*>(g.A),
              static_cast<const float*>(g.B), g.M, g.K, g.lda, g.ldb, tiles_n, n_rows_b, b_split, g.b_weights ? 1 : 0, ep);
@@ -178,21 +180,16 @@ cudaError_t launch_tile(const GemmCall& g, int tiles_n, int b_split, int n_rows_
 
 template <int EPI>
 cudaError_t launch(const GemmCall& g, int tiles_n, int b_split, int n_rows_b, const EpiParams& ep, cudaStream_t s) {
-  static int n_sms = 0;
-  if (n_sms == 0) {
-    int dev = 0, n = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    n_sms = n > 0 ? n : 1;
-  }
+  int dev = 0;
+  const int n_sms = current_sms(&dev);
   const bool vec = g.K % 4 == 0 && g.lda % 4 == 0 && g.ldb % 4 == 0 &&
                    ((reinterpret_cast<uintptr_t>(g.A) | reinterpret_cast<uintptr_t>(g.B)) & 15) == 0;
   // 16-row tiles until 32-row tiles alone put a block on every SM (512 x 256: 64 against 128 blocks)
   const bool tall = static_cast<int64_t>(tiles_n) * ((g.M + 31) / 32) >= n_sms;
   if (vec)
-    return tall ? launch_tile<EPI, 32, true>(g, tiles_n, b_split, n_rows_b, ep, s)
-                : launch_tile<EPI, 16, true>(g, tiles_n, b_split, n_rows_b, ep, s);
-  return launch_tile<EPI, 32, false>(g, tiles_n, b_split, n_rows_b, ep, s);
+    return tall ? launch_tile<EPI, 32, true>(g, dev, tiles_n, b_split, n_rows_b, ep, s)
+                : launch_tile<EPI, 16, true>(g, dev, tiles_n, b_split, n_rows_b, ep, s);
+  return launch_tile<EPI, 32, false>(g, dev, tiles_n, b_split, n_rows_b, ep, s);
 }
 }  // namespace
 

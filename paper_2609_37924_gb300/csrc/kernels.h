@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include "epilogue.cuh"
+#include "per_device.h"
 
 namespace tadm {
 
@@ -25,6 +26,18 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+// The current device (*dev) and its SM count, at least 1.
+inline int current_sms(int* dev) {
+  static PerDevice sms;
+  *dev = 0;
+  cudaGetDevice(dev);
+  const int d = *dev, n = sms.get(d, [d] {
+    int v = 0;
+    return cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, d) == cudaSuccess ? v : 0;
+  });
+  return n > 0 ? n : 1;
 }
 
 struct GemmCall {
