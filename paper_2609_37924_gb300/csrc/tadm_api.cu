@@ -11,6 +11,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/tadm.h"
@@ -317,17 +318,28 @@ void probe_end(tadm_handle* h, cudaStream_t s, int idx, int kind, double flops, 
   h->probe_bytes[idx] = bytes;
 }
 
+// B of a GEMM.  The kernels load a model weight ahead of their grid dependency: every GEMM here follows another kernel
+// of the same stream, whose own wait covered whatever wrote the weights.  What a call computes itself must not be named
+// a weight, so each caller says which of the two it passes; a bare pointer does not convert.
+struct Operand {
+  const void* p;
+  bool weight;
+};
+Operand weight(const void* p) { return {p, true}; }
+Operand computed(const void* p) { return {p, false}; }
+static_assert(!std::is_convertible<const void*, Operand>::value && !GemmCall{}.b_weights,
+              "B counts as a weight only where its caller says so");
+
 // k_b > 0: A = [hi | lo] holds 2 k_b columns (a split operand) and both halves multiply B's k_b columns;
 // the recorded work is that of the k_b-deep product the method computes.
-tadm_status gemm(tadm_handle* h, const void* A, int64_t a_rows, int lda, const void* B, int ldb, int M, int N, int K,
+tadm_status gemm(tadm_handle* h, const void* A, int64_t a_rows, int lda, const Operand& B, int ldb, int M, int N, int K,
                  int epi, const EpiParams& ep, cudaStream_t s, bool out_f32 = false, const int* m_dev = nullptr,
-                 int k_b = 0, bool b_weights = true) {
+                 int k_b = 0) {
   GemmCall g{};
   g.k_b = k_b;
-  // every call here follows another kernel of the same stream, whose own wait covered whatever wrote the weights
-  g.b_weights = b_weights;
+  g.b_weights = B.weight;
   g.A = A;
-  g.B = B;
+  g.B = B.p;
   g.M = M;
   g.N = N;
   g.K = K;
@@ -400,8 +412,8 @@ tadm_status layer_fwd(tadm_handle* h, int li, float* x, int B, int R, int ctx, i
   ep.q_gain = L.q_norm;
   ep.k_gain = L.k_norm;
   ep.qk_eps = c.norm_eps;
-  TRYS(gemm(h, norm, Mmax, split ? 2 * d : d, L.wqkv, d, M, nqkv, split ? 2 * d : d, EPI_QKV, ep, s, false, nullptr,
-            split ? d : 0));
+  TRYS(gemm(h, norm, Mmax, split ? 2 * d : d, weight(L.wqkv), d, M, nqkv, split ? 2 * d : d, EPI_QKV, ep, s, false,
+            nullptr, split ? d : 0));
   AttnCall a{ep.q, ep.k, ep.v, h->at(h->off.attn), B, c.n_heads, c.n_kv_heads, hd, R, ctx, h->kv_stride, causal,
              h->act_bf16(), h->status()};
   a.window = L.window;
@@ -423,13 +435,13 @@ tadm_status layer_fwd(tadm_handle* h, int li, float* x, int B, int R, int ctx, i
   ey.ldo = d;
   float* post = h->at<float>(h->off.post);
   if (c.sandwich_norm) {
-    TRYS(gemm(h, h->at(h->off.attn), Mmax, q, L.wo, q, M, d, q, EPI_STORE, ey, s, true));
+    TRYS(gemm(h, h->at(h->off.attn), Mmax, q, weight(L.wo), q, M, d, q, EPI_STORE, ey, s, true));
     // x += RMSNorm(o W_o^T) * post_attn; norm = RMSNorm(x) * ffn_norm
     pi = probe_begin(h, s);
     TRY(post_norm_add(x, post, M, d, L.post_attn, L.ffn_norm, c.dtype, c.norm_eps, norm, h->act_bf16(), s));
     probe_end(h, s, pi, kProbeNorm, 0.0);
   } else {
-    TRYS(gemm(h, h->at(h->off.attn), Mmax, q, L.wo, q, M, d, q, EPI_RESID, er, s));
+    TRYS(gemm(h, h->at(h->off.attn), Mmax, q, weight(L.wo), q, M, d, q, EPI_RESID, er, s));
     pi = probe_begin(h, s);
     TRY(rmsnorm_rows(x, M, d, L.ffn_norm, c.dtype, c.norm_eps, norm, d, h->act_bf16(), s));
     probe_end(h, s, pi, kProbeNorm, 0.0);
@@ -438,14 +450,14 @@ tadm_status layer_fwd(tadm_handle* h, int li, float* x, int B, int R, int ctx, i
   eg.out = h->at(h->off.glu);
   eg.ldo = c.ffn;
   eg.glu = c.glu;
-  TRYS(gemm(h, norm, Mmax, d, L.wgu, d, M, c.ffn, d, EPI_GLU, eg, s));
+  TRYS(gemm(h, norm, Mmax, d, weight(L.wgu), d, M, c.ffn, d, EPI_GLU, eg, s));
   if (c.sandwich_norm) {
-    TRYS(gemm(h, h->at(h->off.glu), Mmax, c.ffn, L.wdown, c.ffn, M, d, c.ffn, EPI_STORE, ey, s, true));
+    TRYS(gemm(h, h->at(h->off.glu), Mmax, c.ffn, weight(L.wdown), c.ffn, M, d, c.ffn, EPI_STORE, ey, s, true));
     pi = probe_begin(h, s);
     TRY(post_norm_add(x, post, M, d, L.post_ffn, nullptr, c.dtype, c.norm_eps, nullptr, h->act_bf16(), s));
     probe_end(h, s, pi, kProbeNorm, 0.0);
   } else {
-    TRYS(gemm(h, h->at(h->off.glu), Mmax, c.ffn, L.wdown, c.ffn, M, d, c.ffn, EPI_RESID, er, s));
+    TRYS(gemm(h, h->at(h->off.glu), Mmax, c.ffn, weight(L.wdown), c.ffn, M, d, c.ffn, EPI_RESID, er, s));
   }
   return TADM_OK;
 }
@@ -493,7 +505,7 @@ tadm_status mixer(tadm_handle* h, const float* Z, const float* U, int B, int R, 
   eq.n_kv_heads = fh;
   eq.head_dim = hd;
   eq.rope = 0;
-  TRYS(gemm(h, J, Mmax, 2 * r, h->fw[2], 2 * r, M, 3 * r, 2 * r, EPI_QKV, eq, s));
+  TRYS(gemm(h, J, Mmax, 2 * r, weight(h->fw[2]), 2 * r, M, 3 * r, 2 * r, EPI_QKV, eq, s));
   AttnCall a{eq.q, eq.k, eq.v, h->at(h->off.pa_mo), B, fh, fh, hd, R, 0, R, 0, h->act_bf16(), h->status()};
   TRY(attention(a, s));
   EpiParams e1{};
@@ -503,18 +515,18 @@ tadm_status mixer(tadm_handle* h, const float* Z, const float* U, int B, int R, 
   e1.ldo = r;
   e1.out2 = h->at(h->off.pa_rb);
   e1.ldo2 = r;
-  TRYS(gemm(h, h->at(h->off.pa_mo), Mmax, r, h->fw[3], r, M, r, r, EPI_ADD, e1, s));
+  TRYS(gemm(h, h->at(h->off.pa_mo), Mmax, r, weight(h->fw[3]), r, M, r, r, EPI_ADD, e1, s));
   // EPI_ADD writes fp32 to out; out_bf16 only affects out2 (act copy)
   EpiParams e2{};
   e2.out = h->at(h->off.pa_hid);
   e2.ldo = 2 * r;
-  TRYS(gemm(h, h->at(h->off.pa_rb), Mmax, r, h->fw[4], r, M, 2 * r, r, EPI_SILU, e2, s));
+  TRYS(gemm(h, h->at(h->off.pa_rb), Mmax, r, weight(h->fw[4]), r, M, 2 * r, r, EPI_SILU, e2, s));
   EpiParams e3{};
   e3.base = h->at<float>(h->off.pa_r);
   e3.ldb = r;
   e3.out = phi;
   e3.ldo = r;
-  TRYS(gemm(h, h->at(h->off.pa_hid), Mmax, 2 * r, h->fw[5], 2 * r, M, r, 2 * r, EPI_ADD, e3, s));
+  TRYS(gemm(h, h->at(h->off.pa_hid), Mmax, 2 * r, weight(h->fw[5]), 2 * r, M, r, 2 * r, EPI_ADD, e3, s));
   return TADM_OK;
 }
 
@@ -530,7 +542,7 @@ tadm_status project_scaled(tadm_handle* h, const float* X, float* sc, bool fresh
   EpiParams e{};
   e.out = Z;
   e.ldo = c.fusion_rank;
-  return gemm(h, norm, Mmax, c.d_model, W, c.d_model, M, c.fusion_rank, c.d_model, EPI_STORE, e, s, true);
+  return gemm(h, norm, Mmax, c.d_model, weight(W), c.d_model, M, c.fusion_rank, c.d_model, EPI_STORE, e, s, true);
 }
 
 // A: h = A(c) in place in the cache, where run_S left a copy of c (plus the
@@ -579,7 +591,7 @@ tadm_status run_fusion(tadm_handle* h, int B, int R, const void* cache, cudaStre
     e1.ldo = d;
     e1.out2 = h->at(h->off.f_hid);
     e1.ldo2 = 4 * d;
-    TRYS(gemm(h, u, Mmax, 2 * d, h->fw[4], 2 * d, M, 5 * d, 2 * d, EPI_FUSION1, e1, s));
+    TRYS(gemm(h, u, Mmax, 2 * d, weight(h->fw[4]), 2 * d, M, 5 * d, 2 * d, EPI_FUSION1, e1, s));
     EpiParams e2{};
     e2.base = cv.h;
     e2.ldb = d;
@@ -588,7 +600,7 @@ tadm_status run_fusion(tadm_handle* h, int B, int R, const void* cache, cudaStre
     e2.bias = h->fw[7];
     e2.out = h->at(h->off.f_pre);
     e2.ldo = d;
-    TRYS(gemm(h, h->at(h->off.f_hid), Mmax, 4 * d, h->fw[6], 4 * d, M, d, 4 * d, EPI_FUSION2, e2, s));
+    TRYS(gemm(h, h->at(h->off.f_hid), Mmax, 4 * d, weight(h->fw[6]), 4 * d, M, d, 4 * d, EPI_FUSION2, e2, s));
     pi = probe_begin(h, s);
     TRY(layernorm_rows(h->at<float>(h->off.f_pre), M, d, h->fw[8], h->fw[9], c.dtype, c.norm_eps, x, s));
     probe_end(h, s, pi, kProbeNorm, 0.0);
@@ -608,7 +620,7 @@ tadm_status run_fusion(tadm_handle* h, int B, int R, const void* cache, cudaStre
   eg.vec = h->fw[7];
   eg.bias = h->fw[8];
   eg.out = h->at(h->off.pa_g);
-  TRYS(gemm(h, F, Mmax, 4 * r, h->fw[6], 4 * r, M, r, 4 * r, EPI_PA_GATE, eg, s));
+  TRYS(gemm(h, F, Mmax, 4 * r, weight(h->fw[6]), 4 * r, M, r, 4 * r, EPI_PA_GATE, eg, s));
   EpiParams eu{};
   eu.base = cv.h;
   eu.ldb = d;
@@ -616,7 +628,7 @@ tadm_status run_fusion(tadm_handle* h, int B, int R, const void* cache, cudaStre
   eu.rowscale = cv.sH;
   eu.out = x;
   eu.ldo = d;
-  return gemm(h, Mb, Mmax, r, h->fw[9], r, M, d, r, EPI_PA_UP, eu, s);
+  return gemm(h, Mb, Mmax, r, weight(h->fw[9]), r, M, d, r, EPI_PA_UP, eu, s);
 }
 
 // D on x, then the output head and the per-row (conf, tok).  With
@@ -647,7 +659,7 @@ tadm_status run_D_head(tadm_handle* h, int B, int R, float* logits, cudaStream_t
   e.mask_id = c.vocab - 1;
   e.logits = logits;
   e.ld_logits = c.vocab;
-  TRYS(gemm(h, norm, Mmax, d, h->lm_head, d, Mh, c.vocab, d, EPI_LMHEAD, e, s));
+  TRYS(gemm(h, norm, Mmax, d, weight(h->lm_head), d, Mh, c.vocab, d, EPI_LMHEAD, e, s));
   TRY(combine_partials(h->at<float>(h->off.part), Mh, h->n_part_tiles, h->at<float>(h->off.conf),
                        h->at<int32_t>(h->off.tok), s, idx));
   return TADM_OK;
@@ -1340,7 +1352,8 @@ tadm_status tadm_generate_remdm(tadm_handle* h, const int32_t* prompt, int batch
     e.mask_id = mask;
     e.logits = logits_scratch;
     e.ld_logits = c.vocab;
-    TRYS(gemm(h, norm, Mmax, c.d_model, h->lm_head, c.d_model, bound, c.vocab, c.d_model, EPI_LMHEAD, e, s, false, cnt));
+    TRYS(gemm(h, norm, Mmax, c.d_model, weight(h->lm_head), c.d_model, bound, c.vocab, c.d_model, EPI_LMHEAD, e, s,
+              false, cnt));
     TRY(remdm_sample(logits_scratch, c.vocab, bound, idx, act, out, total, batch, R, c.vocab, mask, top_p, seed, n, s,
                      cnt));
     h->counters.shared_layers += c.n_shared;
@@ -1480,7 +1493,7 @@ tadm_status tadm_generate_entropy_bound(tadm_handle* h, const int32_t* prompt, i
     e.mask_id = mask;
     e.logits = logits;
     e.ld_logits = c.vocab;
-    TRYS(gemm(h, norm, Mmax, c.d_model, h->lm_head, c.d_model, n_rows, c.vocab, c.d_model, EPI_LMHEAD, e, s));
+    TRYS(gemm(h, norm, Mmax, c.d_model, weight(h->lm_head), c.d_model, n_rows, c.vocab, c.d_model, EPI_LMHEAD, e, s));
     const double tau = tau_min + (tau_max - tau_min) * n / steps;
     const int last = n == 1;
     // max and argmax from the head's partials; q = exp((l - max) / tau) and Z for s = (q E) / Z
@@ -1491,8 +1504,7 @@ tadm_status tadm_generate_entropy_bound(tadm_handle* h, const int32_t* prompt, i
         EpiParams es{};
         es.out = sig;
         es.ldo = c.d_model;
-        TRYS(gemm(h, p, n_rows, c.vocab, et, c.vocab, n_rows, c.d_model, c.vocab, EPI_STORE, es, s, true, nullptr, 0,
-                  false));                    // E^T is written by this call
+        TRYS(gemm(h, p, n_rows, c.vocab, computed(et), c.vocab, n_rows, c.d_model, c.vocab, EPI_STORE, es, s, true));
       }
       TRY(eb_accept(ent, batch, R, prompt_len, out, total, c.vocab, eta, seed, i, s));
     }
