@@ -27,6 +27,7 @@
 
 #include "epilogue.cuh"
 #include "kernels.h"
+#include "tile_rule.h"
 
 namespace tadm {
 
@@ -700,18 +701,18 @@ cudaError_t launch_epi(const CUtensorMap& ta, const CUtensorMap& tb, const CUten
   return cudaGetLastError();
 }
 
-// CTA-pair kernel: `pairs` = 256-row x 256-column tiles; the grid is capped at
-// the number of 2-CTA clusters that fit on the GPU at once (a persistent grid
-// larger than that would run its last clusters after the others).
-template <int EPI, int PBN = 256, bool SPLIT = false>
-cudaError_t launch_epi_pair(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc,
-                            const CUtensorMap& tc2, const TcArgs& a, int pairs, cudaStream_t s) {
+// 2-CTA clusters of a pair kernel that fit on the GPU at once (0: its shared-memory attribute failed, *err says why)
+template <int EPI, int PBN, bool SPLIT>
+int max_clusters(cudaError_t* err) {
   constexpr size_t smem = PairCfg<PBN>::SMEM;
-  static int max_clusters = 0;
-  if (max_clusters == 0) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_tc2_kernel<EPI, PBN, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
+  static int clusters = 0;
+  if (clusters == 0) {
+    *err = cudaFuncSetAttribute(gemm_tc2_kernel<EPI, PBN, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                static_cast<int>(smem));
+    if (*err != cudaSuccess) {
+      cudaGetLastError();
+      return 0;
+    }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(g_num_sms & ~1);
     cfg.blockDim = dim3(NUM_THREADS);
@@ -721,10 +722,23 @@ cudaError_t launch_epi_pair(const CUtensorMap& ta, const CUtensorMap& tb, const 
       cudaGetLastError();
       n = g_num_sms / 2;
     }
-    max_clusters = n;
+    clusters = n;
   }
-  const int clusters = std::min(pairs, max_clusters);
-  launch_pdl(gemm_tc2_kernel<EPI, PBN, SPLIT>, 2 * clusters, NUM_THREADS, smem, s, ta, tb, tc, tc2, a);
+  return clusters;
+}
+
+// CTA-pair kernel: `pairs` = 256-row x PBN-column tiles (times K slices); the
+// grid is capped at the number of clusters that fit on the GPU at once (a
+// persistent grid larger than that would run its last clusters after the
+// others).
+template <int EPI, int PBN = 256, bool SPLIT = false>
+cudaError_t launch_epi_pair(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc,
+                            const CUtensorMap& tc2, const TcArgs& a, int pairs, cudaStream_t s) {
+  cudaError_t e = cudaSuccess;
+  const int fit = max_clusters<EPI, PBN, SPLIT>(&e);
+  if (fit <= 0) return e;
+  launch_pdl(gemm_tc2_kernel<EPI, PBN, SPLIT>, 2 * std::min(pairs, fit), NUM_THREADS, PairCfg<PBN>::SMEM, s, ta, tb, tc,
+             tc2, a);
   return cudaGetLastError();
 }
 
@@ -900,15 +914,12 @@ const char* gemm_tc(const GemmCall& g, cudaStream_t s) {
     const_cast<GemmCall&>(g).launched = 1;
     return nullptr;
   }
-  // GLU tiles of 96 gate and 96 up columns where their rounds over the clusters
-  // take at most 0.85 of the 256-wide tiles' (a narrower tile re-reads the
-  // activations more often): the 256 x 2 x 21504 projection of a 27 B block
-  // step is 168 tiles on 76 clusters, whose third round is 16 tiles, or 224 in
-  // 2.95 rounds (the step of three layers 978 -> 945 us)
+  // GLU: tiles of 96 gate and 96 up columns where the last round of 128 + 128 is nearly empty
   if (pair_ok && a.splits == 1 && glu && !g.m_dev) {
-    const int cl = std::max(g_num_sms / 2, 1), n192 = (g.N + 95) / 96;
-    const int64_t r256 = (pair_units + cl - 1) / cl, r192 = (m_pairs * n192 + cl - 1) / cl;
-    if (r192 * 192 * 100 <= r256 * 256 * 85) {
+    cudaError_t e256 = cudaSuccess, e192 = cudaSuccess;
+    const int n192 = (g.N + 95) / 96;
+    if (glu_tiles_192(pair_units, max_clusters<EPI_GLU, 256, false>(&e256), static_cast<int64_t>(m_pairs) * n192,
+                      max_clusters<EPI_GLU, 192, false>(&e192))) {
       CUtensorMap tbn;
       if (!make_map(&tbn, g.B, b_rows, k_b, g.ldb, 96)) return "tensor map (B, 96 rows) encode failed";
       TcArgs a2 = a;
