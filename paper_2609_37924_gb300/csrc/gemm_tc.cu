@@ -804,12 +804,15 @@ const char* gemm_tc(const GemmCall& g, cudaStream_t s) {
   const int f32_ld = g.epi == EPI_STORE ? g.ep.ldo : g.ep.ld_logits;
   if (tma_ok(f32_out, f32_ld, g.N, 4) && make_f32_map(&tc, f32_out, g.M, g.N, f32_ld)) a.ep.f32_tma = 1;
   const int tiles = ((g.M + BM - 1) / BM) * a.n_tiles_n;
-  // split-K when the tiles cannot fill the SMs and K is long: fixed-order
-  // reduction afterwards, so results do not depend on the split
+  // split-K when the tiles cannot fill the SMs and K is long: the slices are
+  // added in a fixed order, so results repeat for a shape on a device.  Their
+  // number follows from tiles, SMs and scratch, and with it the last bits: a
+  // row's result may change with the number of rows.
   const int kblocks = (g.K + BK - 1) / BK;
   a.splits = 1;
   a.kb_per_split = kblocks;
   a.ldp = a.n_tiles_n * BN;
+  const bool may_split = g.split_buf && !g.m_dev && splitk_takes(g.epi, a.ep, a.ldp);
   // CTA-pair tiles that keep >= 40% of the SMs busy beat split-K: no fp32
   // partials, no reduction launches.  Residual, fusion-output and QKV GEMMs
   // whose 256-wide pair tiles would occupy at most half the SMs (the
@@ -829,7 +832,7 @@ const char* gemm_tc(const GemmCall& g, cudaStream_t s) {
   // receives 32 KB per k-block (256 x 128 pair tiles: 24 KB for half the MMA
   // work; 128 x 256 tiles: 48 KB for the same work).
   const bool wide_fill = 2 * m_pairs * a.n_tiles_n * 10 >= g_num_sms * 6;
-  if (pair_ok && elem_reduce && !wide_fill && g.split_buf && !g.m_dev && kblocks >= 8) {
+  if (pair_ok && elem_reduce && !wide_fill && may_split && kblocks >= 8) {
     const int pu = m_pairs * a.n_tiles_n;
     int sp = std::min(std::min((g_num_sms / 2) / pu, kblocks / 4), 16);
     const size_t per = static_cast<size_t>(g.M) * a.ldp * sizeof(float);
@@ -859,7 +862,7 @@ const char* gemm_tc(const GemmCall& g, cudaStream_t s) {
   // activation operand once per cluster) likewise: 256-wide pair tiles with
   // split-K; the QKV epilogue (QK-norm, RoPE, Q / K / V writes) runs in the
   // split-K reduction on the slice-ordered sum.
-  if (narrow && g.epi == EPI_QKV && g.split_buf && !g.m_dev && kblocks >= 16) {
+  if (narrow && g.epi == EPI_QKV && may_split && kblocks >= 16) {
     const int pu = m_pairs * a.n_tiles_n;
     int sp = std::min(std::min((g_num_sms / 2) / pu, kblocks / 8), 16);
     const size_t per = static_cast<size_t>(g.M) * a.ldp * sizeof(float);
@@ -886,7 +889,7 @@ const char* gemm_tc(const GemmCall& g, cudaStream_t s) {
   }
   // at least four k-blocks a slice (with two for the paired-attention mixer's few-tile GEMMs the 27 B block step took
   // 924 us and not 943, but its fused latents moved: their sums were cut in other places)
-  if (g.split_buf && !g.m_dev && !pairs_fill && tiles * 3 < g_num_sms * 2 && kblocks >= 8) {
+  if (may_split && !pairs_fill && tiles * 3 < g_num_sms * 2 && kblocks >= 8) {
     int sp = std::min(std::min(g_num_sms / tiles, kblocks / 4), 16);
     const size_t per = static_cast<size_t>(g.M) * a.ldp * sizeof(float);
     while (sp > 1 && sp * per > g.split_bytes) --sp;

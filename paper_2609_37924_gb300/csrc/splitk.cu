@@ -3,63 +3,44 @@
 // that sum, in one launch with coalesced reads: element-wise for the epilogues
 // whose outputs depend on one column (GLU: a gate and an up column), a warp
 // per head row for QKV (QK-norm, RoPE, cache write), a warp per row for the
-// paired-attention gate.  The output head, and outputs that are not 16-byte
-// aligned, take two launches: the sum into slice 0, then the epilogue, one
-// thread per (output row, column group) of a 256-column tile.
-// The two launches cost 15 us for the QKV projection of a 32-row block step,
-// 9 us for its GLU and 20 us for the gate of 256 rows (16 to 64 blocks, rows
-// read by one lane each).  With one launch each a batch-1 block step 542 -> 496 us, a 27 B block step
-// 1108 -> 1060 us.
+// paired-attention gate.  The output head, whose partials need whole 128-column
+// runs of a row, takes two launches: the sum into slice 0, then the epilogue,
+// one thread per (output row, half of a 256-column tile).  Outputs that are not
+// 16-byte aligned are not split (splitk_takes).
+// With two launches for every epilogue the reductions took 15 us for the QKV
+// projection of a 32-row block step, 9 us for its GLU and 20 us for the gate of
+// 256 rows (16 to 64 blocks, rows read by one lane each).  With one launch each
+// a batch-1 block step 542 -> 496 us, a 27 B block step 1108 -> 1060 us.
 #include "kernels.h"
 
 namespace tadm {
 namespace {
 
+// row of slice 0 at a tile's first column
 struct PartSrc {
   static constexpr bool kStaged = false;
-  const float* row;      // partial row of slice 0 at this tile's first column
-  size_t stride;         // between slices
-  int splits;
+  const float* row;
   __device__ __forceinline__ void load(int chunk, float (&v)[32]) {
+    const float4* p = reinterpret_cast<const float4*>(row + 32 * chunk);
 #pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = 0.0f;
-    for (int ks = 0; ks < splits; ++ks) {
-      const float4* p = reinterpret_cast<const float4*>(row + ks * stride + 32 * chunk);
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const float4 t = p[q];
-        v[4 * q] += t.x; v[4 * q + 1] += t.y; v[4 * q + 2] += t.z; v[4 * q + 3] += t.w;
-      }
+    for (int q = 0; q < 8; ++q) {
+      const float4 t = p[q];
+      v[4 * q] = t.x; v[4 * q + 1] = t.y; v[4 * q + 2] = t.z; v[4 * q + 3] = t.w;
     }
   }
 };
 
-// Column groups one thread may take without changing the epilogue's result:
-// the output head keeps the tensor-core path's two partials per tile, the
-// paired-attention gate needs whole rows, GLU pairs gate / up chunks, QKV
-// whole heads; the rest is independent per 32-column chunk.
-template <int EPI>
-__device__ __forceinline__ int reduce_groups(const EpiParams& ep) {
-  if constexpr (EPI == EPI_PA_GATE) return 1;
-  else if constexpr (EPI == EPI_LMHEAD) return 2;
-  else if constexpr (EPI == EPI_GLU) return 4;
-  else if constexpr (EPI == EPI_QKV) return 256 / ep.head_dim;
-  else return 8;
-}
-
-// block: 32 rows x 8 group slots; thread (row, slot) runs group `slot` if it exists
-template <int EPI>
-__global__ void __launch_bounds__(256) splitk_reduce_kernel(EpiParams ep, const float* __restrict__ part,
-                                                            size_t stride, int ldp, int splits) {
+// Output head, phase 2: the epilogue on slice 0.  Block: 32 rows x the two
+// column halves of a tile (the two partials that the tensor-core path writes).
+__global__ void __launch_bounds__(64) splitk_head_kernel(EpiParams ep, const float* __restrict__ part, int ldp) {
   pdl_enter();
-  const int m = blockIdx.x * 32 + (threadIdx.x & 31), slot = threadIdx.x >> 5, nb = blockIdx.y;
-  const int groups = reduce_groups<EPI>(ep);
-  if (m >= ep.M || slot >= groups) return;
-  PartSrc src{part + static_cast<size_t>(m) * ldp + nb * 256, stride, splits};
-  epilogue_row<EPI>(ep, m, nb, 256, src, slot, groups);
+  const int m = blockIdx.x * 32 + (threadIdx.x & 31), nb = blockIdx.y;
+  if (m >= ep.M) return;
+  PartSrc src{part + static_cast<size_t>(m) * ldp + nb * 256};
+  epilogue_row<EPI_LMHEAD>(ep, m, nb, 256, src, threadIdx.x >> 5, 2);
 }
 
-// Phase 1: slice 0 <- sum of all slices in slice order, one float4 per thread.
+// Output head, phase 1: slice 0 <- sum of all slices in slice order, one float4 per thread.
 __global__ void __launch_bounds__(256) splitk_sum_kernel(float* __restrict__ part, size_t stride, size_t n4,
                                                          int splits) {
   pdl_enter();
@@ -107,8 +88,7 @@ __device__ __forceinline__ float4 slice_sum(const float* p, size_t stride, int s
 
 // Element-wise epilogues in one launch: each thread sums four consecutive
 // columns of one row over the slices in slice order, then runs the epilogue on
-// them, with coalesced 16-byte accesses.  Same sums in the same order as the
-// two-phase path below, so the result does not depend on which one ran.
+// them, with coalesced 16-byte accesses.
 // The epilogue's other inputs (residual, base, gate, bias) are read ahead of the
 // grid dependency: their writers ran before the GEMM whose partials this kernel
 // waits for, and that GEMM writes nothing else.
@@ -315,58 +295,58 @@ __global__ void __launch_bounds__(256) splitk_gate_kernel(EpiParams ep, const fl
   static_cast<float*>(ep.out)[m] = sigmoid_f(s + ld_param(ep.bias, ep.bias_bf16, 0));
 }
 
-// Phase 2: the epilogue on slice 0.
 template <int EPI>
-cudaError_t launch(const EpiParams& ep, const float* part, size_t stride, int ldp, int splits, int n_tiles_n,
-                   cudaStream_t s, int* launches) {
-  if constexpr (EPI == EPI_QKV) {
-    if (ep.out_bf16 && (ep.head_dim == 64 || ep.head_dim == 128)) {
-      *launches = 1;
-      const dim3 grid((ep.M + 7) / 8, ep.n_heads + 2 * ep.n_kv_heads);
-      if (ep.head_dim == 64) launch_pdl(splitk_qkv_kernel<64>, grid, 256, 0, s, ep, part, stride, ldp, splits);
-      else launch_pdl(splitk_qkv_kernel<128>, grid, 256, 0, s, ep, part, stride, ldp, splits);
-      return cudaGetLastError();
-    }
-  } else if constexpr (EPI == EPI_PA_GATE) {
-    if (ep.N % 4 == 0 && ep.N <= kGateCols) {
-      *launches = 1;
-      launch_pdl(splitk_gate_kernel, (ep.M + 7) / 8, 256, 0, s, ep, part, stride, ldp, splits);
-      return cudaGetLastError();
-    }
-  } else if constexpr (EPI != EPI_LMHEAD) {
-    if (elem_ok(EPI, ep, ldp)) {
-      *launches = 1;
-      const size_t n = static_cast<size_t>(ep.M) * (ep.N / 4);
-      launch_pdl(splitk_elem_kernel<EPI>, static_cast<unsigned>((n + 255) / 256), 256, 0, s, ep, part, stride, ldp,
-                 splits);
-      return cudaGetLastError();
-    }
-  }
-  *launches = 2;
+cudaError_t launch_elem(const EpiParams& ep, const float* part, size_t stride, int ldp, int splits, cudaStream_t s) {
+  const size_t n = static_cast<size_t>(ep.M) * (ep.N / 4);
+  launch_pdl(splitk_elem_kernel<EPI>, static_cast<unsigned>((n + 255) / 256), 256, 0, s, ep, part, stride, ldp, splits);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_qkv(const EpiParams& ep, const float* part, size_t stride, int ldp, int splits, cudaStream_t s) {
+  const dim3 grid((ep.M + 7) / 8, ep.n_heads + 2 * ep.n_kv_heads);
+  if (ep.head_dim == 64) launch_pdl(splitk_qkv_kernel<64>, grid, 256, 0, s, ep, part, stride, ldp, splits);
+  else launch_pdl(splitk_qkv_kernel<128>, grid, 256, 0, s, ep, part, stride, ldp, splits);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_head(const EpiParams& ep, float* part, size_t stride, int ldp, int splits, int n_tiles_n,
+                        cudaStream_t s) {
   const size_t n4 = static_cast<size_t>(ep.M) * ldp / 4;
-  launch_pdl(splitk_sum_kernel, static_cast<unsigned>((n4 + 255) / 256), 256, 0, s, const_cast<float*>(part), stride, n4,
-                                                                            splits);
-  dim3 grid((ep.M + 31) / 32, n_tiles_n);
-  launch_pdl(splitk_reduce_kernel<EPI>, grid, 256, 0, s, ep, part, stride, ldp, 1);
+  launch_pdl(splitk_sum_kernel, static_cast<unsigned>((n4 + 255) / 256), 256, 0, s, part, stride, n4, splits);
+  launch_pdl(splitk_head_kernel, dim3((ep.M + 31) / 32, n_tiles_n), 64, 0, s, ep, part, ldp);
   return cudaGetLastError();
 }
 }  // namespace
 
-const char* splitk_reduce(int epi, const EpiParams& ep, const float* part, size_t stride, int ldp, int splits,
-                          int n_tiles_n, cudaStream_t s, int* launches) {
+bool splitk_takes(int epi, const EpiParams& ep, int ldp) {
+  switch (epi) {
+    case EPI_LMHEAD: return true;
+    case EPI_QKV: return ep.out_bf16 && (ep.head_dim == 64 || ep.head_dim == 128);
+    case EPI_PA_GATE: return ep.N % 4 == 0 && ep.N <= kGateCols;
+    default: return elem_ok(epi, ep, ldp);
+  }
+}
+
+const char* splitk_reduce(int epi, const EpiParams& ep, float* part, size_t stride, int ldp, int splits, int n_tiles_n,
+                          cudaStream_t s, int* launches) {
+  if (!splitk_takes(epi, ep, ldp)) return "split-K reduction of an output that it does not take";
+  *launches = epi == EPI_LMHEAD ? 2 : 1;
   cudaError_t e;
   switch (epi) {
-    case EPI_STORE: e = launch<EPI_STORE>(ep, part, stride, ldp, splits, n_tiles_n, s, launches); break;
-    case EPI_RESID: e = launch<EPI_RESID>(ep, part, stride, ldp, splits, n_tiles_n, s, launches); break;
-    case EPI_QKV: e = launch<EPI_QKV>(ep, part, stride, ldp, splits, n_tiles_n, s, launches); break;
-    case EPI_GLU: e = launch<EPI_GLU>(ep, part, stride, ldp, splits, n_tiles_n, s, launches); break;
-    case EPI_FUSION1: e = launch<EPI_FUSION1>(ep, part, stride, ldp, splits, n_tiles_n, s, launches); break;
-    case EPI_FUSION2: e = launch<EPI_FUSION2>(ep, part, stride, ldp, splits, n_tiles_n, s, launches); break;
-    case EPI_LMHEAD: e = launch<EPI_LMHEAD>(ep, part, stride, ldp, splits, n_tiles_n, s, launches); break;
-    case EPI_PA_UP: e = launch<EPI_PA_UP>(ep, part, stride, ldp, splits, n_tiles_n, s, launches); break;
-    case EPI_SILU: e = launch<EPI_SILU>(ep, part, stride, ldp, splits, n_tiles_n, s, launches); break;
-    case EPI_ADD: e = launch<EPI_ADD>(ep, part, stride, ldp, splits, n_tiles_n, s, launches); break;
-    case EPI_PA_GATE: e = launch<EPI_PA_GATE>(ep, part, stride, ldp, splits, n_tiles_n, s, launches); break;
+    case EPI_STORE: e = launch_elem<EPI_STORE>(ep, part, stride, ldp, splits, s); break;
+    case EPI_RESID: e = launch_elem<EPI_RESID>(ep, part, stride, ldp, splits, s); break;
+    case EPI_QKV: e = launch_qkv(ep, part, stride, ldp, splits, s); break;
+    case EPI_GLU: e = launch_elem<EPI_GLU>(ep, part, stride, ldp, splits, s); break;
+    case EPI_FUSION1: e = launch_elem<EPI_FUSION1>(ep, part, stride, ldp, splits, s); break;
+    case EPI_FUSION2: e = launch_elem<EPI_FUSION2>(ep, part, stride, ldp, splits, s); break;
+    case EPI_LMHEAD: e = launch_head(ep, part, stride, ldp, splits, n_tiles_n, s); break;
+    case EPI_PA_UP: e = launch_elem<EPI_PA_UP>(ep, part, stride, ldp, splits, s); break;
+    case EPI_SILU: e = launch_elem<EPI_SILU>(ep, part, stride, ldp, splits, s); break;
+    case EPI_ADD: e = launch_elem<EPI_ADD>(ep, part, stride, ldp, splits, s); break;
+    case EPI_PA_GATE:
+      launch_pdl(splitk_gate_kernel, (ep.M + 7) / 8, 256, 0, s, ep, part, stride, ldp, splits);
+      e = cudaGetLastError();
+      break;
     default: return "unknown epilogue";
   }
   return e == cudaSuccess ? nullptr : cudaGetErrorString(e);
