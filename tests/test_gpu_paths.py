@@ -97,6 +97,25 @@ def test_remdm_nucleus_draws(T, V, R, top_p):
             assert _nucleus_ok(logits[b * R + r], mask, top_p, u[b, r, 2], got[b, r]), (b, r, got[b, r])
 
 
+# more positions than one scan of the actions takes (32768), with drawing rows in
+# every part of it and several per block: each draws once, the others keep their token
+def test_remdm_many_positions(T):
+    B, R, V, mask, top_p, seed, step = 9, 7400, 30, 29, 0.9, 79, 3
+    rng = np.random.default_rng(9)
+    logits = rng.standard_normal((B * R, V)).astype(np.float32)
+    z = rng.integers(0, mask, (B, R)).astype(np.int32)
+    z[rng.random((B, R)) < 1 / 24] = mask
+    zt = torch.from_numpy(z).cuda()
+    act = torch.empty(B * R, dtype=torch.int32, device="cuda")
+    T.tadm_remdm_update(zt, torch.from_numpy(logits).cuda(), 0, mask, 0.0, 1.0, top_p, seed, step, act)
+    got, u = zt.cpu().numpy(), wl.remdm_uniforms(seed, step, B, R)
+    assert (got[z != mask] == z[z != mask]).all()
+    rows = np.argwhere(z == mask)
+    assert (rows[:, 0] * R + rows[:, 1] > 2 * 32768).any() and len(rows) > 2 * 304
+    for b, r in rows:
+        assert _nucleus_ok(logits[b * R + r], mask, top_p, u[b, r, 2], got[b, r]), (b, r, got[b, r])
+
+
 # a NaN logit holds no mass and is never drawn; a row without any mass (every
 # weight e^(l - max) is 0 or NaN) draws nothing and ends (token -1)
 @pytest.mark.parametrize("V", [1001, 30522])
@@ -122,7 +141,7 @@ def f32_tensor(shape, seed):
 
 
 # fp32 GEMM: 16- and 32-row tiles, 16-byte and 4-byte copies, K shorter than a
-# stage, K ending inside a group's 16 columns, one row and one column
+# stage, K ending inside a stage's 64 columns, one row and one column
 @pytest.mark.parametrize("M,N,K", [(1, 1, 1), (17, 65, 4), (15, 64, 68), (33, 130, 257), (31, 2000, 132), (700, 900, 260),
                                    (300, 1100, 30)])
 def test_gemm_f32_tiles(T, M, N, K):
@@ -165,7 +184,7 @@ def test_attention_f32_tiles(T, hd, Hq, Hkv, rows, ctx, causal, window, pad):
 
 # split-K reductions of every epilogue (QKV per head row, GLU, fusion gate /
 # hidden / output, paired-attention gate, add, up) at row counts around their
-# 16-row blocks, both head widths, QK-norm, and the paired-attention kernels
+# 8-row blocks, both head widths, QK-norm, and the paired-attention kernels
 @pytest.mark.parametrize("hd,fusion,qk_norm,batch,rows", [(128, "gated_mlp", False, 3, 11), (64, "gated_mlp", True, 1, 1),
                                                           (128, "paired_attn", True, 2, 24), (64, "paired_attn", False, 5, 32),
                                                           (128, "paired_attn", False, 1, 17)])
@@ -200,7 +219,7 @@ def test_few_row_steps_match_the_oracle(T, hd, fusion, qk_norm, batch, rows):
 def test_attention_pipelined_hd64(T, B, Hq, Hkv, rows, ctx, causal):
     hd, n = 64, ctx + rows
     stride = (n + 7) // 8 * 8
-    assert ((Hq // Hkv) * rows + 127) // 128 * Hkv * B > 152
+    assert ((Hq // Hkv) * rows + 127) // 128 * Hkv * B > torch.cuda.get_device_properties(0).multi_processor_count
     g = torch.Generator(device="cuda").manual_seed(rows)
     q = (2.0 * torch.randn((B, Hq, rows, hd), generator=g, device="cuda")).to(torch.bfloat16)
     k = torch.randn((B, Hkv, stride, hd), generator=g, device="cuda").to(torch.bfloat16)
