@@ -764,7 +764,6 @@ const char* gemm_tc(const GemmCall& g, cudaStream_t s) {
   a.b_split = glu ? g.N : 0;
   a.n_tiles_n = glu ? (g.N + BN / 2 - 1) / (BN / 2) : (g.N + BN - 1) / BN;
   a.kb_wrap = g.k_b > 0 ? g.k_b / BK : 0;
-  a.m_fast = b_rows * k_b > static_cast<int64_t>(g.M) * g.K;
   if (glu && g.N % (BN / 2)) return "GLU GEMM needs the FFN width to be a multiple of 128";
   if (g.epi == EPI_QKV && BN % g.ep.head_dim) return "head_dim must divide 256";
   if (g.epi == EPI_PA_GATE && g.N > BN) return "gate GEMM needs N <= 256";
@@ -803,6 +802,10 @@ const char* gemm_tc(const GemmCall& g, cudaStream_t s) {
                                                               : nullptr;
   const int f32_ld = g.epi == EPI_STORE ? g.ep.ldo : g.ep.ld_logits;
   if (tma_ok(f32_out, f32_ld, g.N, 4) && make_f32_map(&tc, f32_out, g.M, g.N, f32_ld)) a.ep.f32_tma = 1;
+  // tile order (see tile_coords); fp32 / bf16 outputs that leave by row stores stay N-fastest: neighbouring column tiles
+  // share lines there (300 x 30522 x 768, fp32 out: 57 us, M-fastest 72; 4096 rows 486 and 503)
+  const bool row_stores = (g.epi == EPI_STORE && !a.staged && !a.ep.f32_tma) || (f32_out && !a.ep.f32_tma);
+  a.m_fast = b_rows * k_b > static_cast<int64_t>(g.M) * g.K && !row_stores;
   const int tiles = ((g.M + BM - 1) / BM) * a.n_tiles_n;
   // split-K when the tiles cannot fill the SMs and K is long: the slices are
   // added in a fixed order, so results repeat for a shape on a device.  Their
