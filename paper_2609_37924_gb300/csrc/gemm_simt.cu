@@ -16,11 +16,11 @@
 // float4 reads fall into different banks.  16-row tiles run six stages, one
 // block per SM: a launch that starts while its predecessor's last blocks run
 // otherwise packs three blocks onto the first SMs that come free.  512 rows,
-// launched alone: W_down and W_o (N 256, K 1024 and 256) 17.8 us on average,
-// QKV (N 768, K 256) 13.5, GLU (N 2 x 1024, K 256) 23.6, fusion hidden (N 1280,
-// K 512) 40.8; with 64 x 64 tiles and 16 columns of K per synchronous step the
-// residual projections took 95 us, QKV 36, GLU 38.  Eight warps of half as many
-// columns: 10.9 -> 12.2 ms a generation.
+// events around each launch: W_down and W_o (N 256, K 1024 and 256) 15.5 us on
+// average, QKV (N 768, K 256) 16.2, GLU (N 2 x 1024, K 256) 26, fusion hidden
+// (N 1280, K 512) 42; with 64 x 64 tiles and 16 columns of K per synchronous
+// step the residual projections took 77 us, QKV 33, GLU 37, fusion hidden 71.
+// Eight warps of half as many columns: 10.9 -> 12.2 ms a generation.
 // EPI_GLU tiles hold 32 gate and 32 up columns; EPI_QKV needs head_dim <= 64.
 #include "kernels.h"
 
@@ -66,23 +66,35 @@ __global__ void __launch_bounds__(NT, TM == 16 ? 1 : 2) gemm_simt_kernel(const f
   constexpr int W = VEC ? 4 : 1, CPR = TK / W;      // copies per row of a stage
   float* sA = smem;                                 // [STAGES][TM][LDK]
   float* sB = smem + STAGES * TM * LDK;             // [STAGES][TN][LDK]
+  // A thread copies the same columns of every RPC-th row of a stage: its source is one pointer that steps by whole
+  // rows.  With a row, a column and a 64-bit product per copy the copies' own instructions paced the kernel: 4096 x 4095
+  // x 1023 (4-byte copies) 1589 -> 979 us, 4096 x 4096 x 512 514 -> 470, a fp32 generation of the tiny model 10.6 -> 10.0 ms.
+  constexpr int RPC = NT / CPR;                     // rows that the block covers at a time
+  const int r_in = tid / CPR, c_in = tid % CPR * W;
   auto load_a = [&](int ks) {
-    float* dst = sA + (ks % STAGES) * TM * LDK;
-    for (int i = tid; i < TM * CPR; i += NT) {
-      const int r = i / CPR, c = (i % CPR) * W, gk = ks * TK + c;
-      const bool ok = m0 + r < M && gk < K;
-      cp_async(dst + r * LDK + c, ok ? A + static_cast<size_t>(m0 + r) * lda + gk : A, 4 * W, ok, VEC);
+    float* dst = sA + (ks % STAGES) * TM * LDK + r_in * LDK + c_in;
+    const int gk = ks * TK + c_in;
+    const float* src = A + static_cast<size_t>(m0 + r_in) * lda + gk;
+    const int rows = gk < K ? M - m0 - r_in : 0;    // rows of this thread's column that exist
+#pragma unroll
+    for (int r = 0; r < TM; r += RPC) {
+      cp_async(dst + r * LDK, r < rows ? src : A, 4 * W, r < rows, VEC);
+      src += static_cast<size_t>(RPC) * lda;
     }
   };
   auto load_b = [&](int ks) {
-    float* dst = sB + (ks % STAGES) * TN * LDK;
-    for (int i = tid; i < TN * CPR; i += NT) {
-      const int r = i / CPR, c = (i % CPR) * W, gk = ks * TK + c;
-      int gn;
-      if (b_split > 0) gn = r < TN / 2 ? nb * (TN / 2) + r : b_split + nb * (TN / 2) + (r - TN / 2);
-      else gn = nb * TN + r;
+    float* dst = sB + (ks % STAGES) * TN * LDK + r_in * LDK + c_in;
+    const int gk = ks * TK + c_in;
+    // GLU: the tile's first half are gate rows, its second half their up rows
+    const int n0 = b_split > 0 ? nb * (TN / 2) : nb * TN, up = b_split > 0 ? b_split - TN / 2 : 0;
+    const float* src = B + static_cast<size_t>(n0 + r_in) * ldb + gk;
+#pragma unroll
+    for (int r = 0; r < TN; r += RPC) {
+      const int gn = n0 + r_in + r + (r >= TN / 2 ? up : 0);
       const bool ok = gn < n_rows_b && gk < K;
-      cp_async(dst + r * LDK + c, ok ? B + static_cast<size_t>(gn) * ldb + gk : B, 4 * W, ok, VEC);
+      const float* p = r >= TN / 2 ? src + static_cast<ptrdiff_t>(up) * ldb : src;
+      cp_async(dst + r * LDK, ok ? p : B, 4 * W, ok, VEC);
+      src += static_cast<size_t>(RPC) * ldb;
     }
   };
   if (b_early) {
