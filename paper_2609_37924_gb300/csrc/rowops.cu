@@ -131,13 +131,16 @@ __global__ void __launch_bounds__(256) embed_block_kernel(const int32_t* __restr
   }
 }
 
-// One row of d <= 8192 columns (d % 4 == 0) held by a 256-thread block: thread
-// t has the float4 at 4 t + 1024 i.  Few-row launches are paced by the latency
-// of one row; a block per row reads it once, with every load in flight.
-constexpr int kRowVec = 8;
-__device__ __forceinline__ void load_row_block(const float* __restrict__ x, int d, float4 (&v)[kRowVec]) {
+// One row of d <= 1024 NV columns (d % 4 == 0) held by a 256-thread block:
+// thread t has the float4 at 4 t + 1024 i, i < NV.  Few-row launches are paced
+// by the latency of one row; a block per row reads it once, with every load in
+// flight.  NV is the row's own width (1, 2, 4 or 8): held as eight vectors, a
+// narrow row's registers left two blocks per SM, and launches near 1024 rows
+// were slower than reading the row twice (1023 x 768: 3.6 us, 5.6 held so).
+template <int NV>
+__device__ __forceinline__ void load_row_block(const float* __restrict__ x, int d, float4 (&v)[NV]) {
 #pragma unroll
-  for (int i = 0; i < kRowVec; ++i) {
+  for (int i = 0; i < NV; ++i) {
     const int j = 4 * threadIdx.x + 1024 * i;
     v[i] = j < d ? *reinterpret_cast<const float4*>(x + j) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   }
@@ -173,18 +176,18 @@ __device__ __forceinline__ void store4<bf16>(void* out, size_t i, const float4& 
       make_uint2(*reinterpret_cast<uint32_t*>(&a), *reinterpret_cast<uint32_t*>(&b));
 }
 
-// rmsnorm_block_kernel for d <= 8192 with the row in registers and 8- / 16-byte
+// rmsnorm_block_kernel for d <= 1024 NV with the row in registers and 8- / 16-byte
 // accesses (16-byte aligned pointers, ldo % 4 == 0)
-template <class T>
+template <class T, int NV>
 __global__ void __launch_bounds__(256) rmsnorm_block_reg_kernel(const float* __restrict__ x, int d,
                                                                 const void* __restrict__ gain, int w_bf16, float eps,
                                                                 void* __restrict__ out, int ldo,
                                                                 const int32_t* __restrict__ rows_idx, int lo_off) {
   __shared__ float red[8];
   const int m = blockIdx.x;
-  float4 v[kRowVec], gw[kRowVec];
+  float4 v[NV], gw[NV];
 #pragma unroll
-  for (int i = 0; i < kRowVec; ++i) {               // weights: read while the previous kernel finishes
+  for (int i = 0; i < NV; ++i) {               // weights: read while the previous kernel finishes
     const int j = 4 * threadIdx.x + 1024 * i;
     if (j < d) gw[i] = ldw4(gain, w_bf16, j);
   }
@@ -192,10 +195,10 @@ __global__ void __launch_bounds__(256) rmsnorm_block_reg_kernel(const float* __r
   load_row_block(x + static_cast<size_t>(rows_idx ? rows_idx[m] : m) * d, d, v);
   float ss = 0.0f;
 #pragma unroll
-  for (int i = 0; i < kRowVec; ++i) ss += v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
+  for (int i = 0; i < NV; ++i) ss += v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
   const float inv = rsqrtf(block_sum256(ss, red) / static_cast<float>(d) + eps);
 #pragma unroll
-  for (int i = 0; i < kRowVec; ++i) {
+  for (int i = 0; i < NV; ++i) {
     const int j = 4 * threadIdx.x + 1024 * i;
     if (j >= d) break;
     const float4 g = gw[i];
@@ -818,11 +821,17 @@ const char* rmsnorm_rows(const float* x, int M, int d, const void* gain, int w_b
   if (!act_bf16) lo_off = 0;       // fp32 activations are not split
   if (lo_off > 0 && (lo_off < d || lo_off + d > ldo)) return "split operand: the remainder columns must follow the row";
   if (M < kFewRows) {
-    if (d % 4 == 0 && d <= 1024 * kRowVec && ldo % 4 == 0 && lo_off % 4 == 0 && all16({x, gain, out})) {
-      if (act_bf16)
-        launch_pdl(rmsnorm_block_reg_kernel<bf16>, M, 256, 0, s, x, d, gain, w_bf16, eps, out, ldo, rows_idx, lo_off);
-      else
-        launch_pdl(rmsnorm_block_reg_kernel<float>, M, 256, 0, s, x, d, gain, w_bf16, eps, out, ldo, rows_idx, lo_off);
+    if (d % 4 == 0 && d <= 8192 && ldo % 4 == 0 && lo_off % 4 == 0 && all16({x, gain, out})) {
+      auto go = [&](auto k) { launch_pdl(k, M, 256, 0, s, x, d, gain, w_bf16, eps, out, ldo, rows_idx, lo_off); };
+      auto wide = [&](auto t) {
+        using A = decltype(t);
+        if (d <= 1024) go(rmsnorm_block_reg_kernel<A, 1>);
+        else if (d <= 2048) go(rmsnorm_block_reg_kernel<A, 2>);
+        else if (d <= 4096) go(rmsnorm_block_reg_kernel<A, 4>);
+        else go(rmsnorm_block_reg_kernel<A, 8>);
+      };
+      if (act_bf16) wide(bf16{});
+      else wide(float{});
       return err();
     }
     if (act_bf16)
