@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(256) combine_block_kernel(const float* __restr
   pdl_enter();
   __shared__ float sv[32];
   __shared__ int si[32];
-  __shared__ float2 term[kCombineTiles];            // (sum, weight) of a tile; (0, 0) for one without a token
+  extern __shared__ __align__(16) float2 term[];    // [n_tiles] (sum, weight) of a tile; (0, 0) for one without a token
   const float* p = part + static_cast<size_t>(blockIdx.x) * n_tiles * 3;
   float mx = -INFINITY;
   int arg = -1;
@@ -1083,8 +1083,10 @@ const char* confidence_rows(const float* logits, int rows, int vocab, int ld, in
 const char* combine_partials(const float* part, int rows, int n_tiles, float* conf, int32_t* tok, cudaStream_t s,
                              const int32_t* rows_idx) {
   if (rows <= 0) return nullptr;
-  if (rows <= 1024 && n_tiles >= 64 && n_tiles <= kCombineTiles) {   // a row is a chain of n_tiles / 32 loads for one warp
-    launch_pdl(combine_block_kernel, rows, 256, 0, s, part, n_tiles, conf, tok, rows_idx);
+  // a row is a chain of n_tiles / 32 loads for one warp: a block per row up to as many rows as it has tiles (1000 tiles,
+  // 500 rows: 10.4 -> 6.7 us, 1000 rows 10.7 -> 7.7; 256 tiles, 128 rows 3.27 -> 3.16, 512 rows 3.18 and 3.38)
+  if (rows <= 1024 && rows <= n_tiles && n_tiles >= 64 && n_tiles <= kCombineTiles) {
+    launch_pdl(combine_block_kernel, rows, 256, n_tiles * sizeof(float2), s, part, n_tiles, conf, tok, rows_idx);
     return err();
   }
   launch_pdl(combine_kernel, (rows + 7) / 8, 256, 0, s, part, rows, n_tiles, conf, tok, rows_idx);
