@@ -4,6 +4,7 @@
 // LayerNorm of the gated-MLP fusion (App. C.2), the RMS scales and feature
 // concatenations of the paired-attention fusion (App. C.1), the RoPE table,
 // and canvas set-up.
+#include <algorithm>
 #include <cstdlib>
 #include <initializer_list>
 
@@ -93,9 +94,9 @@ __global__ void embed_kernel(const int32_t* __restrict__ z, int ldz, int rows, i
   }
 }
 
-// embed_kernel with a 256-thread block per row, for few rows (32 x 2048: 10 ->
-// 6 us with the copy behind it): eight bf16 (16 bytes) per thread and step.  d % 8 == 0, 16-byte
-// aligned bf16 table, outputs and add.
+// embed_kernel with a block per row (a thread per eight columns, up to 256), for
+// few rows (32 x 2048: 10 -> 6 us with the copy behind it): eight bf16 (16 bytes)
+// per thread and step.  d % 8 == 0, 16-byte aligned bf16 table, outputs and add.
 __global__ void __launch_bounds__(256) embed_block_kernel(const int32_t* __restrict__ z, int ldz, int rows,
                                                           const bf16* __restrict__ E, int d, int vocab,
                                                           float* __restrict__ out, float* __restrict__ out2,
@@ -110,7 +111,7 @@ __global__ void __launch_bounds__(256) embed_block_kernel(const int32_t* __restr
   const float sc = a && add_div ? 1.0f / add_div[ar] : 1.0f;
   const bf16* e = E + static_cast<size_t>(tok) * d;
   float* o = out + static_cast<size_t>(m) * d;
-  for (int j = threadIdx.x * 8; j < d; j += 2048) {
+  for (int j = threadIdx.x * 8; j < d; j += 8 * blockDim.x) {
     const uint4 raw = *reinterpret_cast<const uint4*>(e + j);
     const __nv_bfloat162* p2 = reinterpret_cast<const __nv_bfloat162*>(&raw);
     float4 v[2];
@@ -794,9 +795,13 @@ static bool all16(std::initializer_list<const void*> ps) {
   return true;
 }
 
-// below this many rows a block per row keeps more SMs busy than a warp per row (LayerNorm: the widths of the register
-// kernels from 1024 columns; narrower rows leave most of a block idle)
+// below this many rows a block per row keeps more SMs busy than a warp per row
 constexpr int kFewRows = 1024;
+// LayerNorm of the register kernels' widths from 1024 columns (narrower rows leave most of a block idle): a block per
+// row, whose result has the warp kernel's bits, up to these many rows (one: 2048 columns, 768 rows 6.4 us, by warps 7.5,
+// 1023 rows 8.1 and 6.9; 1024 columns 4.2 and 4.2, 5.2 and 4.3.  Pair: 2048 columns, 896 rows 10.8 and 11.8, 1023 rows
+// 12.0 and 11.9; 1024 columns 6.0 and 6.3, 6.7 and 6.5)
+constexpr int kFewRowsLn = 768, kFewRowsLnPair = 896;
 
 const char* embed_rows(const int32_t* z, int ldz, int batch, int rows, const void* E, int e_bf16, int d, int vocab,
                        float* out, float* out2, cudaStream_t s, const float* add, int add_first,
@@ -806,7 +811,7 @@ const char* embed_rows(const int32_t* z, int ldz, int batch, int rows, const voi
   if (d % 4) return "d_model must be a multiple of 4";
   if (add && (add_first < 0 || add_first > rows)) return "self-conditioning rows out of range";
   if (M < kFewRows && e_bf16 && d % 8 == 0 && all16({E, out, out2, add})) {
-    launch_pdl(embed_block_kernel, M, 256, 0, s, z, ldz, rows, static_cast<const bf16*>(E), d, vocab, out, out2, add,
+    launch_pdl(embed_block_kernel, M, std::min(256, (d / 8 + 31) / 32 * 32), 0, s, z, ldz, rows, static_cast<const bf16*>(E), d, vocab, out, out2, add,
                add_first, add_div);
     return err();
   }
@@ -877,7 +882,7 @@ static bool ln_pair_reg(const float* c, const float* h, int M, int d, const void
 const char* ln_pair_rows(const float* c, const float* h, int M, int d, const void* wc, const void* bc, const void* wh,
                          const void* bh, int w_bf16, float eps, void* u, int act_bf16, cudaStream_t s) {
   if (M <= 0) return nullptr;
-  if (M < kFewRows && (d == 1024 || d == 2048) && all16({c, h, wc, bc, wh, bh, u})) {
+  if (M <= kFewRowsLnPair && (d == 1024 || d == 2048) && all16({c, h, wc, bc, wh, bh, u})) {
     auto go = [&](auto k) { launch_pdl(k, 2 * M, 256, 0, s, c, h, wc, bc, wh, bh, w_bf16, eps, u); };
     if (d == 1024) act_bf16 ? go(ln_pair_block_kernel<bf16, 4>) : go(ln_pair_block_kernel<float, 4>);
     else act_bf16 ? go(ln_pair_block_kernel<bf16, 8>) : go(ln_pair_block_kernel<float, 8>);
@@ -898,7 +903,7 @@ const char* ln_pair_rows(const float* c, const float* h, int M, int d, const voi
 const char* layernorm_rows(const float* x, int M, int d, const void* w, const void* b, int w_bf16, float eps,
                            float* out, cudaStream_t s) {
   if (M <= 0) return nullptr;
-  if (M < kFewRows && (d == 1024 || d == 2048) && all16({x, w, b, out})) {
+  if (M <= kFewRowsLn && (d == 1024 || d == 2048) && all16({x, w, b, out})) {
     if (d == 1024) launch_pdl(layernorm_block_kernel<4>, M, 256, 0, s, x, w, b, w_bf16, eps, out);
     else launch_pdl(layernorm_block_kernel<8>, M, 256, 0, s, x, w, b, w_bf16, eps, out);
     return err();
