@@ -11,15 +11,20 @@
 // Layouts: q [B, Hq, rows, hd]; k [B, Hkv, kv_stride, hd];
 // v transposed [B, Hkv, hd, kv_stride]; o [B*rows, Hq*hd].
 //
-// bf16, rows >= 128 (attn_tc_kernel): tcgen05.  One CTA = 128 query rows of
-//   one (batch, head).  Warp 0 streams Q once and K / V^T tiles of 128 keys
-//   (2-stage ring) with TMA; warp 1 issues S = Q K^T into TMEM and, once the
-//   probabilities are in shared memory, O_tile = P V into TMEM; warps 2..5
-//   own one query row per thread: masked softmax on the S row, P as bf16
-//   into the 128-byte-swizzled operand layout; O accumulates in TMEM across
-//   key tiles, rescaled only when a row's running max grows by more than 2^8.
-// bf16, short rows (attn_bf16_kernel): mma.sync m16n8k16 flash attention;
-//   a CTA takes 64 rows of all query heads of one KV group (one K/V read).
+// bf16 (attn_tc_kernel): tcgen05, any row count.  One CTA = 128 virtual rows
+//   (the query heads of a KV group x canvas rows) of one (batch, KV head), and
+//   a range of the keys where CTAs would leave SMs idle.  The softmax warps
+//   stage Q; warp 0 streams K / V^T tiles of 128 or 64 keys (2-stage ring)
+//   with TMA; warp 1 issues S = Q K^T into TMEM and, once the probabilities
+//   are in shared memory, O += P V; warps 2..5 own one virtual row per thread:
+//   masked softmax on the S row, P as bf16 into the 128-byte-swizzled operand
+//   layout; O accumulates in TMEM across key tiles, rescaled only when a row's
+//   running max grows by more than 2^8.
+// bf16, pipelined (attn_db_kernel): the same with S double-buffered, for hd 64
+//   launches of more CTAs than SMs and hd 128 launches of one full wave.
+// bf16, K / V strides that TMA cannot address (attn_bf16_kernel): mma.sync
+//   m16n8k16 flash attention; a CTA takes 64 rows of all query heads of one KV
+//   group (one K/V read).
 // fp32: shared-memory tiles on the CUDA cores, 16 query rows per block.
 #include <cudaTypedefs.h>
 #include <algorithm>
@@ -588,7 +593,7 @@ __global__ void __launch_bounds__(192, AttnDbCfg<HD_>::MIN_BLOCKS)
           umma_commit(&s_full[sb]);
         }
         if (i >= 1) {
-          // O += P(j) V(j) for the previous tile, once its probabilities are in shared memory
+          // O += P(j) V(j) for the previous tile, once its probabilities are written (hd 64: TMEM, hd 128: shared memory)
           const int j = i - 1, pb = j & 1, st = j % NST;
           if (!warp_wait_bounded(&p_full[pb], (j >> 1) & 1, abort_flag, args.status)) break;
           tc_fence_after();

@@ -231,11 +231,11 @@ __device__ __forceinline__ void umma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, u
       "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-// umma_commit: arrive once on `bar` when every tcgen05 op issued so far by the
-// elected lane is done (warp-collective).
+
 // -------------------------------------------- programmatic dependent launch
 // Every kernel of the library calls this before its first access to memory
-// that another kernel writes: it waits until the previous kernel of the
+// that a kernel in flight may write (weights and results two launches back are
+// read ahead of it): it waits until the previous kernel of the
 // stream has completed and its writes are visible (a no-op when there is no
 // programmatic dependency), then lets the next kernel start launching; that
 // kernel's CTAs wait in this same call, so launch latency and whatever a
@@ -313,6 +313,8 @@ __device__ __forceinline__ void umma_commit_pair_mc(uint64_t* bar, uint16_t mask
       : "memory");
 }
 
+// umma_commit: arrive once on `bar` when every tcgen05 op issued so far by the
+// elected lane is done (warp-collective).
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
   asm volatile(
       "{\n\t.reg .pred e;\n\t"
