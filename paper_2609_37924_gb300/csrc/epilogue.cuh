@@ -287,8 +287,20 @@ __device__ __forceinline__ void epilogue_row(const EpiParams& p, int m, int n_bl
               xv[i] = ok ? p.resid[m_i * p.ldr + n] : 0.0f;
             } else {
               xv[i] = ok ? p.base[m_i * p.ldb + n] : 0.0f;
-              if constexpr (EPI == EPI_FUSION2) gv[i] = ok ? ld_param(p.gate, p.out_bf16, static_cast<int>(m_i * p.ldg + n)) : 0.0f;
               if constexpr (EPI == EPI_PA_UP) gv[i] = ok ? static_cast<const float*>(p.gate)[m_i] * p.rowscale[m_i] : 0.0f;
+            }
+          }
+          if constexpr (EPI == EPI_FUSION2) {       // one branch on the gate's type, not one per load
+            const size_t g0 = static_cast<size_t>(src.row0 + h0) * p.ldg + n;
+            if (p.out_bf16) {
+              const bf16* gp = static_cast<const bf16*>(p.gate) + g0;
+#pragma unroll
+              for (int i = 0; i < 16; ++i)
+                gv[i] = h0 + i < nrows && col_ok ? __bfloat162float(gp[static_cast<size_t>(i) * p.ldg]) : 0.0f;
+            } else {
+              const float* gp = static_cast<const float*>(p.gate) + g0;
+#pragma unroll
+              for (int i = 0; i < 16; ++i) gv[i] = h0 + i < nrows && col_ok ? gp[static_cast<size_t>(i) * p.ldg] : 0.0f;
             }
           }
 #pragma unroll
