@@ -264,11 +264,11 @@ def test_glu_192_wide_tiles(T, ffn, glu, rows):
     tm.close()
 
 
-# fp32 results of a row do not depend on how many rows the launch has: 16- and
-# 32-row GEMM tiles, block- and warp-per-row reduction of the head's tiles, one
+# fp32 GEMM, head and attention: a row's results do not depend on how many rows
+# the launch has: 16- and 32-row GEMM tiles, block- and warp-per-row reduction of the head's tiles, one
 # or several attention blocks (equal to the last bit: a sampler compares
 # confidences that may be that close)
-@pytest.mark.parametrize("rows", [1, 100, 1024])
+@pytest.mark.parametrize("rows", [1, 60, 100, 1024])
 def test_f32_rows_alone(T, rows):
     g = torch.Generator(device="cuda").manual_seed(3)
     d, vocab, M = 64, 4165, 1100
